@@ -126,7 +126,8 @@ const char* litevlm_select_last_error(litevlm_select_t handle);
 
 /* Number of kernels the last call on this handle enqueued (0 after an error
  * or a call with nothing to do); for counting launches (the score call runs
- * one kernel, two with the full key set). */
+ * one kernel, one more with the full key set, and one more when the re-read
+ * kernel splits the heads of a request and their partial rows are added up). */
 int32_t litevlm_select_last_launches(litevlm_select_t handle);
 
 /* Static description of a status code. */
@@ -359,8 +360,8 @@ litevlm_status_t litevlm_select_host_view(litevlm_select_t handle, const void* h
  * followed by litevlm_select_topk on them, with the arguments of those two
  * calls. When the score launch splits the heads of a request over several
  * CTAs, the top-k kernel adds the head-group partial rows itself (in the same
- * order as the score kernel would, so the scores are bit-identical) instead of
- * the score kernel's ticketed fold, which shortens the critical path of small
+ * order as the score call would, so the scores are bit-identical) instead of
+ * the score call's fold, which shortens the critical path of small
  * batches. It does so when batch <= 256, N_b <= 8192 and head groups x the
  * largest N_b <= 32768 (the partial values one top-k CTA reads); otherwise it
  * runs the two calls unchanged.
@@ -484,8 +485,11 @@ litevlm_status_t litevlm_select_set_debug_flags(litevlm_select_t handle, int32_t
  * Scratch: two static device arrays in this library, one per device:
  * 4 MiB of partial scores and 64 KiB of fold tickets.
  *   - Limit 1: total_visual / 128 + 2 * batch + 2 <= 16384.
- *   - Limit 2: when the chosen launch splits the query heads over G > 1 CTA
- *     groups, G * total_visual <= 1048576.
+ *   - Limit 2: when the launch splits the query heads over G > 1 CTA groups,
+ *     G * total_visual <= 1048576. The limit is applied to a launch shape fixed
+ *     by the batch's sizes, so it does not move when litevlm_select_score's
+ *     choice improves; where that choice needs more than the scratch holds, the
+ *     fixed shape is launched.
  *   - A call beyond either limit returns LITEVLM_ERR_WORKSPACE and enqueues
  *     nothing. Limit 1 is checked before any CUDA call.
  *   - A call that splits the heads clears the tickets it uses with

@@ -155,16 +155,6 @@ struct ScoreChoice {
     lvs::ScorePlan plan;
 };
 
-// Picks the score kernel and its launch shape. Cost unit: one tile-head of
-// the resident kernel with one TMEM head buffer (its MMAs, then its epilogue;
-// about 1.2 us at 64 text columns on GB300). A CTA also pays ~6 units (launch,
-// TMEM, pipeline fill) and, with one buffer, ~1 unit per head for the cluster
-// exchange. With two buffers the MMAs and the statistics exchange overlap the
-// epilogue, which then costs ~0.6 units per tile-head plus ~2.1 per head
-// (measured on GB300 at 3 tiles per CTA), and a head takes at least the time
-// its K tiles need at the CTA's share of HBM bandwidth. Waves of CTAs come from the measured
-// cluster occupancy of the kernel. The re-read kernel streams every K tile
-// twice (weight 1.6).
 // True when every request has the same, non-zero, visual and text token
 // counts (the resident kernel's flattened schedule needs it).
 bool uniform_batch(int batch, const int32_t* seq_offsets_h, const int32_t* text_offsets_h)
@@ -177,8 +167,29 @@ bool uniform_batch(int batch, const int32_t* seq_offsets_h, const int32_t* text_
     return true;
 }
 
+// Picks the score kernel and its launch shape by modelled time (microseconds,
+// fitted on GB300 to launches of 1 to 128 requests; KernelCosts below).
+//   Resident kernel: a CTA takes 8 to start and leave (2 more with a fold of
+// several head groups); a head with one TMEM buffer takes 0.8 a tile plus 0.8 for
+// the cluster exchange, with two buffers (MMAs and exchange under the epilogue)
+// 0.6 a tile plus 2.1, and at least the time its K tiles need at the CTA's share
+// of HBM bandwidth. Waves of CTAs come from the measured cluster occupancy.
+//   Re-read kernel: 6 to start (launch, set-up, first copies and contractions
+// from cold memory) and leave; per head two passes over the tiles, 1.2 a tile for
+// 256-byte rows with more than 64 text rows (the contractions' operands come out
+// of shared memory at its full rate beside the copies coming in), 1.0 up to 64,
+// 0.75 for 128-byte rows; 1.5 for the exchange over a cluster, 0.5 within one CTA;
+// the fold is a launch of its own, 2. It computes every contraction twice but has
+// no phases that wait for one another and no clusters to place; it is taken where
+// its model is more than 10% below: ragged batches (12 requests of 2 to 20 tiles,
+// T up to 127, 32 / 8 heads: 47 against 108 us), not large uniform ones (128 x 27
+// tiles, T = 64: 1000 against 734 us) nor short single requests, where both take
+// the time of a launch (12 tiles, 16 heads: 11.4 and 11.9 us).
+//   limit_rule: the older model by which the no-alloc entry point decides whether
+// a batch is within its static scratch (so that what it takes does not move with
+// the plans); in units of 1.17 us, the re-read kernel's times 1.6.
 ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* seq_offsets_h, int max_t, int row_bytes,
-                                bool fp8, bool uniform = false)
+                                bool fp8, bool uniform = false, bool limit_rule = false)
 {
     const litevlm_select_config_t& c = h->cfg;
     const int hq = c.num_q_heads;
@@ -202,20 +213,29 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     mix((uint64_t)row_bytes);
     mix((uint64_t)c.flags);
     mix((uint64_t)(uniform && h->allow_flat));
+    mix((uint64_t)limit_rule);
     for (int b = 0; b < batch; ++b) mix((uint64_t)td[b]);
     for (const auto& m : h->plan_memo)
         if (m.used && m.key == key) return ScoreChoice{m.resident, m.plan};
     const lvs::BatchTiles bt{td, batch};
 
     const int cmax = lvs::res_max_cluster(row_bytes, slot_cols);
-    const double unit_s = 1.17e-6, hbm_bytes_per_s = 6.8e12;
+    const double hbm_bytes_per_us = 6.8e6;
     const double tile_bytes = (double)lvs::kTileRows * row_bytes;
     double tc_cost = 0.0;
     int* tcap = h->tc_capacity[mrows == 64 ? 0 : 1];
     for (int cl = 1; cl <= lvs::kMaxCluster; ++cl)
         if (tcap[cl] < 0) tcap[cl] = lvs::tc_cluster_capacity(row_bytes, fp8, mrows, cl);
-    ScoreChoice best{false, lvs::plan_score(bt, hq, c.num_kv_heads, lvs::kTileRows * row_bytes, tcap, &tc_cost)};
-    double best_cost = 1.6 * tc_cost;
+    const double u = 1.17;
+    const lvs::KernelCosts res_costs = limit_rule ? lvs::KernelCosts{6.0 * u, u, u, 0.25 * u, 2.0 * u, false}
+                                                  : lvs::KernelCosts{8.0, 0.8, 0.8, 0.25, 2.0, false};
+    const double two_tile = limit_rule ? 0.6 * u : 0.6, two_head = limit_rule ? 2.1 * u : 2.1;
+    const lvs::KernelCosts tc_costs =
+        limit_rule ? lvs::KernelCosts{9.6 * u, 1.6 * u, 1.6 * u, 0.4 * u, 3.2 * u, false}
+                   : lvs::KernelCosts{6.0, row_bytes == 256 ? (max_t > 64 ? 1.2 : 1.0) : 0.75, 1.5, 0.5, 2.0, true};
+    ScoreChoice best{false, lvs::plan_score(bt, hq, c.num_kv_heads, row_bytes, tcap, tc_costs, limit_rule ? 2.0 : 1.0,
+                                            &tc_cost)};
+    double best_cost = limit_rule ? tc_cost : tc_cost / 0.9;
     const int max_tiles = batch > 0 ? td[0] : 0;
     const bool split_queries = (c.flags & LITEVLM_FLAG_SCORE_SPLIT_QUERIES) != 0;
     const int kflags = c.flags & ~(LITEVLM_FLAG_QUERY_LAST_TOKEN | LITEVLM_FLAG_SCORE_SPLIT_QUERIES);
@@ -257,13 +277,13 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
                         const int t = (tiles + cl - 1) / cl;
                         double per_head;
                         if (nb == 1) {
-                            per_head = (double)t + (cl > 1 ? 1.0 : 0.25);
+                            per_head = t * res_costs.tile + (cl > 1 ? res_costs.exchange : res_costs.exchange_one);
                         } else {
-                            const double stream = t * tile_bytes * active / hbm_bytes_per_s / unit_s;
-                            per_head = 0.6 * t + 2.1;
+                            const double stream = t * tile_bytes * active / hbm_bytes_per_us;
+                            per_head = two_tile * t + two_head;
                             if (stream > per_head) per_head = stream;
                         }
-                        return 6.0 + (g > 1 ? 2.0 : 0.0) + hpg * per_head;
+                        return res_costs.start + (g > 1 ? res_costs.fold : 0.0) + hpg * per_head;
                     };
                     const double cost = lvs::makespan(bt, g, cap / cl, item_cost);
                     if (cost < best_cost - 1e-9) {
@@ -305,10 +325,10 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
                     if (k1 - k0 + 1 > parts) parts = k1 - k0 + 1;
                 }
                 if (parts > hq) continue;
-                const double per_head = (double)tpc + (cl > 1 ? 1.0 : 0.25);
+                const double per_head = tpc * res_costs.tile + (cl > 1 ? res_costs.exchange : res_costs.exchange_one);
                 const long long per_cluster = (pairs + nclu - 1) / nclu;
                 const double boundaries = (double)per_cluster / hq_r + 1.0;
-                double cost = 6.0 + (double)per_cluster * per_head + 2.0 * boundaries;
+                double cost = res_costs.start + (double)per_cluster * per_head + res_costs.fold * boundaries;
                 if (kflags == LITEVLM_FLAG_SCORE_RESIDENT_FLAT) cost -= 1e200;  // forced: any flat plan beats the others
                 if (cost < best_cost - 1e-9) {
                     best_cost = cost;
@@ -520,7 +540,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
                             const int32_t* text_offsets_h, const void* k_vis, const int32_t* seq_offsets_d,
                             const int32_t* seq_offsets_h, float q_scale, float k_scale, float* scores,
                             const CtxKeys* ctx, litevlm_stream_t stream, bool allow_defer = false,
-                            int* deferred_groups = nullptr, size_t clear_tickets = 0)
+                            int* deferred_groups = nullptr, size_t clear_tickets = 0, bool limit_rule = false)
 {
     if (deferred_groups) *deferred_groups = 0;
     const litevlm_select_config_t& c = h->cfg;
@@ -560,7 +580,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
         s = debug_mirror(h, ctx->sys_offsets_d, ctx->sys_offsets_h, (int64_t)batch + 1, "sys_offsets", stream);
     if (s != LITEVLM_OK) return s;
     const ScoreChoice choice = choose_score_kernel(h, batch, seq_offsets_h, max_t, row_bytes, fp8,
-                                                   uniform_batch(batch, seq_offsets_h, text_offsets_h));
+                                                   uniform_batch(batch, seq_offsets_h, text_offsets_h), limit_rule);
     const lvs::ScorePlan& plan = choice.plan;
     if (plan.tiles_per_cta > lvs::kMaxTilesPerCta)
         return fail(h, LITEVLM_ERR_UNSUPPORTED, "request too long for one cluster");
@@ -642,7 +662,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     }
     // a caller whose tickets may not be at rest (the no-alloc entry point's
     // shared static scratch) has them cleared here, after every host-side check
-    if (clear_tickets > 0 && plan.groups > 1) {
+    if (clear_tickets > 0 && choice.resident && plan.groups > 1) {
         const cudaError_t ce = cudaMemsetAsync(h->counters, 0, sizeof(int32_t) * clear_tickets, (cudaStream_t)stream);
         if (ce != cudaSuccess) return cuda_fail(h, ce, "clearing the fold tickets");
     }
@@ -652,6 +672,24 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
             : lvs::launch_score(tm_q, tm_k, p, plan, batch, row_bytes, fp8, mrows, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "score launch");
     h->last_launches = ctx ? 2 : 1;
+    if (!choice.resident && plan.groups > 1 && !p.defer_fold) {
+        lvs::FoldArgs f{};
+        f.partials = h->partials;
+        f.out = scores;
+        f.seq_off = seq_offsets_d;
+        f.text_off = text_offsets_d;
+        f.total_vis = tot_n;
+        f.batch = batch;
+        f.groups = plan.groups;
+        f.hq = c.num_q_heads;
+        f.query_last = p.query_last;
+        f.nv = p.nv;
+        std::memcpy(f.so_v, p.so_v, sizeof(f.so_v));
+        std::memcpy(f.to_v, p.to_v, sizeof(f.to_v));
+        const cudaError_t fe = lvs::launch_fold(f, sh.max_n, (cudaStream_t)stream);
+        if (fe != cudaSuccess) return cuda_fail(h, fe, "fold launch");
+        ++h->last_launches;
+    }
     return LITEVLM_OK;
 }
 }  // namespace
@@ -820,7 +858,7 @@ litevlm_status_t litevlm_select_score_topk(litevlm_select_t h, int32_t batch, co
     const cudaError_t e = lvs::launch_topk(batch, scores, seq_offsets_d, keep_k_d, keep_ratio, kept_idx,
                                            out_offsets_d, max_n, sh, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "topk launch");
-    h->last_launches = 2;
+    ++h->last_launches;
     return LITEVLM_OK;
 }
 
@@ -1316,18 +1354,31 @@ extern "C" litevlm_status_t litevlm_select_score_noalloc(int32_t num_q_heads, in
     h.cfg.qk_dtype = qk_dtype;
     h.cfg.flags = 0;
 
-    // ---- the plan litevlm_select_score will take, checked against the partials' size
-    int32_t plan[4];
-    litevlm_status_t s = litevlm_select_score_plan(&h, batch, text_offsets_h, seq_offsets_h, plan);
-    if (s == LITEVLM_OK && plan[3] > 1 && (int64_t)plan[3] * tot_n > kNoAllocPartialFloats)
-        s = fail(&h, LITEVLM_ERR_WORKSPACE,
-                 "head groups x total_visual exceeds the static partial-score scratch (1048576 floats)");
+    // ---- the partials' size limit, by the limit rule's plan; the launch takes
+    // litevlm_select_score's plan where its partials fit too, else that one
+    ScoreShape sh;
+    litevlm_status_t s = check_score_shape(&h, batch, text_offsets_h, seq_offsets_h, &sh);
+    bool limit_plan = false;
+    if (s == LITEVLM_OK && sh.tot_n > 0) {
+        const int row_bytes = head_dim * (fam == 2 ? 1 : 2);
+        auto groups_of = [&](bool rule) {
+            const ScoreChoice ch = choose_score_kernel(&h, batch, seq_offsets_h, sh.max_t, row_bytes, fam == 2,
+                                                       uniform_batch(batch, seq_offsets_h, text_offsets_h), rule);
+            return (int64_t)ch.plan.groups;
+        };
+        const int64_t g = groups_of(true);
+        if (g > 1 && g * tot_n > kNoAllocPartialFloats)
+            s = fail(&h, LITEVLM_ERR_WORKSPACE,
+                     "head groups x total_visual exceeds the static partial-score scratch (1048576 floats)");
+        const int64_t gn = groups_of(false);
+        limit_plan = gn > 1 && gn * tot_n > kNoAllocPartialFloats;
+    }
     // the tickets start at zero (a launch that gave up may have left some
     // taken): score_impl clears them after all of its host-side checks, right
     // before the launch, so a rejected call enqueues nothing
     if (s == LITEVLM_OK)
         s = score_impl(&h, batch, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d, seq_offsets_h,
-                       q_scale, k_scale, scores, nullptr, stream, false, nullptr, (size_t)n_tickets);
+                       q_scale, k_scale, scores, nullptr, stream, false, nullptr, (size_t)n_tickets, limit_plan);
     {
         std::lock_guard<std::mutex> lock(g_noalloc_mutex);
         NoAllocDevice& d = g_noalloc[dev];

@@ -51,6 +51,31 @@ __device__ __forceinline__ bool wait_phase_cluster(uint32_t bar, uint32_t parity
     }
 }
 
+// The same waits for the re-read score kernel, whose warps wait often and for a
+// short time: kPolls polls of a few instructions between two looks at the abort
+// flag and the clock. The suspend-time hint above compiles to a loop around
+// NANOSLEEP, and a look at flag and clock on every poll to a dozen instructions;
+// both took issue slots from the warps of the SM sub-partition that had work
+// (fp8_ragged 151 -> 141 us). The resident kernel's long waits are better asleep
+// (sweep 734 us, 739 with polls).
+constexpr uint32_t kPolls = 64;
+
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool poll_phase(uint32_t bar, uint32_t parity, const Ctl& c)
+{
+    if (CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    for (;;) {
+        if (*c.abort) return false;
+        if (CLUSTER ? mbar_poll_cluster(bar, parity, kPolls) : mbar_poll(bar, parity, kPolls)) return true;
+        if (clock64() - t0 > c.budget) {
+            *c.abort = 1;
+            atomicOr(c.err, kErrTimeout);
+            return false;
+        }
+    }
+}
+
 // Online (max, sum 2^(x*c - max*c)) update of one row over NV columns.
 template <int NV>
 __device__ __forceinline__ void row_stats_update(const float* v, int valid, float cl, float& m, float& l)
@@ -105,6 +130,60 @@ __device__ __forceinline__ void row_stats_update(const float* v, int valid, floa
     m = m_new;
 }
 
+// Largest of the first NV values.
+template <int NV>
+__device__ __forceinline__ float row_max(const float* v)
+{
+    float m0 = v[0], m1 = v[1], m2 = v[2], m3 = v[3];
+#pragma unroll
+    for (int c = 4; c + 8 <= NV; c += 8) {
+        m0 = fmax3(m0, v[c], v[c + 1]);
+        m1 = fmax3(m1, v[c + 2], v[c + 3]);
+        m2 = fmax3(m2, v[c + 4], v[c + 5]);
+        m3 = fmax3(m3, v[c + 6], v[c + 7]);
+    }
+    m0 = fmax3(m0, v[NV - 4], v[NV - 3]);
+    m1 = fmax3(m1, v[NV - 2], v[NV - 1]);
+    return fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+}
+
+// s01, s23 += 2^(v * cl + nrc) over NV values (nrc: minus the scaled reference, twice)
+template <int NV>
+__device__ __forceinline__ void row_sum_exp(const float* v, float2 cl2, float2 nrc2, float2& s01, float2& s23)
+{
+#pragma unroll
+    for (int c = 0; c < NV; c += 4) {
+        const float2 x01 = ffma2(make_float2(v[c], v[c + 1]), cl2, nrc2);
+        const float2 x23 = ffma2(make_float2(v[c + 2], v[c + 3]), cl2, nrc2);
+        s01 = fadd2(s01, make_float2(ex2(x01.x), ex2(x01.y)));
+        s23 = fadd2(s23, make_float2(ex2(x23.x), ex2(x23.y)));
+    }
+}
+
+// s01, s23 += 2^(v * cl + nb[c]) over 16 columns; nb (shared memory, 16-byte
+// aligned) holds minus each column's merged statistic
+__device__ __forceinline__ void col_sum_exp16(const float* v, float2 cl2, const float* nb, float2& s01, float2& s23)
+{
+#pragma unroll
+    for (int c = 0; c < 16; c += 4) {
+        const float4 bb = *reinterpret_cast<const float4*>(nb + c);
+        const float2 x01 = ffma2(make_float2(v[c], v[c + 1]), cl2, make_float2(bb.x, bb.y));
+        const float2 x23 = ffma2(make_float2(v[c + 2], v[c + 3]), cl2, make_float2(bb.z, bb.w));
+        s01 = fadd2(s01, make_float2(ex2(x01.x), ex2(x01.y)));
+        s23 = fadd2(s23, make_float2(ex2(x23.x), ex2(x23.y)));
+    }
+}
+
+// (m, l) += (mo, lo): two sums of 2^((s - reference) * c) of one row under the larger reference
+__device__ __forceinline__ void merge_row(float& m, float& l, float mo, float lo, float cl)
+{
+    const float mm = fmaxf(m, mo);
+    if (mm != -INFINITY) {
+        l = (l > 0.f ? l * ex2((m - mm) * cl) : 0.f) + (lo > 0.f ? lo * ex2((mo - mm) * cl) : 0.f);
+        m = mm;
+    }
+}
+
 // log2(2^x + 2^y) for the merged statistic b and a normaliser term of other
 // keys in the same unit (x finite)
 __device__ __forceinline__ float log2_add(float x, float y)
@@ -142,10 +221,6 @@ __device__ __forceinline__ int fold_ticket_index(int b, int n0, int t) { return 
 // (default: the head groups) that own a tile adds the partials of that tile
 // in index order and writes the scores. `nthreads` threads (ids 0..nthreads-1, synchronised by
 // named barrier `bar_id`) take part; `flags` is shared memory for mt ints.
-// Each thread sums R rows at a time, with the loads of all R rows (up to 16
-// partials each) in flight together: a CTA that folds a long request's tiles
-// alone pays one L2 round trip per R rows instead of one per row.
-template <int R = 1>
 __device__ __forceinline__ void fold_tiles(const ScoreLaunch& p, int b, int n0, int N, int T, int tile_begin,
                                            int mt, int tid, int nthreads, uint32_t bar_id, volatile int* flags,
                                            int parts = 0)
@@ -163,61 +238,24 @@ __device__ __forceinline__ void fold_tiles(const ScoreLaunch& p, int b, int n0, 
     named_bar_sync(bar_id, nthreads);
     __threadfence();
     const float denom = (float)p.hq * (float)T;
-    if constexpr (R == 1) {
-        // (tile, row) pairs spread over all threads; up to 16 group partials in
-        // flight per row, added in group order
-        for (int x = tid; x < mt * kTileRows; x += nthreads) {
-            const int tl = x / kTileRows;
-            if (!flags[tl]) continue;
-            const int j = (tile_begin + tl) * kTileRows + (x - tl * kTileRows);
-            if (j >= N) continue;
-            const float* src = p.partials + n0 + j;
-            float sum = 0.f;
-            for (int g = 0; g < parts; g += 16) {
-                float v[16];
+    // (tile, row) pairs spread over all threads; up to 16 group partials in
+    // flight per row, added in group order
+    for (int x = tid; x < mt * kTileRows; x += nthreads) {
+        const int tl = x / kTileRows;
+        if (!flags[tl]) continue;
+        const int j = (tile_begin + tl) * kTileRows + (x - tl * kTileRows);
+        if (j >= N) continue;
+        const float* src = p.partials + n0 + j;
+        float sum = 0.f;
+        for (int g = 0; g < parts; g += 16) {
+            float v[16];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) v[q] = g + q < parts ? __ldcg(src + (int64_t)(g + q) * p.total_vis) : 0.f;
+            for (int q = 0; q < 16; ++q) v[q] = g + q < parts ? __ldcg(src + (int64_t)(g + q) * p.total_vis) : 0.f;
 #pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    if (g + q < parts) sum += v[q];
-            }
-            p.out[n0 + j] = sum / denom;
+            for (int q = 0; q < 16; ++q)
+                if (g + q < parts) sum += v[q];
         }
-    } else {
-        // thread tid takes rows x = tid + k * nthreads, R of them at a time, their
-        // group partials added in group order
-        for (int x0 = tid; x0 < mt * kTileRows; x0 += R * nthreads) {
-            int j[R];
-            bool live[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int x = x0 + r * nthreads;
-                const int tl = x / kTileRows;
-                j[r] = (tile_begin + tl) * kTileRows + (x - tl * kTileRows);
-                live[r] = x < mt * kTileRows && flags[tl] && j[r] < N;
-            }
-            float sum[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) sum[r] = 0.f;
-            for (int g = 0; g < parts; g += 16) {
-                float v[R][16];
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        v[r][q] = live[r] && g + q < parts
-                                      ? __ldcg(p.partials + n0 + j[r] + (int64_t)(g + q) * p.total_vis)
-                                      : 0.f;
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        if (g + q < parts) sum[r] += v[r][q];
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if (live[r]) p.out[n0 + j[r]] = sum[r] / denom;
-        }
+        p.out[n0 + j] = sum / denom;
     }
 }
 

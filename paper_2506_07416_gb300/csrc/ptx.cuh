@@ -150,6 +150,45 @@ __device__ __forceinline__ bool mbar_try_wait_cluster_sleep(uint32_t bar, uint32
     return ok != 0;
 }
 
+// up to `polls` tests in a row, in as few instructions as a loop takes
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_t polls)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\tmov.u32 n, %3;\n\t"
+        "POLL:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE;\n\t"
+        "sub.u32 n, n, 1;\n\t"
+        "setp.ne.u32 q, n, 0;\n\t"
+        "@q bra POLL;\n\t"
+        "DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(polls)
+        : "memory");
+    return ok != 0;
+}
+
+__device__ __forceinline__ bool mbar_poll_cluster(uint32_t bar, uint32_t parity, uint32_t polls)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\tmov.u32 n, %3;\n\t"
+        "POLL:\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE;\n\t"
+        "sub.u32 n, n, 1;\n\t"
+        "setp.ne.u32 q, n, 0;\n\t"
+        "@q bra POLL;\n\t"
+        "DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(polls)
+        : "memory");
+    return ok != 0;
+}
+
 // arrive on an mbarrier of another CTA of the cluster (address from mapa)
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar)
 {

@@ -74,6 +74,20 @@ struct ScorePlan {
     int qsplit = 1;           // resident kernel: 2 = each head's text rows as two pseudo-heads (64-row kernel)
 };
 
+// The head groups' partial rows added up (re-read kernel with several groups).
+struct FoldArgs {
+    const float* partials;    // [groups][total_vis]
+    float* out;               // scores [sum N]
+    const int32_t* seq_off;   // device [batch+1]
+    const int32_t* text_off;  // device [batch+1]
+    int64_t total_vis;
+    int32_t batch, groups, hq, query_last;
+    int32_t nv;               // > 0: the offsets by value, as in ScoreLaunch
+    int32_t so_v[kOffsetsByValue + 1];
+    int32_t to_v[kOffsetsByValue + 1];
+};
+cudaError_t launch_fold(const FoldArgs& a, int max_n, cudaStream_t stream);
+
 // Host helpers (score_tc.cu)
 // The batch as the planners see it: 128-token tiles per request, largest first.
 struct BatchTiles {
@@ -122,9 +136,18 @@ double makespan(const BatchTiles& bt, int g, int slots, const Cost& cost)
     return mx;
 }
 
+// Modelled times of the planners, in microseconds: a CTA's start and end, a tile
+// of a head, a head's statistics exchange over a cluster / within one CTA, and a
+// fold of several head groups (per CTA, or once when it is a launch of its own).
+struct KernelCosts {
+    double start, tile, exchange, exchange_one, fold;
+    bool fold_once;
+};
 // cap_by_cluster[c]: CTAs of the re-read kernel resident at once with clusters of c (<= 0: unusable)
-ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int tile_bytes, const int* cap_by_cluster,
-                     double* cost_out);
+// window_one: slices of K that must stay in L2 for the re-read of a CTA without a
+// cluster (2 in a cluster)
+ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int row_bytes, const int* cap_by_cluster,
+                     const KernelCosts& costs, double window_one, double* cost_out);
 int tc_cluster_capacity(int row_bytes, bool fp8, int mrows, int cluster);
 cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const ScoreLaunch& p,
                          const ScorePlan& plan, int batch, int row_bytes, bool fp8, int mrows, cudaStream_t stream);

@@ -11,10 +11,10 @@
 // head group); CTA r of the cluster owns a contiguous range of 128-token tiles
 // of the request. For every query head h of the group:
 //   pass 1: D1 = Q_h * K_tile^T on tcgen05 (M = 64 or 128 text rows, N = 128
-//           visual columns) into TMEM; one or two epilogue threads per text row
-//           keep an online (max, sum of 2^x) over the columns of all the CTA's
-//           tiles;
-//   exchange: each CTA publishes its per-row (m, l) in shared memory and
+//           visual columns) into TMEM; each epilogue thread keeps, for its text
+//           row, a reference logit and the sum of 2^((s - ref) * c) over its
+//           columns of the CTA's tiles;
+//   exchange: each CTA publishes its per-row (ref, sum) in shared memory and
 //           signals every CTA of the cluster by remote mbarrier arrivals; each
 //           CTA merges the C partials in rank order (deterministic) into
 //           b_hi = m_hi * c + log2(l_hi), c = scale * log2(e);
@@ -28,13 +28,30 @@
 // The K tiles stream through a TMA ring for both passes (the pass-2 re-read of
 // a CTA's few tiles is normally served by L2). Scores are summed over the heads
 // of the group in shared memory; with one head group they are final, with
-// several the CTAs write partial rows and the last CTA of the request to finish
-// (atomic ticket) adds them in a fixed order.
+// several the CTAs write partial rows and a small kernel launched behind this one
+// adds them in a fixed order over all SMs (the last CTA of a request to finish
+// used to: 28 rows of 1280 tokens through one SM made a tail of 6 to 8 us).
 //
-// Warp roles (448 threads): warp 0 = TMA producer, warp 1 = TMEM allocator and
-// MMA issuer, warps 2..13 = epilogue in three warpgroups (TMEM lane quadrant =
-// warp % 4); the contractions of both passes cycle through four 128-column
-// TMEM buffers and warpgroup g takes units u with u % 3 == g.
+// The reference of pass 1 is not the running maximum: any logit of the row
+// within 2^+-96 of the row's largest serves, since the sums are floating point
+// and the reference cancels in b. A thread takes the largest of the first 32
+// columns it sees, and moves it (to the larger maximum, rescaling its sum) only
+// when a sum passes 2^96, checked once per tile while the logits are still in
+// tensor memory. The loop is then one fused multiply-add (packed in
+// pairs), one 2^x and one add (packed) per logit, in both passes.
+//
+// Warp roles (352 threads): warp 0 = TMA producer, warps 1 and 2 = MMA issuers
+// (warp 1 also allocates TMEM), warps 3..10 = epilogue, two warpgroups (TMEM
+// lane quadrant = warp % 4). A contraction unit is one tile of one pass; the
+// units cycle through four 128-column TMEM buffers in issue order, and unit u
+// belongs to issuer u & 1 and to warpgroup u & 1: two independent pipelines,
+// each with one buffer being read and one being filled. Eight epilogue warps keep
+// the exponential unit as busy as sixteen do (4.8 cycles per 2^x and SM quarter
+// against 4.0 at best) and leave 168 registers a thread for straight-line blocks
+// of 64 columns: a branch per 32 columns (the reference check, the column count)
+// kept a warp from overlapping one block's sums with the next one's exponents and
+// cost 40% (P1 work per tile of two warps of an SM quarter: 1900 cycles, 1230 is
+// the exponential unit's share).
 // Every wait is bounded (clock budget); on expiry the kernel sets the error
 // word, drains its own copies and MMAs, frees TMEM and returns.
 
@@ -48,10 +65,15 @@ namespace lvs {
 
 namespace {
 
-constexpr int kEpiWG = 3;                    // epilogue warpgroups
+constexpr int kEpiWG = 2;                    // epilogue warpgroups
 constexpr int kEpiThreads = 128 * kEpiWG;
-constexpr int kThreads = 64 + kEpiThreads;
+constexpr int kThreads = 96 + kEpiThreads;
 constexpr int kStatSlots = 4;  // stats of heads s-3..s may be live across the cluster
+template <int N>
+struct Blocks {
+    static constexpr int value = N;
+};
+constexpr float kSumLimit = 7.9e28f;  // about 2^96: a pass-1 sum beyond moves its reference
 
 // Shared-memory plan. The ring gets whatever is left of the 227 KB after the
 // Q double buffer and the bookkeeping; every variant needs more than half of
@@ -66,18 +88,19 @@ struct SmemLayout {
     // Q(s+2) load while pass 2 of head s is still reading Q(s).
     static constexpr int QBUF = MROWS == 64 ? 3 : 2;
     static constexpr int FIXED = QBUF * Q_BYTES + kMaxTilesPerCta * kTileRows * 4 + kStatSlots * kMaxText * 8 +
-                                 2 * kMaxText * 4 + (kEpiWG - 1) * kMaxText * 8 + kMaxTilesPerCta * 4 + 512 + 64 +
+                                 2 * kMaxText * 4 + 2 * (kEpiWG - 1) * kMaxText * 8 + 512 + 64 +
                                  1024;
     static constexpr int STAGES_FIT = (227 * 1024 - FIXED) / TILE_BYTES;
-    static constexpr int kStages = STAGES_FIT > 10 ? 10 : STAGES_FIT;
+    // even: a stage then always belongs to the same issuer (unit u uses stage
+    // u % kStages), which makes its waits on the stage's phases sound
+    static constexpr int kStages = STAGES_FIT > 10 ? 10 : STAGES_FIT & ~1;
     static constexpr int OFF_K = 0;
     static constexpr int OFF_Q = OFF_K + kStages * TILE_BYTES;
     static constexpr int OFF_ACC = OFF_Q + QBUF * Q_BYTES;
     static constexpr int OFF_STATS = OFF_ACC + kMaxTilesPerCta * kTileRows * 4;
     static constexpr int OFF_B2 = OFF_STATS + kStatSlots * kMaxText * 8;
-    static constexpr int OFF_XS = OFF_B2 + 2 * kMaxText * 4;  // [kEpiWG - 1][128] float2: other warpgroups' row stats
-    static constexpr int OFF_FLAGS = OFF_XS + (kEpiWG - 1) * kMaxText * 8;  // [32] int, fold flags
-    static constexpr int OFF_BAR = OFF_FLAGS + kMaxTilesPerCta * 4;
+    static constexpr int OFF_XS = OFF_B2 + 2 * kMaxText * 4;  // [head & 1][kEpiWG - 1][128] float2: other warpgroups' row stats
+    static constexpr int OFF_BAR = OFF_XS + 2 * (kEpiWG - 1) * kMaxText * 8;
     // k_full[S], k_empty[S], q_full[QBUF], q_empty[QBUF], t1_full[2], t1_empty[2],
     // t2_full[2], t2_empty[2], stats[4], drain
     static constexpr int NBAR = 2 * kStages + 2 * QBUF + 2 * 4 + kStatSlots + 2;
@@ -97,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t FMT = FP8 ? 0u : 1u;
     constexpr int kStages = L::kStages;
     constexpr int QBUF = L::QBUF;
-    static_assert(kStages >= 3, "ring depth");
+    static_assert(kStages >= 4 && kStages % 2 == 0, "ring depth");
     static_assert(L::ALLOC > 116 * 1024, "one CTA per SM");
     static_assert(L::ALLOC <= 227 * 1024, "shared memory per CTA");
 
@@ -131,8 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int t0 = p.query_last && t1 > tq ? t1 - 1 : tq;  // last-token queries: one row
     const int T = t1 - t0;
     const bool multi = p.groups > 1;
-    // Uniform for the whole cluster (same request). With several head groups
-    // every CTA must still take its fold ticket, so only shape errors return.
+    // Uniform for the whole cluster (same request).
     if (T > MROWS || (N > 0 && T <= 0) || N <= 0) {
         if (p.extra) griddep_wait();
         if (N > 0 && threadIdx.x == 0 && rank == 0 && hg == 0) atomicOr(p.err, kErrShape);
@@ -144,6 +166,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tile_end = min(n_tiles, tile_begin + tpc);
     const int mt = tile_end - tile_begin;
     const int n2 = (T + 15) & ~15;
+    // pass 1 runs with M = 64 for a request of at most 64 text rows, also in the
+    // 128-row instance: its rows then lie in 16 lanes of each of the four lane
+    // quadrants, so all SM sub-partitions work on them
+    const bool m64 = MROWS == 64 || T <= 64;
     const int G = p.hq / p.hkv;
     const int hpg = p.heads_per_group;
     const float cl = p.c_log2;
@@ -162,7 +188,6 @@ __global__ void __launch_bounds__(kThreads, 1)
               DRAIN = STATS + kStatSlots, STALL = DRAIN + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 4);
-    volatile int* fold_flags = reinterpret_cast<volatile int*>(smem + L::OFF_FLAGS);
     float* acc_s = reinterpret_cast<float*>(smem + L::OFF_ACC);
     float2* stats_s = reinterpret_cast<float2*>(smem + L::OFF_STATS);
     float* b2_s = reinterpret_cast<float*>(smem + L::OFF_B2);
@@ -175,16 +200,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int i = 0; i < QBUF; ++i) {
             mbar_init(BAR(Q_FULL + i), 1);
-            mbar_init(BAR(Q_EMPTY + i), 1);
+            mbar_init(BAR(Q_EMPTY + i), 2);  // one commit per issuer
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 4; ++i) {
             mbar_init(BAR(U_FULL + i), 1);
-            mbar_init(BAR(U_EMPTY + i), 4);   // one arrival per warp of the consuming warpgroup
-            mbar_init(BAR(U_FULL + 2 + i), 1);
-            mbar_init(BAR(U_EMPTY + 2 + i), 4);
+            mbar_init(BAR(U_EMPTY + i), 4);  // one arrival per warp of the consuming warpgroup
         }
         for (int i = 0; i < kStatSlots; ++i) mbar_init(BAR(STATS + i), csize);
-        mbar_init(BAR(DRAIN), 1);
+        mbar_init(BAR(DRAIN), 2);
         mbar_init(BAR(STALL), 1);  // nothing ever arrives (the debug stall below)
         *abort_flag = 0;
         fence_mbar_init_cluster();
@@ -223,10 +246,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // that nothing completes before issuing any copy, so this wait runs out
             // of budget and every other wait of the launch runs out or sees the
             // abort flag, with no copy or contraction in flight.
-            bool ok = !p.stall || wait_phase(BAR(STALL), 0, ctl);
+            bool ok = !p.stall || poll_phase(BAR(STALL), 0, ctl);
             auto load_tiles = [&](int g) {
                 for (int t = tile_begin; t < tile_end && ok; ++t) {
-                    if (!wait_phase(BAR(K_EMPTY + ks), kph ^ 1, ctl)) { ok = false; break; }
+                    if (!poll_phase(BAR(K_EMPTY + ks), kph ^ 1, ctl)) { ok = false; break; }
                     mbar_arrive_expect_tx(BAR(K_FULL + ks), L::TILE_BYTES);
                     const uint32_t kdst = base + L::OFF_K + ks * L::TILE_BYTES;
 #pragma unroll
@@ -241,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (s < hpg) {
                     const int h = hg * hpg + s;
                     const int qb = s % QBUF;
-                    if (!wait_phase(BAR(Q_EMPTY + qb), ((s / QBUF) & 1) ^ 1, ctl)) break;
+                    if (!poll_phase(BAR(Q_EMPTY + qb), ((s / QBUF) & 1) ^ 1, ctl)) break;
                     mbar_arrive_expect_tx(BAR(Q_FULL + qb), L::Q_BYTES);
                     const uint32_t qdst = base + L::OFF_Q + qb * L::Q_BYTES;
 #pragma unroll
@@ -257,17 +280,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             volatile int no_abort = 0;
             const Ctl drain_ctl{&no_abort, p.err, kWaitBudgetCycles};
             for (int s = 0; s < kStages; ++s)
-                if (k_issued[s] > 0) wait_phase(BAR(K_FULL + s), (uint32_t)(k_issued[s] - 1) & 1u, drain_ctl);
+                if (k_issued[s] > 0) poll_phase(BAR(K_FULL + s), (uint32_t)(k_issued[s] - 1) & 1u, drain_ctl);
             for (int s = 0; s < QBUF; ++s)
-                if (q_issued[s] > 0) wait_phase(BAR(Q_FULL + s), (uint32_t)(q_issued[s] - 1) & 1u, drain_ctl);
+                if (q_issued[s] > 0) poll_phase(BAR(Q_FULL + s), (uint32_t)(q_issued[s] - 1) & 1u, drain_ctl);
         }
         __syncwarp();
         cluster_wait();
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
+    } else if (warp <= 2) {
+        // ------------------------------------------------------------ MMA issuers
+        // Lane 0 of warps 1 and 2; issuer `who` takes the units u with (u & 1)
+        // == who, their stages and TMEM buffers (both counts are even). The
+        // operand descriptors are made once per head (Q) and unit (K); each K
+        // step adds a constant to the start-address field (shared-memory
+        // offsets stay below 256 KB, so the 14-bit field never carries).
         if (lane == 0) {
+            const uint32_t who = (uint32_t)(warp - 1);
             if (mt > 0) {
-                const uint32_t idesc1 = idesc_make(MROWS, 128, FMT);
+                const uint32_t idesc1 = idesc_make(m64 ? 64 : 128, 128, FMT);
                 const uint32_t idesc2 = idesc_make(128, (uint32_t)n2, FMT);
                 uint32_t ks = 0, kph = 0, ui = 0;
                 bool ok = true;
@@ -275,29 +304,31 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int pass = 0; pass < 2 && ok; ++pass) {
                         if (pass == 0 && s >= hpg) continue;
                         if (pass == 1 && s < lag) continue;
-                        const int hs = pass == 0 ? s : s - lag;  // head of this unit
+                        const int hs = pass == 0 ? s : s - lag;  // head of these units
                         const int qb = hs % QBUF;
                         if (pass == 0) {
-                            if (!wait_phase(BAR(Q_FULL + qb), (hs / QBUF) & 1, ctl)) { ok = false; break; }
+                            if (!poll_phase(BAR(Q_FULL + qb), (hs / QBUF) & 1, ctl)) { ok = false; break; }
                             tc_fence_after();
                         }
-                        const uint32_t qaddr = base + L::OFF_Q + qb * L::Q_BYTES;
-                        for (int t = tile_begin; t < tile_end; ++t) {
-                            if (!wait_phase(BAR(K_FULL + ks), kph, ctl)) { ok = false; break; }
+                        const uint64_t qdesc = sdesc_k_sw128(base + L::OFF_Q + qb * L::Q_BYTES);
+                        for (int t = tile_begin; t < tile_end; ++t, ++ui) {
+                            const uint32_t st_ks = ks, st_ph = kph;
+                            if (++ks == kStages) { ks = 0; kph ^= 1; }
+                            if ((ui & 1u) != who) continue;
                             const uint32_t ub = ui & 3, uph = (ui >> 2) & 1;
-                            if (!wait_phase(BAR(U_EMPTY + ub), uph ^ 1, ctl)) {
+                            if (!poll_phase(BAR(K_FULL + st_ks), st_ph, ctl) ||
+                                !poll_phase(BAR(U_EMPTY + ub), uph ^ 1, ctl)) {
                                 ok = false;
                                 break;
                             }
                             tc_fence_after();
-                            const uint32_t kaddr = base + L::OFF_K + ks * L::TILE_BYTES;
+                            const uint64_t kdesc = sdesc_k_sw128(base + L::OFF_K + st_ks * L::TILE_BYTES);
                             const uint32_t d = tmem + ub * 128u;
 #pragma unroll
                             for (int st = 0; st < KSTEPS; ++st) {
-                                const uint32_t koff = (st >> 2) * (kTileRows * 128) + (st & 3) * 32;
-                                const uint32_t qoff = (st >> 2) * (MROWS * 128) + (st & 3) * 32;
-                                const uint64_t qd = sdesc_k_sw128(qaddr + qoff);
-                                const uint64_t kd = sdesc_k_sw128(kaddr + koff);
+                                constexpr uint64_t kQ16 = MROWS * 128 / 16, kK16 = kTileRows * 128 / 16;
+                                const uint64_t qd = qdesc + (uint64_t)(st >> 2) * kQ16 + (uint64_t)(st & 3) * 2;
+                                const uint64_t kd = kdesc + (uint64_t)(st >> 2) * kK16 + (uint64_t)(st & 3) * 2;
                                 if (pass == 0) {
                                     if (FP8) mma_f8(d, qd, kd, idesc1, st > 0);
                                     else mma_f16(d, qd, kd, idesc1, st > 0);
@@ -307,11 +338,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 }
                             }
                             mma_commit(BAR(U_FULL + ub));
-                            mma_commit(BAR(K_EMPTY + ks));
-                            ++ui;
-                            if (++ks == kStages) { ks = 0; kph ^= 1; }
+                            mma_commit(BAR(K_EMPTY + st_ks));
                         }
-                        if (pass == 1 && ok) mma_commit(BAR(Q_EMPTY + qb));  // last reader of Q(hs)
+                        // Q(hs) is free once both issuers' contractions of its pass 2 are done
+                        if (pass == 1 && ok) mma_commit(BAR(Q_EMPTY + qb));
                     }
                 }
             }
@@ -319,89 +349,138 @@ __global__ void __launch_bounds__(kThreads, 1)
             mma_commit(BAR(DRAIN));
             volatile int no_abort = 0;
             const Ctl drain_ctl{&no_abort, p.err, kWaitBudgetCycles};
-            wait_phase(BAR(DRAIN), 0, drain_ctl);
+            poll_phase(BAR(DRAIN), 0, drain_ctl);
         }
         __syncwarp();
         cluster_wait();
     } else {
         // ------------------------------------------------------------ epilogue
         cluster_wait();  // the peers' barriers and buffers exist before any statistics go out
-        // Three warpgroups (warps 2-5, 6-9, 10-13). The contractions of both
-        // passes cycle through four TMEM buffers in issue order; warpgroup g
-        // takes the units u with u % 3 == g, in order, so while one warpgroup
-        // reads a buffer the others' units are being filled. A unit's buffer
-        // was last used by unit u - 4, which belongs to another warpgroup and
-        // comes earlier in that warpgroup's order, so no wait is circular. Control flow is identical within a
-        // warpgroup (named barriers); after an abort every wait returns at once
-        // and the steps run out.
+        // Two warpgroups; warpgroup wg takes the units u with (u & 1) == wg. A
+        // unit's buffer was last used by unit u - 4 of the same warpgroup. Control
+        // flow is identical within a warpgroup (named barriers); after an abort
+        // every wait returns at once and the steps run out.
         const int quad = warp & 3;
-        const int wg = (warp - 2) >> 2;                       // 0 .. kEpiWG - 1
-        const int et = threadIdx.x - 64;                      // 0..255
+        const int wg = (warp - 3) >> 2;                       // 0 .. kEpiWG - 1
+        const int et = threadIdx.x - 96;                      // 0 .. kEpiThreads - 1
         const int vrow = quad * 32 + lane;                    // pass 2: TMEM lane = visual token in tile
-        const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-        // pass 1 row of this thread: M=128 -> lane; M=64 -> lanes 16q..16q+15, two column halves
-        const int prow = MROWS == 128 ? quad * 32 + lane : quad * 16 + (lane & 15);
-        const int phalf = MROWS == 128 ? 0 : (lane >> 4);
-        const bool p1_live = MROWS == 128 ? (quad * 32 < T) : (quad * 16 < T);
+        const uint32_t tcol = tmem + ((uint32_t)(quad * 32) << 16);
+        // pass 1 row of this thread: M = 128 -> lane; M = 64 -> lanes 16q..16q+15, two
+        // column halves
+        const int prow = !m64 ? quad * 32 + lane : quad * 16 + (lane & 15);
+        const bool p1_live = !m64 ? (quad * 32 < T) : (quad * 16 < T);
         for (int tl = wg; tl < mt; tl += kEpiWG) acc_s[tl * kTileRows + vrow] = 0.f;
+        const float2 cl2 = make_float2(cl, cl);
+        // this warp has read buffer ub: hand it back
+        auto release = [&](uint32_t ub) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(BAR(U_EMPTY + ub));
+        };
         uint32_t ui = 0;  // contraction units in issue order (both passes)
         for (int s = 0; s < hpg + lag; ++s) {
             if (s < hpg) {
-                // ---- pass 1 of head s: online row statistics over this warpgroup's tiles
-                float m = -INFINITY, l = 0.f;
-                for (int t = tile_begin; t < tile_end; ++t, ++ui) {
-                    const uint32_t ub = ui & 3;
-                    if ((int)(ui % kEpiWG) != wg) continue;
-                    wait_phase(BAR(U_FULL + ub), (ui >> 2) & 1, ctl);
-                    tc_fence_after();
-                    const uint32_t ta = tmem + lane_off + ub * 128u;
-                    // 32 columns at a time: M = 64 -> this thread's half of the row
-                    // (columns 64 * phalf + [0, 64)); M = 128 -> the whole row
-                    constexpr int NH = MROWS == 128 ? 4 : 2;
+                // ---- pass 1 of head s: row sums over this warpgroup's tiles
+                float ref = -INFINITY, nrc = 0.f;           // reference logit and -(ref * c)
+                float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
+                // One tile: a row's columns (128; 64 with M = 64, the other 64 with the
+                // thread 16 lanes on), in blocks of 64; `ld` reads 32 columns from c.
+                auto tile = [&](auto ld, auto blocks, uint32_t ub, int valid, bool first, bool full) {
+                    constexpr int NB = decltype(blocks)::value;
+                    // columns past the request's end: 2^-inf adds nothing
+                    auto ld_masked = [&](int c, float (&v)[32]) {
+                        ld(c, v);
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int hh = 0; hh < NH; ++hh) {
+                        for (int e = 0; e < 32; ++e) v[e] = c + e < valid ? v[e] : -INFINITY;
+                    };
+                    auto sum_masked = [&]() {
+#pragma unroll 1
+                        for (int c = 0; c < NB * 64; c += 32) {
+                            float v[32];
+                            ld_masked(c, v);
+                            row_sum_exp<32>(v, cl2, make_float2(nrc, nrc), s01, s23);
+                        }
+                    };
+                    if (first) {
                         float v[32];
-                        if (p1_live) {
-                            if constexpr (MROWS == 128) tmem_ld32(ta + hh * 32, v);
-                            else tmem_ld16x2_32<64>(ta + hh * 32, v);
-                            tmem_wait_ld();
-                        }
-                        if (hh == NH - 1) {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(BAR(U_EMPTY + ub));
-                        }
-                        if (p1_live) {
-                            const int valid = N - t * kTileRows - (MROWS == 128 ? 0 : phalf * 64) - hh * 32;
-                            row_stats_update<32>(v, valid, cl, m, l);
-                        }
+                        ld_masked(0, v);
+                        ref = row_max<32>(v);
+                        nrc = ref == -INFINITY ? 0.f : -(ref * cl);
                     }
+                    const float2 o01 = s01, o23 = s23;
+                    if (full) {
+#pragma unroll
+                        for (int k = 0; k < NB; ++k) {
+                            float va[32], vb[32];
+                            ld(k * 64, va);
+                            ld(k * 64 + 32, vb);
+                            tmem_wait_ld();
+                            row_sum_exp<32>(va, cl2, make_float2(nrc, nrc), s01, s23);
+                            row_sum_exp<32>(vb, cl2, make_float2(nrc, nrc), s01, s23);
+                        }
+                    } else {
+                        sum_masked();
+                    }
+                    // a logit far above the reference (or not a number), or no reference
+                    // yet: take the tile's maximum into the reference and redo the tile
+                    if (__any_sync(0xffffffffu, !((s01.x + s01.y) + (s23.x + s23.y) < kSumLimit) || ref == -INFINITY)) {
+                        float m = ref;
+#pragma unroll 1
+                        for (int c = 0; c < NB * 64; c += 32) {
+                            float v[32];
+                            ld_masked(c, v);
+                            m = fmaxf(m, row_max<32>(v));
+                        }
+                        const float f = ref == -INFINITY ? 0.f : ex2((ref - m) * cl);
+                        ref = m;
+                        nrc = m == -INFINITY ? 0.f : -(m * cl);
+                        s01 = make_float2(o01.x * f, o01.y * f);
+                        s23 = make_float2(o23.x * f, o23.y * f);
+                        sum_masked();
+                    }
+                    release(ub);
+                };
+                bool started = false;  // a tile of this row has been summed (warp-uniform)
+                for (int t = tile_begin; t < tile_end; ++t, ++ui) {
+                    if ((int)(ui % kEpiWG) != wg) continue;
+                    const uint32_t ub = ui & 3;
+                    poll_phase(BAR(U_FULL + ub), (ui >> 2) & 1, ctl);
+                    tc_fence_after();
+                    if (!p1_live) {
+                        release(ub);
+                        continue;
+                    }
+                    const uint32_t ta = tcol + ub * 128u;
+                    const int left = N - t * kTileRows;  // columns of the request in this tile
+                    const bool first = !started, full = left >= kTileRows;
+                    started = true;
+                    if (MROWS == 128 && !m64)
+                        tile([&](int c, float* v) { tmem_ld32(ta + (uint32_t)c, v); }, Blocks<2>{}, ub, left, first, full);
+                    else
+                        tile([&](int c, float* v) { tmem_ld16x2_32<64>(ta + (uint32_t)c, v); }, Blocks<1>{}, ub,
+                             left - (lane >> 4) * 64, first, full);
                 }
-                if (MROWS == 64) {
-                    // merge the two column halves of each row (threads t and t ^ 16)
+                float m = ref, l = (s01.x + s01.y) + (s23.x + s23.y);
+                if (m64) {
+                    // merge the two column parts of each row (threads t and t ^ 16)
                     const float mo = __shfl_xor_sync(0xffffffffu, m, 16);
                     const float lo = __shfl_xor_sync(0xffffffffu, l, 16);
-                    const float mm = fmaxf(m, mo);
-                    if (mm != -INFINITY) {
-                        l = (l > 0.f ? l * ex2((m - mm) * cl) : 0.f) + (lo > 0.f ? lo * ex2((mo - mm) * cl) : 0.f);
-                        m = mm;
-                    }
+                    merge_row(m, l, mo, lo, cl);
                 }
                 // ---- merge the warpgroups, publish (m, l) of head s to the cluster
-                const bool writer = MROWS == 128 || lane < 16;
-                if (wg > 0 && writer) xs_s[(wg - 1) * kMaxText + prow] = make_float2(m, l);
+                const bool writer = !m64 || lane < 16;
+                // (double-buffered by head: the other warpgroups may publish head s + 1
+                // while the first one is still reading head s)
+                float2* xs = xs_s + (s & 1) * (kEpiWG - 1) * kMaxText;
+                if (wg > 0 && writer) xs[(wg - 1) * kMaxText + prow] = make_float2(m, l);
                 named_bar_sync(1, kEpiThreads);
                 if (wg == 0) {
                     if (writer) {
 #pragma unroll
                         for (int o_wg = 1; o_wg < kEpiWG; ++o_wg) {  // fixed order: deterministic
-                            const float2 o = xs_s[(o_wg - 1) * kMaxText + prow];
-                            const float mm = fmaxf(m, o.x);
-                            if (mm != -INFINITY) {
-                                l = (l > 0.f ? l * ex2((m - mm) * cl) : 0.f) +
-                                    (o.y > 0.f ? o.y * ex2((o.x - mm) * cl) : 0.f);
-                                m = mm;
-                            }
+                            const float2 o = xs[(o_wg - 1) * kMaxText + prow];
+                            merge_row(m, l, o.x, o.y, cl);
                         }
                         stats_s[(s % kStatSlots) * kMaxText + prow] = make_float2(m, l);
                     }
@@ -411,18 +490,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // threads wrote before the named barrier, and the arrivals'
                     // fences (each waits for this SM's memory traffic to settle)
                     // overlap instead of running one after another
-                    if (et < (int)csize) mbar_arrive_remote(mapa_shared(BAR(STATS + s % kStatSlots), (uint32_t)et));
+                    if (csize > 1 && et < (int)csize)
+                        mbar_arrive_remote(mapa_shared(BAR(STATS + s % kStatSlots), (uint32_t)et));
                 }
             }
             if (s >= lag) {
-                // ---- merge the cluster's statistics of head s-1
+                // ---- merge the cluster's statistics of head s - lag
                 const int hs = s - lag;
                 const int slot = hs % kStatSlots;
                 float* b2 = b2_s + (hs & 1) * kMaxText;
                 if (wg == 0) {
-                    wait_phase_cluster(BAR(STATS + slot), (uint32_t)(hs / kStatSlots) & 1u, ctl);
+                    // (a CTA that is its own cluster reads its own rows, ordered by the named barrier above)
+                    if (csize > 1) poll_phase<true>(BAR(STATS + slot), (uint32_t)(hs / kStatSlots) & 1u, ctl);
                     if (et < T) {
-                        float bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + et) * 8u, csize, cl);
+                        float bm;
+                        if (csize > 1) {
+                            bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + et) * 8u, csize, cl);
+                        } else {
+                            const float2 st = stats_s[slot * kMaxText + et];
+                            bm = fmaf(st.x, cl, __log2f(st.y));
+                        }
                         if (p.extra) {
                             griddep_wait();
                             bm = log2_add(bm, p.extra[(int64_t)(t0 + et) * p.hq + hg * hpg + hs]);
@@ -433,43 +520,37 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 named_bar_sync(1, kEpiThreads);
-                // ---- pass 2 of head s-1: per-visual-token sums of probabilities
+                // ---- pass 2 of head hs: per-visual-token sums of probabilities
                 for (int t = tile_begin; t < tile_end; ++t, ++ui) {
-                    const uint32_t ub = ui & 3;
                     if ((int)(ui % kEpiWG) != wg) continue;
-                    wait_phase(BAR(U_FULL + ub), (ui >> 2) & 1, ctl);
+                    const uint32_t ub = ui & 3;
+                    poll_phase(BAR(U_FULL + ub), (ui >> 2) & 1, ctl);
                     tc_fence_after();
-                    const uint32_t ta = tmem + lane_off + ub * 128u;
                     float2 a01 = make_float2(0.f, 0.f), a23 = make_float2(0.f, 0.f);
-                    const float2 cl2 = make_float2(cl, cl);
+                    const uint32_t ta = tcol + ub * 128u;
 #pragma unroll
-                    for (int hh = 0; hh < MROWS / 32; ++hh) {
-                        const int c0 = hh * 32;
-                        if (c0 < n2) {
-                            float v[32];
-                            if (c0 + 32 <= n2) tmem_ld32(ta + c0, v);
-                            else tmem_ld16(ta + c0, v);
+                    for (int c0 = 0; c0 < MROWS; c0 += 64) {
+                        if (n2 >= c0 + 64) {  // a straight-line block of 64 columns
+                            float va[32], vb[32];
+                            tmem_ld32(ta + (uint32_t)c0, va);
+                            tmem_ld32(ta + (uint32_t)(c0 + 32), vb);
                             tmem_wait_ld();
-#pragma unroll
-                            for (int k = 0; k < 2; ++k) {
-                                if (c0 + k * 16 < n2) {
-#pragma unroll
-                                    for (int e = 0; e < 16; e += 4) {
-                                        const float4 bb = *reinterpret_cast<const float4*>(b2 + c0 + k * 16 + e);
-                                        const float2 x01 = ffma2(make_float2(v[k * 16 + e], v[k * 16 + e + 1]), cl2,
-                                                                 make_float2(bb.x, bb.y));
-                                        const float2 x23 = ffma2(make_float2(v[k * 16 + e + 2], v[k * 16 + e + 3]),
-                                                                 cl2, make_float2(bb.z, bb.w));
-                                        a01 = fadd2(a01, make_float2(ex2(x01.x), ex2(x01.y)));
-                                        a23 = fadd2(a23, make_float2(ex2(x23.x), ex2(x23.y)));
-                                    }
-                                }
-                            }
+                            if (n2 == c0 + 64) release(ub);
+                            col_sum_exp16(va, cl2, b2 + c0, a01, a23);
+                            col_sum_exp16(va + 16, cl2, b2 + c0 + 16, a01, a23);
+                            col_sum_exp16(vb, cl2, b2 + c0 + 32, a01, a23);
+                            col_sum_exp16(vb + 16, cl2, b2 + c0 + 48, a01, a23);
+                        } else if (n2 > c0) {  // the last 16, 32 or 48
+                            float va[32], vb[16];
+                            tmem_ld32(ta + (uint32_t)c0, va);
+                            tmem_ld16(ta + (uint32_t)(c0 + 32), vb);
+                            tmem_wait_ld();
+                            release(ub);
+                            col_sum_exp16(va, cl2, b2 + c0, a01, a23);
+                            if (n2 > c0 + 16) col_sum_exp16(va + 16, cl2, b2 + c0 + 16, a01, a23);
+                            if (n2 > c0 + 32) col_sum_exp16(vb, cl2, b2 + c0 + 32, a01, a23);
                         }
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(BAR(U_EMPTY + ub));
                     acc_s[(t - tile_begin) * kTileRows + vrow] += (a01.x + a01.y) + (a23.x + a23.y);
                 }
             }
@@ -485,7 +566,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 else p.partials[(int64_t)hg * p.total_vis + n0 + j] = a;
             }
         }
-        if (multi && !p.defer_fold) fold_tiles<4>(p, b, n0, N, T, tile_begin, mt, et, kEpiThreads, 1, fold_flags);
         tc_fence_before();
     }
 
@@ -497,6 +577,34 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (p.extra) griddep_wait();  // returns at once for threads that already waited
     cluster_sync_all();  // peers are done reading this CTA's statistics
+}
+
+// scores = sum over the head groups' partial rows, in group order, / (Hq * T):
+// grid (256-token chunks of the longest request, requests)
+constexpr int kFoldThreads = 256;
+
+__global__ void __launch_bounds__(kFoldThreads) fold_kernel(const __grid_constant__ FoldArgs a)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    for (int b = blockIdx.y; b < a.batch; b += gridDim.y) {
+        const int n0 = a.nv > 0 ? a.so_v[b] : a.seq_off[b];
+        const int N = (a.nv > 0 ? a.so_v[b + 1] : a.seq_off[b + 1]) - n0;
+        const int j = blockIdx.x * kFoldThreads + threadIdx.x;
+        if (j >= N) continue;
+        const int T = a.query_last ? 1 : (a.nv > 0 ? a.to_v[b + 1] - a.to_v[b] : a.text_off[b + 1] - a.text_off[b]);
+        const float* src = a.partials + n0 + j;
+        float sum = 0.f;
+        for (int g = 0; g < a.groups; g += 16) {
+            float v[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) v[q] = g + q < a.groups ? __ldcg(src + (int64_t)(g + q) * a.total_vis) : 0.f;
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                if (g + q < a.groups) sum += v[q];
+        }
+        a.out[n0 + j] = sum / ((float)a.hq * (float)T);
+    }
 }
 
 template <int ROW_BYTES, bool FP8, int MROWS>
@@ -576,10 +684,9 @@ bool score_shape_supported(int head_dim, bool fp8)
     return head_dim == 64 || head_dim == 128;
 }
 
-// CTAs of one cluster size that run at once with one CTA per SM (GPC packing
-// on a 152-SM GB300: 1, 2 -> 152; 4 -> 144; 8 -> 120; 16 -> 112).
-ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int tile_bytes, const int* cap_by_cluster,
-                     double* cost_out)
+// Launch shape of the re-read kernel with the lowest modelled time.
+ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int row_bytes, const int* cap_by_cluster,
+                     const KernelCosts& costs, double window_one, double* cost_out)
 {
     ScorePlan best{1, 1, 1};
     double best_cost = 1e300;
@@ -589,6 +696,7 @@ ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int tile_bytes, cons
         return best;
     }
     const int G = hq / hkv;
+    const double tile_bytes = (double)kTileRows * row_bytes;
     for (int pass = 0; pass < 2 && best_cost >= 1e299; ++pass) {
         for (int c = 1; c <= kMaxCluster; ++c) {
             const int tpc = (max_tiles + c - 1) / c;
@@ -600,26 +708,24 @@ ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int tile_bytes, cons
                 if (hq % g) continue;
                 const long long ctas = (long long)bt.n * c * g;
                 const int hpg = hq / g;
-                // L2 window of the pass-2 re-read: while a CTA streams up to two
-                // slices (pass 1 of the next head, rest of the current one) the
-                // tiles it re-reads must survive in L2. Groups that split a GQA
-                // key head share its tiles. The bound is loose (160 MB against
-                // 126 MB of L2): the re-read follows pass 1 within one head, and
-                // on GB300 whole-request CTAs with this nominal window measured
-                // faster than clusters of two (fp8_ragged: 176 vs 201 us).
+                // L2 window of the pass-2 re-read: while a CTA streams a slice (in a
+                // cluster up to two: pass 1 of the next head, rest of the current one)
+                // the tiles it re-reads must survive in L2. Groups that split a GQA
+                // key head share its tiles. The bound is loose (160 MB against 126 MB
+                // of L2): the re-read follows pass 1 within one head, and whole-request
+                // CTAs measured faster than clusters of two up to there (full keys,
+                // 16 requests of 4 to 21 tiles: 39.1 against 42.6 us).
                 const long long active = ctas < cap ? ctas : cap;
                 const int share = hpg >= G ? 1 : G / hpg;
-                const double window = 2.0 * tpc * tile_bytes * (double)active / share;
+                const double window = (c > 1 ? 2.0 : window_one) * tpc * tile_bytes * (double)active / share;
                 if (pass == 0 && window > 160.0 * 1024 * 1024) continue;
-                // one cluster (item): one tile-head of work per tile and head, plus
-                // a fixed launch / pipeline fill cost of about 6 tile-heads and a
-                // cluster exchange of about 1 tile-head per head; a fold when g > 1
                 auto item_cost = [&](int tiles) {
                     const int t = (tiles + c - 1) / c;
                     return tiles <= 0 ? 1.0
-                                      : (double)t * hpg + 6.0 + (c > 1 ? 1.0 : 0.25) * hpg + (g > 1 ? 2.0 : 0.0);
+                                      : costs.start + (g > 1 && !costs.fold_once ? costs.fold : 0.0) +
+                                            hpg * (t * costs.tile + (c > 1 ? costs.exchange : costs.exchange_one));
                 };
-                const double cost = makespan(bt, g, cap / c, item_cost);
+                const double cost = makespan(bt, g, cap / c, item_cost) + (g > 1 && costs.fold_once ? costs.fold : 0.0);
                 if (cost < best_cost - 1e-9) {
                     best_cost = cost;
                     best = ScorePlan{c, tpc, g};
@@ -629,6 +735,19 @@ ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int tile_bytes, cons
     }
     if (cost_out) *cost_out = best_cost;
     return best;
+}
+
+cudaError_t launch_fold(const FoldArgs& a, int max_n, cudaStream_t stream)
+{
+    if (a.batch <= 0 || max_n <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((max_n + kFoldThreads - 1) / kFoldThreads), (unsigned)(a.batch < 65535 ? a.batch : 65535), 1);
+    cfg.blockDim = dim3(kFoldThreads, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fold_kernel, a);
 }
 
 cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const ScoreLaunch& p,

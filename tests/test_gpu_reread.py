@@ -1,0 +1,110 @@
+"""The re-read score kernel where its rules change path: 64 / 65 text rows (pass 1
+with M = 64 or 128, mixed in one batch), partial and single tiles, one and several
+head groups, and logits that leave the reference of the first tile behind by more
+than the 2^96 its sums may grow (upwards, so that pass 1 redoes a tile, and
+downwards)."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import assert_scores_close, to_device
+from paper_2506_07416_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def sel():
+    if not torch.cuda.is_available():
+        pytest.fail("the GPU tests need a CUDA device")
+    from paper_2506_07416_gb300 import select
+    return select
+
+
+def _w(name, n, t, hq, hkv, d=128, dtype="bf16", sigma=0.3, seed=41):
+    return inputs.Workload(name, len(n), list(n), list(t), hq, hkv, d, 256, dtype, keep_ratio=0.3, sigma=sigma,
+                           seed=seed)
+
+
+CASES = [
+    _w("rows_64_65_128", [300, 257, 128, 1, 640], [64, 65, 128, 1, 63], 8, 4),
+    _w("rows_up_to_64", [129, 127, 900], [64, 17, 1], 8, 8),
+    _w("d64_rows", [300, 513], [65, 33], 14, 2, d=64),
+    _w("e4m3_rows", [700, 130, 128], [32, 128, 64], 8, 8, dtype="e4m3"),
+    _w("long_one_head", [5000], [100], 1, 1),
+]
+
+
+def _scores(s, x, xd):
+    g = s.score(xd["q"], xd["text_offsets"], xd["k"], xd["seq_offsets"], xd["q_scale"], xd["k_scale"],
+                seq_offsets_h=x["seq_offsets"], text_offsets_h=x["text_offsets"])
+    s.check_device()
+    return g.cpu().numpy()
+
+
+@pytest.mark.parametrize("w", CASES, ids=lambda w: w.name)
+def test_rows_tiles_and_groups(sel, w):
+    x = inputs.make_numpy(w)
+    xd = to_device(x, w)
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel="reread")
+    assert s.score_plan(x["text_offsets"], x["seq_offsets"])[0] == 1
+    o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, w.head_dim, w.dtype,
+                     x["q_scale"], x["k_scale"])
+    g = _scores(s, x, xd)
+    assert_scores_close(g, o, w.dtype)
+    np.testing.assert_array_equal(g, _scores(s, x, xd))
+    s.close()
+
+
+@pytest.mark.parametrize("t", [20, 64, 100])
+@pytest.mark.parametrize("later", [40.0, -40.0])
+def test_logits_far_from_the_first_tiles_reference(sel, t, later):
+    # every query is one unit direction times 10; the keys of the first 128 tokens lie near 0 along it, those
+    # of token 200 on at `later` +- 1: logits 10 * later / sqrt(128) = +-35 and, times 4 in token 333, +-141 nats
+    # (204 in log2), beyond the 96 that pass 1 lets its sums grow.
+    # x = s * c - b is rounded at |x| <= 2 * 204: relative error of 2^x up to 408 * 2^-24 * ln 2 = 1.7e-5,
+    # well inside the bf16 bound of 2e-3.
+    w = _w("far", [700], [t], 4, 2)
+    rng = np.random.Generator(np.random.PCG64(3))
+    d = rng.standard_normal(128)
+    d /= np.linalg.norm(d)
+    q = 10.0 * d + 0.02 * rng.standard_normal((t, w.hq, 128))
+    k = 0.1 * rng.standard_normal((700, w.hkv, 128))
+    k[200:] += (later + rng.standard_normal((500, w.hkv, 1))) * d
+    k[333] *= 4.0
+    x = {"q": inputs.f32_to_bf16_bits(q.astype(np.float32)), "k": inputs.f32_to_bf16_bits(k.astype(np.float32)),
+         "seq_offsets": w.seq_offsets(), "text_offsets": w.text_offsets(), "q_scale": 1.0, "k_scale": 1.0}
+    xd = to_device(x, w)
+    s = sel.Selector(1, 700, t, w.hq, w.hkv, 128, "bf16", score_kernel="reread")
+    o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, 128, "bf16")
+    assert_scores_close(_scores(s, x, xd), o, "bf16")
+    s.close()
+
+
+def test_no_alloc_limit_does_not_follow_the_plan(sel):
+    """A batch whose chosen launch would need more partial rows than the static scratch holds, but whose fixed
+    shape does not, is still taken."""
+    for copies in (3, 4, 5, 6, 8, 10):
+        w = _w("limit", [2600, 1800, 3000, 2400] * copies, [100, 65, 90, 128] * copies, 32, 8)
+        so, to = w.seq_offsets(), w.text_offsets()
+        s = sel.Selector(w.batch, w.total_vis, w.total_txt, 32, 8, 128, "bf16")
+        plan = s.score_plan(to, so)
+        if plan[3] * w.total_vis > 1 << 20:
+            break
+        s.close()
+    else:
+        pytest.fail("no batch among these splits its heads beyond the scratch")
+    xd = inputs.make_torch(w, "cuda")
+    ref = s.score(xd["q"], xd["text_offsets"], xd["k"], xd["seq_offsets"], seq_offsets_h=so, text_offsets_h=to)
+    s.check_device()
+    out = torch.full((w.total_vis,), float("nan"), device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    sel.score_noalloc(32, 8, 128, "bf16", w.batch, xd["q"], xd["text_offsets"], to, xd["k"], xd["seq_offsets"], so,
+                      1.0, 1.0, out, err)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    # two kernels, sums in another order: 32-bit rounding over at most 128 * 32 terms a score
+    assert float(((out - ref).abs() / ref).max()) < 1e-5
+    s.close()
