@@ -133,12 +133,13 @@ int64_t keep_count_host(int32_t n, float ratio)
 }
 
 litevlm_status_t encode_rows_map(litevlm_select_t h, CUtensorMap* map, const void* base, int32_t head_dim,
-                                 int32_t heads, int64_t rows, int box_rows, bool fp8, const char* what)
+                                 int32_t heads, int64_t rows, int box_rows, bool fp8, const char* what,
+                                 int box_heads = 1)
 {
     const int esize = fp8 ? 1 : 2;
     const cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)heads, (cuuint64_t)rows};
     const cuuint64_t strides[2] = {(cuuint64_t)head_dim * esize, (cuuint64_t)heads * head_dim * esize};
-    const cuuint32_t box[3] = {(cuuint32_t)(128 / esize), 1u, (cuuint32_t)box_rows};
+    const cuuint32_t box[3] = {(cuuint32_t)(128 / esize), (cuuint32_t)box_heads, (cuuint32_t)box_rows};
     const cuuint32_t estride[3] = {1u, 1u, 1u};
     const CUresult r = h->encode(map, fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                                  const_cast<void*>(base), dims, strides, box, estride,
@@ -176,7 +177,7 @@ bool uniform_batch(int batch, const int32_t* seq_offsets_h, const int32_t* text_
 // of HBM bandwidth. Waves of CTAs come from the measured cluster occupancy.
 //   Re-read kernel: 6 to start (launch, set-up, first copies and contractions
 // from cold memory) and leave; per head two passes over the tiles, 1.2 a tile for
-// 256-byte rows with more than 64 text rows (the contractions' operands come out
+// 256-byte rows with more than 64 query rows (the contractions' operands come out
 // of shared memory at its full rate beside the copies coming in), 1.0 up to 64,
 // 0.75 for 128-byte rows; 1.5 for the exchange over a cluster, 0.5 within one CTA;
 // the fold is a launch of its own, 2. It computes every contraction twice but has
@@ -223,18 +224,24 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     const double hbm_bytes_per_us = 6.8e6;
     const double tile_bytes = (double)lvs::kTileRows * row_bytes;
     double tc_cost = 0.0;
-    int* tcap = h->tc_capacity[mrows == 64 ? 0 : 1];
+    // query heads of a key head that fit beside each other in the re-read kernel's 128 rows
+    const int G = hq / c.num_kv_heads;
+    int hp = 1;
+    for (int d = 2; d <= G && !limit_rule; ++d)
+        if (G % d == 0 && d * max_t <= lvs::kMaxText) hp = d;
+    int* tcap = h->tc_capacity[hp * max_t <= 64 ? 0 : 1];
     for (int cl = 1; cl <= lvs::kMaxCluster; ++cl)
-        if (tcap[cl] < 0) tcap[cl] = lvs::tc_cluster_capacity(row_bytes, fp8, mrows, cl);
+        if (tcap[cl] < 0) tcap[cl] = lvs::tc_cluster_capacity(row_bytes, fp8, hp * max_t <= 64 ? 64 : 128, cl);
     const double u = 1.17;
     const lvs::KernelCosts res_costs = limit_rule ? lvs::KernelCosts{6.0 * u, u, u, 0.25 * u, 2.0 * u, false}
                                                   : lvs::KernelCosts{8.0, 0.8, 0.8, 0.25, 2.0, false};
     const double two_tile = limit_rule ? 0.6 * u : 0.6, two_head = limit_rule ? 2.1 * u : 2.1;
     const lvs::KernelCosts tc_costs =
         limit_rule ? lvs::KernelCosts{9.6 * u, 1.6 * u, 1.6 * u, 0.4 * u, 3.2 * u, false}
-                   : lvs::KernelCosts{6.0, row_bytes == 256 ? (max_t > 64 ? 1.2 : 1.0) : 0.75, 1.5, 0.5, 2.0, true};
-    ScoreChoice best{false, lvs::plan_score(bt, hq, c.num_kv_heads, row_bytes, tcap, tc_costs, limit_rule ? 2.0 : 1.0,
-                                            &tc_cost)};
+                   : lvs::KernelCosts{6.0, row_bytes == 256 ? (hp * max_t > 64 ? 1.2 : 1.0) : 0.75, 1.5, 0.5, 2.0, true};
+    ScoreChoice best{false, lvs::plan_score(bt, hq / hp, c.num_kv_heads, row_bytes, tcap, tc_costs,
+                                            limit_rule ? 2.0 : 1.0, &tc_cost)};
+    best.plan.hp = hp;
     double best_cost = limit_rule ? tc_cost : tc_cost / 0.9;
     const int max_tiles = batch > 0 ? td[0] : 0;
     const bool split_queries = (c.flags & LITEVLM_FLAG_SCORE_SPLIT_QUERIES) != 0;
@@ -585,10 +592,11 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     if (plan.tiles_per_cta > lvs::kMaxTilesPerCta)
         return fail(h, LITEVLM_ERR_UNSUPPORTED, "request too long for one cluster");
     const bool qsplit = choice.resident && plan.qsplit == 2;
-    const int mrows = max_t <= 64 || qsplit ? 64 : 128;  // text rows of a head's (pseudo-head's) MMA
+    // query rows of a head's (pseudo-head's, head block's) MMA
+    const int mrows = max_t * plan.hp <= 64 || qsplit ? 64 : 128;
 
     CUtensorMap tm_q, tm_k;
-    s = encode_rows_map(h, &tm_q, q_text, c.head_dim, c.num_q_heads, tot_t, mrows, fp8, "q_text");
+    s = encode_rows_map(h, &tm_q, q_text, c.head_dim, c.num_q_heads, tot_t, mrows / plan.hp, fp8, "q_text", plan.hp);
     if (s != LITEVLM_OK) return s;
     s = encode_rows_map(h, &tm_k, k_vis, c.head_dim, c.num_kv_heads, tot_n, lvs::kTileRows, fp8, "k_vis");
     if (s != LITEVLM_OK) return s;

@@ -26,8 +26,11 @@ struct ScoreLaunch {
     int32_t* err;
     int64_t total_vis;        // partial-row stride
     int32_t hq, hkv;
-    int32_t heads_per_group;
+    int32_t heads_per_group;  // (re-read kernel: head blocks)
     int32_t groups;
+    // re-read kernel: query heads of one key head whose text rows share a
+    // contraction (a head block), and text rows per Q tile (instance rows / hp)
+    int32_t hp, box_rows;
     int32_t ctas_per_request; // cluster size * groups
     int32_t slot_cols;        // resident kernel: TMEM columns per slot (query rows per head, rounded up to 16)
     // resident kernel: 1, or 2 when each query head's text rows run as two
@@ -72,6 +75,7 @@ struct ScorePlan {
     int res_nb = 1;           // resident kernel: TMEM head buffers
     int flat = 0;             // resident kernel: clusters of the flattened (request, head) schedule, 0: none
     int qsplit = 1;           // resident kernel: 2 = each head's text rows as two pseudo-heads (64-row kernel)
+    int hp = 1;               // re-read kernel: query heads per head block
 };
 
 // The head groups' partial rows added up (re-read kernel with several groups).

@@ -10,7 +10,7 @@
 // Work decomposition. One thread-block cluster of C CTAs serves one (request,
 // head group); CTA r of the cluster owns a contiguous range of 128-token tiles
 // of the request. For every query head h of the group:
-//   pass 1: D1 = Q_h * K_tile^T on tcgen05 (M = 64 or 128 text rows, N = 128
+//   pass 1: D1 = Q_h * K_tile^T on tcgen05 (M = 64 or 128 query rows, N = 128
 //           visual columns) into TMEM; each epilogue thread keeps, for its text
 //           row, a reference logit and the sum of 2^((s - ref) * c) over its
 //           columns of the CTA's tiles;
@@ -21,6 +21,11 @@
 //   pass 2: D2 = K_tile * Q_h^T (M = 128 visual rows, N = T rounded up to 16)
 //           into TMEM; one epilogue thread per visual token adds
 //           sum_i 2^(s_ij * c - b_hi) to its running score.
+// Text rows are packed: the hp query heads of one key head that fit beside each
+// other in 128 rows (hp * T <= 128) form a head block, row i * hp + h of its Q
+// tile being text row i of head h. "Head" below means such a block: it streams
+// the key head's tiles once instead of hp times (last-token queries of 64
+// requests, 32 / 8 heads: 314 -> 106 us).
 // Software pipeline with one head of look-ahead: pass 1 of head s+1 runs while
 // the statistics of head s travel across the cluster, then pass 2 of head s
 // (a CTA that is its own cluster has nothing to wait for and runs the two
@@ -154,8 +159,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int t0 = p.query_last && t1 > tq ? t1 - 1 : tq;  // last-token queries: one row
     const int T = t1 - t0;
     const bool multi = p.groups > 1;
+    const int hp = p.hp, R = T * hp;  // query heads and rows of a head block
     // Uniform for the whole cluster (same request).
-    if (T > MROWS || (N > 0 && T <= 0) || N <= 0) {
+    if (R > MROWS || (N > 0 && T <= 0) || N <= 0) {
         if (p.extra) griddep_wait();
         if (N > 0 && threadIdx.x == 0 && rank == 0 && hg == 0) atomicOr(p.err, kErrShape);
         return;
@@ -165,11 +171,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tile_begin = min(n_tiles, (int)rank * tpc);
     const int tile_end = min(n_tiles, tile_begin + tpc);
     const int mt = tile_end - tile_begin;
-    const int n2 = (T + 15) & ~15;
-    // pass 1 runs with M = 64 for a request of at most 64 text rows, also in the
+    const int n2 = (R + 15) & ~15;
+    // pass 1 runs with M = 64 for a request of at most 64 query rows, also in the
     // 128-row instance: its rows then lie in 16 lanes of each of the four lane
     // quadrants, so all SM sub-partitions work on them
-    const bool m64 = MROWS == 64 || T <= 64;
+    const bool m64 = MROWS == 64 || R <= 64;
     const int G = p.hq / p.hkv;
     const int hpg = p.heads_per_group;
     const float cl = p.c_log2;
@@ -211,6 +217,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(BAR(STALL), 1);  // nothing ever arrives (the debug stall below)
         *abort_flag = 0;
         fence_mbar_init_cluster();
+    }
+    // Q rows past the copied box (MROWS not a multiple of hp) enter pass 2 as
+    // columns whose terms are 2^-inf: they must be numbers
+    for (int x = threadIdx.x; x < QBUF * L::KB * (MROWS - hp * p.box_rows) * 8; x += kThreads) {
+        const int rows = MROWS - hp * p.box_rows, blk = x / (rows * 8), o = x - blk * (rows * 8);
+        *reinterpret_cast<uint4*>(smem + L::OFF_Q + blk * MROWS * 128 + hp * p.box_rows * 128 + o * 16) =
+            make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async_shared();
     }
     if (warp == 0 && lane == 0) {
         tma_prefetch_desc(&tm_q);
@@ -262,10 +276,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             };
             for (int s = 0; s < hpg + lag && ok; ++s) {
                 if (s < hpg) {
-                    const int h = hg * hpg + s;
+                    const int h = (hg * hpg + s) * hp;
                     const int qb = s % QBUF;
                     if (!poll_phase(BAR(Q_EMPTY + qb), ((s / QBUF) & 1) ^ 1, ctl)) break;
-                    mbar_arrive_expect_tx(BAR(Q_FULL + qb), L::Q_BYTES);
+                    mbar_arrive_expect_tx(BAR(Q_FULL + qb), (uint32_t)(L::KB * 128 * hp * p.box_rows));
                     const uint32_t qdst = base + L::OFF_Q + qb * L::Q_BYTES;
 #pragma unroll
                     for (int kb = 0; kb < L::KB; ++kb)
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     ++q_issued[qb];
                     load_tiles(h / G);
                 }
-                if (s >= lag && ok) load_tiles((hg * hpg + s - lag) / G);
+                if (s >= lag && ok) load_tiles((hg * hpg + s - lag) * hp / G);
             }
             // drain: the last load of every slot lands before the CTA leaves
             // (these waits ignore the abort flag)
@@ -368,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // pass 1 row of this thread: M = 128 -> lane; M = 64 -> lanes 16q..16q+15, two
         // column halves
         const int prow = !m64 ? quad * 32 + lane : quad * 16 + (lane & 15);
-        const bool p1_live = !m64 ? (quad * 32 < T) : (quad * 16 < T);
+        const bool p1_live = !m64 ? (quad * 32 < R) : (quad * 16 < R);
         for (int tl = wg; tl < mt; tl += kEpiWG) acc_s[tl * kTileRows + vrow] = 0.f;
         const float2 cl2 = make_float2(cl, cl);
         // this warp has read buffer ub: hand it back
@@ -502,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (wg == 0) {
                     // (a CTA that is its own cluster reads its own rows, ordered by the named barrier above)
                     if (csize > 1) poll_phase<true>(BAR(STATS + slot), (uint32_t)(hs / kStatSlots) & 1u, ctl);
-                    if (et < T) {
+                    if (et < R) {
                         float bm;
                         if (csize > 1) {
                             bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + et) * 8u, csize, cl);
@@ -512,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                         if (p.extra) {
                             griddep_wait();
-                            bm = log2_add(bm, p.extra[(int64_t)(t0 + et) * p.hq + hg * hpg + hs]);
+                            bm = log2_add(bm, p.extra[(int64_t)(t0 + et / hp) * p.hq + (hg * hpg + hs) * hp + et % hp]);
                         }
                         b2[et] = -bm;  // stored negated: the fma addend of pass 2
                     } else {
@@ -755,7 +769,9 @@ cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const
 {
     ScoreLaunch q = p;
     q.groups = plan.groups;
-    q.heads_per_group = p.hq / plan.groups;
+    q.hp = plan.hp;
+    q.box_rows = mrows / plan.hp;
+    q.heads_per_group = p.hq / plan.hp / plan.groups;
     q.ctas_per_request = plan.cluster * plan.groups;
     if (fp8) {
         return mrows == 64 ? launch_variant<128, true, 64>(tm_q, tm_k, q, plan, batch, stream)

@@ -34,6 +34,11 @@ CASES = [
     _w("d64_rows", [300, 513], [65, 33], 14, 2, d=64),
     _w("e4m3_rows", [700, 130, 128], [32, 128, 64], 8, 8, dtype="e4m3"),
     _w("long_one_head", [5000], [100], 1, 1),
+    _w("pack7_126_rows", [300, 128, 77], [18, 5, 1], 14, 2),
+    _w("pack7_63_rows", [300, 129], [9, 4], 7, 1, d=64),
+    _w("pack4_128_rows", [513, 40, 1200], [32, 31, 7], 16, 4),
+    _w("pack2_of_4", [257, 640], [64, 33], 8, 2),
+    _w("pack4_e4m3", [400, 129], [16, 3], 8, 2, dtype="e4m3"),
 ]
 
 
@@ -55,6 +60,36 @@ def test_rows_tiles_and_groups(sel, w):
     g = _scores(s, x, xd)
     assert_scores_close(g, o, w.dtype)
     np.testing.assert_array_equal(g, _scores(s, x, xd))
+    s.close()
+
+
+@pytest.mark.parametrize("query", ["all", "last"])
+@pytest.mark.parametrize("t", [[18, 7], [30, 11]])
+def test_packed_heads_with_the_full_key_set(sel, t, query):
+    w = _w("packed_full", [300, 150], t, 14, 2)
+    x = inputs.make_numpy(w)
+    xd = to_device(x, w)
+    n_sys = [5, 0]
+    c = inputs.context_keys_numpy(w, n_sys, seed=24)
+    dev = lambda a: torch.from_numpy(a.view(np.int16).copy()).view(torch.bfloat16).cuda()
+    sys_off = np.concatenate([[0], np.cumsum(n_sys)]).astype(np.int32)
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel="reread",
+                     query=query)
+    out = s.score_full_keys(xd["q"], xd["text_offsets"], xd["k"], xd["seq_offsets"], dev(c["k_sys"]),
+                            torch.from_numpy(sys_off).cuda(), dev(c["k_txt"]), seq_offsets_h=x["seq_offsets"],
+                            text_offsets_h=x["text_offsets"], sys_offsets_h=sys_off)
+    s.check_device()
+    if query == "all":
+        o = oracle.score_full(x["q"], x["k"], c["k_sys"], c["k_txt"], x["seq_offsets"], x["text_offsets"], sys_off,
+                              w.hq, w.hkv, w.head_dim, w.dtype)
+    else:  # the last text row sees every text key: a one-row request whose other text keys count as system keys
+        to = x["text_offsets"]
+        rows = np.array([to[1] - 1, to[2] - 1])
+        ks = np.concatenate([c["k_sys"], c["k_txt"][:to[1] - 1], c["k_txt"][to[1]:to[2] - 1]])
+        so2 = np.array([0, 5 + t[0] - 1, 5 + t[0] - 1 + t[1] - 1], np.int32)
+        o = oracle.score_full(x["q"][rows], x["k"], ks, c["k_txt"][rows], x["seq_offsets"],
+                              np.arange(3, dtype=np.int32), so2, w.hq, w.hkv, w.head_dim, w.dtype)
+    assert_scores_close(out.cpu().numpy(), o, w.dtype)
     s.close()
 
 
