@@ -7,19 +7,31 @@
 // cos / sin from a table indexed by the row's position.
 //
 // The RMSNorm weight is folded into W once (fold kernel below), so the
-// contraction reads the raw hidden rows; the per-row scale s_r is a sum of
-// squares taken from the A tiles while they sit in shared memory for the
-// tensor core, and is applied in the epilogue with the bias and the rotation.
+// contraction reads the raw hidden rows, and the per-row scale s_r is applied in
+// the epilogue with the bias and the rotation.
 //
-// One CTA per (128 * MT) x BN output tile (BN = 256 or 128 columns, whole
-// heads; MT = 2 when the grid still gives every SM two tiles): warp 0 streams
-// A (128 * MT rows x 64 hidden) and B (BN rows of W' x 64) tiles by TMA into a
-// 3- or 4-stage ring; warp 1 issues tcgen05.mma (M = 128 per row block,
-// N = BN, K = 16, bf16, fp32 accumulators in TMEM); two epilogue warpgroups sum
-// the squares of their rows of each A tile (a ring slot is free once the MMA
-// and these warps are done with it), then read the accumulator (TMEM lane =
-// row), scale, add the bias, rotate, round to bf16 and store. Every wait is
-// bounded.
+// Row scales: a small kernel launched just before (one warp per row). The
+// contraction kernel starts under it (programmatic dependent launch) and only its
+// epilogue waits for it, so the second read of x overlaps the first tiles. Summing
+// the squares from the A tiles in shared memory instead, as this kernel used to,
+// took a quarter of the shared-memory bandwidth that the contraction needs.
+//
+// Contraction: pairs of CTAs (clusters of two, cta_group::2) work through output
+// tiles of 256 rows x BN columns (BN = 256, or 128 where the columns leave no
+// choice), N tiles fastest, so that the tiles in flight share their rows of x and
+// W' stays in L2. Each CTA stages its 128 rows of x and half of the tile's rows of
+// W' (64 hidden values a stage); one thread of the first CTA issues the
+// tcgen05.mma (M = 256, N = BN, K = 16) for both. A CTA's operands then take
+// 64 bytes a clock out of shared memory and 64 in, its limit of 128; one CTA alone
+// on 128 x 256 needs 96 and 96. Accumulators alternate between two TMEM buffers:
+// the epilogue of a tile runs under the contraction of the next. Against one-CTA
+// tiles of 256 x 256 with the sums taken from shared memory: 27648 x 4096 -> 4096
+// 755 -> 625 us (1.48 PFLOP/s), 6157 x 3584 -> 512 34.3 -> 28 us, 1536 x 2048 ->
+// 2048 25.5 -> 20.3 us (48 tiles on 76 pairs, 10 us of it launch, set-up and the
+// single epilogue).
+//   warp 0: TMA producer; warp 1: TMEM, and in the first CTA the MMA issuer; warps
+//   2-9: epilogue, two warpgroups that split a tile's columns by whole heads.
+// Every wait is bounded.
 
 #include <math.h>
 
@@ -34,24 +46,22 @@ namespace lvs {
 namespace {
 
 constexpr int kProjThreads = 320;  // producer, MMA issuer, two epilogue warpgroups
-constexpr int kProjK = 64;  // hidden values per stage (128 bytes of bf16)
+constexpr int kProjK = 64;         // hidden values per stage (128 bytes of bf16)
+constexpr int kProjRows = 128;     // rows of a tile per CTA
 
-// MT row blocks of 128 per CTA (one accumulator each, MT * BN TMEM columns):
-// MT = 2 halves the operand bytes per MMA cycle (each W' tile serves 256 rows).
-template <int BN, int MT>
+template <int BN>
 struct ProjLayout {
-    static constexpr int A_BYTES = MT * 128 * 128;
-    static constexpr int B_BYTES = BN * 128;
+    static constexpr int A_BYTES = kProjRows * 128;
+    static constexpr int B_BYTES = BN / 2 * 128;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int FIT = (225 * 1024) / STAGE;
-    static constexpr int STAGES = FIT > 4 ? 4 : FIT;
+    static constexpr int STAGES = 192 * 1024 / STAGE;
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + STAGES * A_BYTES;
-    static constexpr int OFF_BAR = OFF_B + STAGES * B_BYTES;  // full[S], empty[S], acc
-    static constexpr int OFF_MISC = OFF_BAR + (2 * STAGES + 1) * 8;
-    static constexpr int OFF_SC = OFF_MISC + 16;               // [128] row scales (MT = 1)
-    static constexpr int ALLOC = OFF_SC + 128 * 4 + 1024;
-    static constexpr int TMEM_COLS = MT * BN;
+    static constexpr int OFF_ROPE = OFF_B + STAGES * B_BYTES;  // 4 KB per epilogue warp
+    static constexpr int OFF_BAR = OFF_ROPE + 8 * 4096;        // full[S], empty[S], acc_full[2], acc_empty[2], drain
+    static constexpr int OFF_MISC = OFF_BAR + (2 * STAGES + 5) * 8;
+    static constexpr int ALLOC = OFF_MISC + 16 + 1024;
+    static constexpr int TMEM_COLS = 2 * BN;
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
@@ -66,71 +76,101 @@ __device__ __forceinline__ uint32_t pack_e4m3(float lo, float hi)
     return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(lo, hi), __NV_SATFINITE, __NV_E4M3);
 }
 
-// 32 consecutive outputs of one row from 16 value pairs: bf16 (64 bytes), or
-// e4m3 codes of y / scale (32 bytes) when the call asked for e4m3
-__device__ __forceinline__ void store_pairs(const ProjArgs& p, int64_t elem, const float2 (&y)[16])
+// 2 * NP consecutive outputs of one row from NP value pairs: bf16, or e4m3 codes
+// of y / scale when the call asked for e4m3
+template <int NP>
+__device__ __forceinline__ void store_pairs(const ProjArgs& p, int64_t elem, const float2 (&y)[NP])
 {
     if (p.y8) {
-        uint32_t o[8];
+        uint32_t o[NP / 2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
+        for (int q = 0; q < NP / 2; ++q)
             o[q] = pack_e4m3(y[2 * q].x * p.out_inv_scale, y[2 * q].y * p.out_inv_scale) |
                    (pack_e4m3(y[2 * q + 1].x * p.out_inv_scale, y[2 * q + 1].y * p.out_inv_scale) << 16);
         uint4* d = reinterpret_cast<uint4*>(p.y8 + elem);
-        d[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        d[1] = make_uint4(o[4], o[5], o[6], o[7]);
-    } else {
-        uint32_t o[16];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) o[q] = pack_bf16(y[q].x, y[q].y);
+        for (int q = 0; q < NP / 8; ++q) d[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+    } else {
+        uint32_t o[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) o[q] = pack_bf16(y[q].x, y[q].y);
         uint4* d = reinterpret_cast<uint4*>(p.y + elem);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) d[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        for (int q = 0; q < NP / 4; ++q) d[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
     }
 }
 
-// scale, bias, rotation and store (bf16 or e4m3) of columns [c_begin, c_end) of one
-// accumulator row (this thread's); the range holds whole heads
-__device__ __forceinline__ void proj_store_row(const ProjArgs& p, uint32_t ta, int64_t grow, int n0, int c_begin,
-                                               int c_end, bool live, float sc)
-{
-    int pos = 0;
-    if (live && p.head_dim > 0) {
-        pos = p.positions[grow];
-        if (pos < 0 || pos >= p.max_positions) {
-            atomicOr(p.err, kErrBounds);
-            pos = 0;
+// A warp's window on the rotation table: the (cos, sin) pairs [16 c, 16 c + 16) of
+// its 32 rows' positions, 128 bytes a row, in 4 KB of its own shared memory. The
+// warp fetches four rows per load instruction (eight lanes a row, whole 128-byte
+// lines); lane r then reads row r, whose 16-byte pieces are stored at piece ^ (r &
+// 7) so that eight lanes hit eight different bank groups. A lane reading its own
+// row straight from global memory touches 32 lines per instruction: 5 M of an L1's
+// wavefronts on 6912 x 4096 -> 4096, 28 instead of 18 us on 1536 x 2048 -> 2048.
+struct RopeWindow {
+    const float2* table;
+    uint8_t* buf;
+    int half, pos, lane;
+    uint4 next[8];
+
+    __device__ __forceinline__ void fetch(int c)
+    {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int rp = __shfl_sync(0xffffffffu, pos, 4 * i + (lane >> 3));
+            const float2* src = table + (int64_t)rp * half + 16 * c + 2 * (lane & 7);
+            const float2 a = __ldg(src), b = __ldg(src + 1);
+            next[i] = make_uint4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(b.x), __float_as_uint(b.y));
         }
     }
+    __device__ __forceinline__ void put()
+    {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + (lane >> 3);
+            *reinterpret_cast<uint4*>(buf + r * 128 + (((lane & 7) ^ (r & 7)) << 4)) = next[i];
+        }
+        __syncwarp();
+    }
+    __device__ __forceinline__ float4 pairs(int j) const  // pairs 2j and 2j + 1 of this lane's row
+    {
+        return *reinterpret_cast<const float4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4));
+    }
+};
+
+// scale, bias, rotation and store (bf16 or e4m3) of columns [c_begin, c_end) of one
+// accumulator row (this thread's); the range holds whole heads. With a rotation the
+// warp's window holds the pairs of chunk 0 on entry (and may be left at another).
+__device__ __forceinline__ void proj_store_row(const ProjArgs& p, uint32_t ta, int64_t grow, int n0, int c_begin,
+                                               int c_end, bool live, float sc, RopeWindow& w)
+{
     const int64_t row0 = grow * (int64_t)p.out_features + n0;  // element index of this tile's first column
     if (p.head_dim > 0) {
-        const int half = p.head_dim / 2;
-        const float2* cs_row = p.rope + (int64_t)pos * half;
-        for (int h0 = c_begin; h0 < c_end; h0 += p.head_dim) {
-            for (int c = 0; c < half; c += 32) {
-                float v1[32], v2[32];
-                tmem_ld32(ta + (uint32_t)(h0 + c), v1);
-                tmem_ld32(ta + (uint32_t)(h0 + half + c), v2);
+        const int half = p.head_dim / 2, nc = half / 16;
+        for (int c = 0; c < nc; ++c) {
+            w.put();
+            if (c + 1 < nc) w.fetch(c + 1);
+            for (int h0 = c_begin; h0 < c_end; h0 += p.head_dim) {
+                float v1[16], v2[16];
+                tmem_ld16(ta + (uint32_t)(h0 + 16 * c), v1);
+                tmem_ld16(ta + (uint32_t)(h0 + half + 16 * c), v2);
                 tmem_wait_ld();
-                if (live) {
-                    float2 a[16], b[16];
+                const int col = n0 + h0 + 16 * c;
+                float2 a[8], b[8];
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int col1 = n0 + h0 + c + j;
-                        const float y1 = fmaf(v1[j], sc, p.bias ? p.bias[col1] : 0.f);
-                        const float y2 = fmaf(v2[j], sc, p.bias ? p.bias[col1 + half] : 0.f);
-                        const float2 cs = cs_row[c + j];
-                        const float r1 = y1 * cs.x - y2 * cs.y, r2 = y2 * cs.x + y1 * cs.y;
-                        if (j & 1) {
-                            a[j / 2].y = r1;
-                            b[j / 2].y = r2;
-                        } else {
-                            a[j / 2].x = r1;
-                            b[j / 2].x = r2;
-                        }
-                    }
-                    store_pairs(p, row0 + h0 + c, a);
-                    store_pairs(p, row0 + h0 + half + c, b);
+                for (int j = 0; j < 8; ++j) {
+                    const float4 cs = w.pairs(j);
+                    const float y1 = fmaf(v1[2 * j], sc, p.bias ? p.bias[col + 2 * j] : 0.f);
+                    const float y2 = fmaf(v2[2 * j], sc, p.bias ? p.bias[col + half + 2 * j] : 0.f);
+                    const float z1 = fmaf(v1[2 * j + 1], sc, p.bias ? p.bias[col + 2 * j + 1] : 0.f);
+                    const float z2 = fmaf(v2[2 * j + 1], sc, p.bias ? p.bias[col + half + 2 * j + 1] : 0.f);
+                    a[j] = make_float2(y1 * cs.x - y2 * cs.y, z1 * cs.z - z2 * cs.w);
+                    b[j] = make_float2(y2 * cs.x + y1 * cs.y, z2 * cs.z + z1 * cs.w);
+                }
+                if (live) {
+                    store_pairs(p, row0 + h0 + 16 * c, a);
+                    store_pairs(p, row0 + h0 + half + 16 * c, b);
                 }
             }
         }
@@ -151,38 +191,44 @@ __device__ __forceinline__ void proj_store_row(const ProjArgs& p, uint32_t ta, i
     }
 }
 
-template <int BN, int MT>
+template <int BN>
 __global__ void __launch_bounds__(kProjThreads, 1)
     proj_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                 const __grid_constant__ ProjArgs p)
 {
-    using L = ProjLayout<BN, MT>;
+    using L = ProjLayout<BN>;
     constexpr int S = L::STAGES;
-    static_assert(S >= 3, "ring depth");
+    static_assert(L::ALLOC > 116 * 1024 && L::ALLOC <= 227 * 1024, "one CTA per SM");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // N tiles run fastest: the CTAs in flight share their A rows (read from DRAM
-    // once, then from L2), and W' (all N tiles) stays in L2
-    const int64_t m0 = (int64_t)blockIdx.y * (128 * MT);
-    const int n0 = (int)blockIdx.x * BN;
+    const int rank = (int)cluster_ctarank();
+    const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
     const int nk = (p.hidden + kProjK - 1) / kProjK;
+    const int ntn = p.out_features / BN;
+    const int ntiles = (int)((p.rows + 2 * kProjRows - 1) / (2 * kProjRows)) * ntn;
 
     const uint32_t bar0 = base + L::OFF_BAR;
     auto FULL = [&](int s) -> uint32_t { return bar0 + 8u * (uint32_t)s; };
     auto EMPTY = [&](int s) -> uint32_t { return bar0 + 8u * (uint32_t)(S + s); };
-    const uint32_t ACC = bar0 + 8u * (uint32_t)(2 * S);
+    auto ACC_FULL = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(2 * S + b); };
+    auto ACC_EMPTY = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(2 * S + 2 + b); };
+    const uint32_t DRAIN = bar0 + 8u * (uint32_t)(2 * S + 4);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 4);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(FULL(s), 1);
-            mbar_init(EMPTY(s), 1 + 4 * MT);  // the MMA commit and the row-sum warps
+            mbar_init(FULL(s), 1);   // first CTA: its arming arrival; both CTAs' copies complete bytes on it
+            mbar_init(EMPTY(s), 1);  // the commit, in both CTAs
         }
-        mbar_init(ACC, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(ACC_FULL(b), 1);
+            mbar_init(ACC_EMPTY(b), 16);  // first CTA: the epilogue warps of both
+        }
+        mbar_init(DRAIN, 1);
         *abort_flag = 0;
         fence_mbar_init_cluster();
     }
@@ -191,122 +237,164 @@ __global__ void __launch_bounds__(kProjThreads, 1)
         tma_prefetch_desc(&tm_w);
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), L::TMEM_COLS);
-        tmem_relinquish();
+        tmem_alloc_pair(smem_u32(tmem_slot), L::TMEM_COLS);
+        tmem_relinquish_pair();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    cluster_sync_all();  // both CTAs' barriers and TMEM exist
     const uint32_t tmem = *tmem_slot;
     const Ctl ctl{abort_flag, p.err, p.wait_budget};
-    griddep_wait();
+    volatile int no_abort = 0;
+    const Ctl drain{&no_abort, p.err, kWaitBudgetCycles};
+    // x and W' come from kernels that had completed before the row-scale kernel
+    // passed its own wait, so only the readers of the scales wait for that one
     griddep_launch_dependents();
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
-            int issued[S];
-            for (int s = 0; s < S; ++s) issued[s] = 0;
-            for (int kc = 0; kc < nk; ++kc) {
-                const int s = kc % S;
-                const uint32_t ph = (uint32_t)(kc / S) & 1u;
-                if (!wait_phase(EMPTY(s), ph ^ 1u, ctl)) break;
-                mbar_arrive_expect_tx(FULL(s), (uint32_t)(L::A_BYTES + L::B_BYTES));
-                // one box of 128 * MT rows: the second row block lands 16 KB after the first
-                tma_load_3d(base + L::OFF_A + s * L::A_BYTES, &tm_x, FULL(s), kc * kProjK, 0, (int32_t)m0);
-                tma_load_3d(base + L::OFF_B + s * L::B_BYTES, &tm_w, FULL(s), kc * kProjK, 0, n0);
-                ++issued[s];
+            int it = 0;
+            bool ok = true;
+            for (int t = pair; t < ntiles && ok; t += npairs) {
+                const int m0 = t / ntn * (2 * kProjRows) + rank * kProjRows;
+                const int n0 = t % ntn * BN + rank * (BN / 2);
+                for (int kc = 0; kc < nk; ++kc, ++it) {
+                    const int s = it % S;
+                    if (!wait_phase(EMPTY(s), ((uint32_t)(it / S) & 1u) ^ 1u, ctl)) { ok = false; break; }
+                    const uint32_t full = mapa_shared(FULL(s), 0);
+                    if (rank == 0) mbar_arrive_expect_tx(FULL(s), 2u * (uint32_t)L::STAGE);
+                    tma_load_3d_pair(base + L::OFF_A + s * L::A_BYTES, &tm_x, full, kc * kProjK, 0, m0);
+                    tma_load_3d_pair(base + L::OFF_B + s * L::B_BYTES, &tm_w, full, kc * kProjK, 0, n0);
+                }
             }
-            volatile int no_abort = 0;
-            const Ctl drain{&no_abort, p.err, kWaitBudgetCycles};
-            for (int s = 0; s < S; ++s)
-                if (issued[s] > 0) wait_phase(FULL(s), (uint32_t)(issued[s] - 1) & 1u, drain);
+            // every stage's last contraction has completed (and with it its copies)
+            // and its commit has arrived here before this CTA may leave
+            for (int s = 0; s < S && s < it && ok; ++s)
+                ok = wait_phase(EMPTY(s), (uint32_t)((it - 1 - s) / S) & 1u, ctl);
+            if (!ok) {  // after an abort: time enough for the copies in flight to land
+                const long long c0 = clock64();
+                while (clock64() - c0 < 1000000) {}
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_make(128, BN, 1u);
+        // ---------------------------------------------------------------- MMA issuer (first CTA)
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = idesc_make(256, BN, 1u);
+            int it = 0, a = 0;
             bool ok = true;
-            for (int kc = 0; kc < nk && ok; ++kc) {
-                const int s = kc % S;
-                if (!wait_phase(FULL(s), (uint32_t)(kc / S) & 1u, ctl)) { ok = false; break; }
+            for (int t = pair; t < ntiles && ok; t += npairs, ++a) {
+                const uint32_t d = tmem + (uint32_t)((a & 1) * BN);
+                if (!wait_phase_cluster(ACC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl)) break;
                 tc_fence_after();
-                const uint32_t a = base + L::OFF_A + s * L::A_BYTES, b = base + L::OFF_B + s * L::B_BYTES;
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
+                for (int kc = 0; kc < nk; ++kc, ++it) {
+                    const int s = it % S;
+                    if (!wait_phase(FULL(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t ad = sdesc_k_sw128(base + L::OFF_A + s * L::A_BYTES);
+                    const uint64_t bd = sdesc_k_sw128(base + L::OFF_B + s * L::B_BYTES);
 #pragma unroll
                     for (int st = 0; st < 4; ++st)
-                        mma_f16(tmem + (uint32_t)(mt * BN), sdesc_k_sw128(a + mt * 128 * 128 + st * 32),
-                                sdesc_k_sw128(b + st * 32), idesc, (kc | st) != 0);
-                mma_commit(EMPTY(s));
+                        mma_f16_pair(d, ad + (uint64_t)st * 2, bd + (uint64_t)st * 2, idesc, (kc | st) != 0);
+                    mma_commit_pair(EMPTY(s));
+                }
+                if (ok) mma_commit_pair(ACC_FULL(a & 1));
             }
-            mma_commit(ACC);  // every contraction above has landed once this arrives
-            volatile int no_abort = 0;
-            const Ctl drain{&no_abort, p.err, kWaitBudgetCycles};
-            wait_phase(ACC, 0, drain);
+            mma_commit_pair(DRAIN);  // every contraction above has landed once this arrives
+            wait_phase(DRAIN, 0, drain);
         }
         __syncwarp();
     } else {
-        // ---------------------------------------------------------------- row sums + epilogue
-        // MT = 2: warpgroup g owns row block g (its sums and its accumulator).
-        // MT = 1: warpgroup 0 takes the row sums, and the two warpgroups split
-        // the columns (whole heads) of the epilogue.
+        // ---------------------------------------------------------------- epilogue
         const int quad = warp & 3;
         const int wg = (warp - 2) >> 2;
-        const int r = quad * 32 + lane;  // row of the 128-row block = TMEM lane
-        float* sc_s = reinterpret_cast<float*>(smem + L::OFF_SC);
-        const bool sums = MT == 2 || wg == 0;
-        float ss0 = 0.f, ss1 = 0.f;
-        if (sums) {
-            const int mt = MT == 2 ? wg : 0;
-            for (int kc = 0; kc < nk; ++kc) {
-                const int s = kc % S;
-                if (!wait_phase(FULL(s), (uint32_t)(kc / S) & 1u, ctl)) break;
-                const uint8_t* row = smem + L::OFF_A + s * L::A_BYTES + mt * 128 * 128 + r * 128;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(row + ((j ^ (r & 7)) << 4));
-                    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float lo = __uint_as_float(w4[q] << 16), hi = __uint_as_float(w4[q] & 0xFFFF0000u);
-                        ss0 = fmaf(lo, lo, ss0);
-                        ss1 = fmaf(hi, hi, ss1);
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(EMPTY(s));
-            }
-        }
-        float sc = rsqrtf((ss0 + ss1) / (float)p.hidden + p.eps);
-        if (MT == 1) {
-            if (wg == 0) sc_s[r] = sc;
-            named_bar_sync(1, 256);
-            sc = sc_s[r];
-        }
-        const bool ok = wait_phase(ACC, 0, ctl);
-        tc_fence_after();
-        const int mt = MT == 2 ? wg : 0;
-        const int64_t grow = m0 + mt * 128 + r;
+        const int r = quad * 32 + lane;  // row of this CTA's half = TMEM lane
+        const int unit = p.head_dim > 32 ? p.head_dim : 32;
         int c_begin = 0, c_end = BN;
-        if (MT == 1) {
-            const int unit = p.head_dim > 32 ? p.head_dim : 32;
-            if ((BN / 2) % unit == 0) {
-                c_begin = wg * (BN / 2);
-                c_end = c_begin + BN / 2;
-            } else if (wg == 1) {
-                c_end = 0;  // the columns cannot be split by whole heads: warpgroup 0 takes all
-            }
+        if ((BN / 2) % unit == 0) {
+            c_begin = wg * (BN / 2);
+            c_end = c_begin + BN / 2;
+        } else if (wg == 1) {
+            c_end = 0;  // the columns cannot be split by whole heads: warpgroup 0 takes all
         }
-        proj_store_row(p, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(mt * BN), grow, n0, c_begin, c_end,
-                       ok && grow < p.rows, sc);
+        RopeWindow w;
+        w.table = p.rope;
+        w.buf = smem + L::OFF_ROPE + (warp - 2) * 4096;
+        w.half = p.head_dim / 2;
+        w.lane = lane;
+        bool waited = false;
+        int a = 0;
+        for (int t = pair; t < ntiles; t += npairs, ++a) {
+            const int64_t grow = (int64_t)(t / ntn) * (2 * kProjRows) + rank * kProjRows + r;
+            const int n0 = t % ntn * BN;
+            if (p.head_dim > 0 && c_begin < c_end) {
+                // positions and table come from kernels before the row-scale kernel
+                w.pos = grow < p.rows ? p.positions[grow] : 0;
+                if (w.pos < 0 || w.pos >= p.max_positions) {
+                    atomicOr(p.err, kErrBounds);
+                    w.pos = 0;
+                }
+                w.fetch(0);
+            }
+            if (!waited) griddep_wait();  // the row scales
+            waited = true;
+            const float sc = grow < p.rows ? p.scale[grow] : 0.f;
+            const bool ok = wait_phase(ACC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl);
+            tc_fence_after();
+            if (c_begin < c_end)
+                proj_store_row(p, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a & 1) * BN), grow, n0, c_begin,
+                               c_end, ok && grow < p.rows, sc, w);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(mapa_shared(ACC_EMPTY(a & 1), 0));
+            if (!ok) break;
+        }
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();  // both CTAs are done with each other's barriers and contractions
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, L::TMEM_COLS);
+        tmem_dealloc_pair(tmem, L::TMEM_COLS);
+    }
+    griddep_wait();  // returns at once for threads that already waited
+}
+
+// scale[r] = 1 / sqrt(mean x_r^2 + eps), one warp per row; x rows are 16-byte
+// aligned (hidden a multiple of 8)
+constexpr int kScaleThreads = 384;
+
+__global__ void __launch_bounds__(kScaleThreads) row_scale_kernel(const uint4* __restrict__ x, float* __restrict__ scale,
+                                                                  int64_t rows, int hidden, float eps)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    const int lane = threadIdx.x & 31, n16 = hidden / 8;
+    const int64_t nw = (int64_t)gridDim.x * (kScaleThreads / 32);
+    for (int64_t r = (int64_t)blockIdx.x * (kScaleThreads / 32) + (threadIdx.x >> 5); r < rows; r += nw) {
+        const uint4* row = x + r * n16;
+        float ss0 = 0.f, ss1 = 0.f;
+        for (int c = lane; c < n16; c += 128) {  // up to four vectors per lane in flight
+            uint4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = c + 32 * u < n16 ? row[c + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t w4[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float lo = __uint_as_float(w4[q] << 16), hi = __uint_as_float(w4[q] & 0xFFFF0000u);
+                    ss0 = fmaf(lo, lo, ss0);
+                    ss1 = fmaf(hi, hi, ss1);
+                }
+            }
+        }
+        float ss = ss0 + ss1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        if (lane == 0) scale[r] = rsqrtf(ss / (float)hidden + eps);
     }
 }
 
@@ -349,22 +437,29 @@ cudaError_t launch_plain(void (*kern)(Args...), unsigned grid, unsigned block, s
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <int BN, int MT>
-cudaError_t launch_proj_variant(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p,
+template <int BN>
+cudaError_t launch_proj_variant(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, int num_sms,
                                 cudaStream_t stream)
 {
-    using L = ProjLayout<BN, MT>;
-    auto kern = proj_kernel<BN, MT>;
+    using L = ProjLayout<BN>;
+    auto kern = proj_kernel<BN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::ALLOC);
     if (e != cudaSuccess) return e;
+    const int64_t ntiles = (p.rows + 2 * kProjRows - 1) / (2 * kProjRows) * (p.out_features / BN);
+    const int64_t pairs = ntiles < num_sms / 2 ? ntiles : num_sms / 2;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.out_features / BN), (unsigned)((p.rows + 128 * MT - 1) / (128 * MT)), 1);
+    cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
     cfg.blockDim = dim3(kProjThreads, 1, 1);
     cfg.dynamicSmemBytes = L::ALLOC;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, tm_x, tm_w, p);
 }
 
@@ -372,23 +467,19 @@ cudaError_t launch_proj_variant(const CUtensorMap& tm_x, const CUtensorMap& tm_w
 
 int proj_tile_cols(int out_features) { return out_features % 256 == 0 ? 256 : 128; }
 
-// 256-row tiles when they still give every SM two tiles, else 128-row tiles
-int proj_tile_rows(int64_t rows, int out_features, int num_sms)
-{
-    const int64_t n_tiles = out_features / proj_tile_cols(out_features);
-    return ((rows + 255) / 256) * n_tiles >= 2LL * num_sms ? 256 : 128;
-}
-
-cudaError_t launch_proj(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, int tile_rows,
-                        cudaStream_t stream)
+cudaError_t launch_proj(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, const void* x,
+                        int num_sms, cudaStream_t stream)
 {
     if (p.rows <= 0) return cudaSuccess;
-    const bool wide = proj_tile_cols(p.out_features) == 256;
-    if (tile_rows == 256)
-        return wide ? launch_proj_variant<256, 2>(tm_x, tm_w, p, stream)
-                    : launch_proj_variant<128, 2>(tm_x, tm_w, p, stream);
-    return wide ? launch_proj_variant<256, 1>(tm_x, tm_w, p, stream)
-                : launch_proj_variant<128, 1>(tm_x, tm_w, p, stream);
+    // one CTA per SM at most, with registers left for a CTA of the contraction
+    // kernel beside it: all start at once, and that kernel starts with them
+    const int64_t want = (p.rows + kScaleThreads / 32 - 1) / (kScaleThreads / 32);
+    const unsigned grid = (unsigned)(want < num_sms ? want : num_sms);
+    cudaError_t e = launch_plain(row_scale_kernel, grid, kScaleThreads, 0, stream, static_cast<const uint4*>(x),
+                                 p.scale, p.rows, (int)p.hidden, p.eps);
+    if (e != cudaSuccess) return e;
+    return proj_tile_cols(p.out_features) == 256 ? launch_proj_variant<256>(tm_x, tm_w, p, num_sms, stream)
+                                                 : launch_proj_variant<128>(tm_x, tm_w, p, num_sms, stream);
 }
 
 cudaError_t launch_fold_norm(const __nv_bfloat16* w, const float* gamma, __nv_bfloat16* out, int64_t total,
