@@ -3,7 +3,8 @@
 sm_103a only (`-gencode arch=compute_103a,code=sm_103a`), translation units
 compiled in parallel, static CUDA runtime, no link against libcuda (the driver
 entry point for TMA descriptors is looked up at run time), so the library
-loads on a machine without a GPU driver.
+loads on a machine without a GPU driver. The Python binding's marshalling is a
+small CPython extension beside it (gcc).
 """
 from __future__ import annotations
 
@@ -11,6 +12,7 @@ import concurrent.futures as cf
 import os
 import shutil
 import subprocess
+import sysconfig
 from typing import List, Optional
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -23,6 +25,7 @@ LIB = os.path.join(PKG, "liblitevlm_select.so")
 OBJ_DEBUG = os.path.join(PKG, "_build_debug")
 LIB_DEBUG = os.path.join(PKG, "liblitevlm_select_debug.so")
 SOURCES = ["api.cu", "score_tc.cu", "score_res.cu", "ctx_stats.cu", "topk.cu", "compact.cu", "splice.cu", "views.cu", "proj.cu"]
+FASTCALL = os.path.join(PKG, "_fastcall.so")  # argument marshalling of the binding (CPython extension)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -45,6 +48,18 @@ def _compile(src: str, extra: List[str], objdir: str = OBJ) -> str:
     return obj
 
 
+def _build_fastcall() -> None:
+    tmp = FASTCALL + f".tmp{os.getpid()}"
+    cmd = [shutil.which("gcc") or "cc", "-O2", "-std=c11", "-Wall", "-Wextra", "-shared", "-fPIC",
+           "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "fastcall.c"), "-o", tmp]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"gcc failed on fastcall.c:\n{r.stdout}\n{r.stderr}")
+    if r.stderr.strip():
+        print(r.stderr.strip())
+    os.replace(tmp, FASTCALL)
+
+
 def build(verbose_ptxas: bool = False, extra_flags: Optional[List[str]] = None, debug: bool = False) -> str:
     """Builds the library (or, with debug=True, the debug variant) and returns
     its path. LITEVLM_NVTX=1 in the environment adds the NVTX ranges to the
@@ -58,8 +73,10 @@ def build(verbose_ptxas: bool = False, extra_flags: Optional[List[str]] = None, 
         extra += ["-DLITEVLM_DEBUG", "-DLITEVLM_NVTX"]
     elif os.environ.get("LITEVLM_NVTX") == "1":
         extra += ["-DLITEVLM_NVTX"]
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        fast = ex.submit(_build_fastcall)
         objs = list(ex.map(lambda s: _compile(s, extra, objdir), SOURCES))
+        fast.result()
     tmp = lib + f".tmp{os.getpid()}"
     cmd = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs, "-ldl"]
     r = subprocess.run(cmd, capture_output=True, text=True)

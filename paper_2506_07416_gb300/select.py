@@ -2,7 +2,9 @@
 
 Argument marshalling only: torch tensors give device pointers and the current
 CUDA stream; every step of the path runs in liblitevlm_select.so. There is no
-CPU fallback: if the library is missing the import of this module fails.
+CPU fallback: if the library is missing the import of this module fails. The hot
+calls convert their arguments in a small CPython extension (_fastcall.so, built
+with the library); the others go through ctypes.
 
 Names follow the C functions: create / destroy / score / topk / compact /
 check_device (litevlm_select_*), plus ``Selector``, a small object that owns
@@ -130,10 +132,26 @@ def _host_i32(a) -> Optional[np.ndarray]:
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():  # (the raw stream: torch.cuda.current_stream() takes 3 to 6 us)
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+def _load_fastcall():
+    try:
+        from . import _fastcall
+    except ImportError as e:
+        raise ImportError(f"_fastcall.so is not built; run __graft_entry__.build() ({e})") from e
+    _fastcall.bind({n: ctypes.cast(getattr(LIB, "litevlm_select_" + n), ctypes.c_void_p).value
+                    for n in ("score", "score_full_keys", "score_topk", "topk", "compact", "splice", "project",
+                              "keep_offsets")}, _host_i32)
+    return _fastcall
+
+
+_FC = _load_fastcall()
 
 
 # ----------------------------------------------------------------------------
@@ -163,20 +181,20 @@ def destroy(handle: int) -> None:
 
 def score(handle: int, batch: int, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d, seq_offsets_h,
           q_scale: float, k_scale: float, scores, stream=None) -> None:
-    to_h, so_h = _host_i32(text_offsets_h), _host_i32(seq_offsets_h)
-    _check(LIB.litevlm_select_score(handle, batch, _ptr(q_text), _ptr(text_offsets_d), _ptr(to_h), _ptr(k_vis),
-                                    _ptr(seq_offsets_d), _ptr(so_h), q_scale, k_scale, _ptr(scores),
-                                    _stream_ptr(stream)), handle)
+    rc = _FC.score(handle, batch, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d, seq_offsets_h,
+                   q_scale, k_scale, scores, _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def score_full_keys(handle: int, batch: int, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d,
                     seq_offsets_h, k_sys, sys_offsets_d, sys_offsets_h, k_text, q_scale: float, k_scale: float,
                     scores, stream=None) -> None:
-    to_h, so_h, yo_h = _host_i32(text_offsets_h), _host_i32(seq_offsets_h), _host_i32(sys_offsets_h)
-    _check(LIB.litevlm_select_score_full_keys(handle, batch, _ptr(q_text), _ptr(text_offsets_d), _ptr(to_h),
-                                              _ptr(k_vis), _ptr(seq_offsets_d), _ptr(so_h), _ptr(k_sys),
-                                              _ptr(sys_offsets_d), _ptr(yo_h), _ptr(k_text), q_scale, k_scale,
-                                              _ptr(scores), _stream_ptr(stream)), handle)
+    rc = _FC.score_full_keys(handle, batch, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d,
+                             seq_offsets_h, k_sys, sys_offsets_d, sys_offsets_h, k_text, q_scale, k_scale, scores,
+                             _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def views(handle: int, batch: int, num_views: int, lexical, logits, tokens_per_view_h, w_lex: float, w_logit: float,
@@ -191,11 +209,11 @@ def views(handle: int, batch: int, num_views: int, lexical, logits, tokens_per_v
 def score_topk(handle: int, batch: int, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d, seq_offsets_h,
                q_scale: float, k_scale: float, scores, keep_k_d, keep_k_h, keep_ratio: float, kept_idx,
                out_offsets_d, out_offsets_h, stream=None) -> None:
-    to_h, so_h, kk_h = _host_i32(text_offsets_h), _host_i32(seq_offsets_h), _host_i32(keep_k_h)
-    _check(LIB.litevlm_select_score_topk(handle, batch, _ptr(q_text), _ptr(text_offsets_d), _ptr(to_h),
-                                         _ptr(k_vis), _ptr(seq_offsets_d), _ptr(so_h), q_scale, k_scale,
-                                         _ptr(scores), _ptr(keep_k_d), _ptr(kk_h), keep_ratio, _ptr(kept_idx),
-                                         _ptr(out_offsets_d), _ptr(out_offsets_h), _stream_ptr(stream)), handle)
+    rc = _FC.score_topk(handle, batch, q_text, text_offsets_d, text_offsets_h, k_vis, seq_offsets_d, seq_offsets_h,
+                        q_scale, k_scale, scores, keep_k_d, keep_k_h, keep_ratio, kept_idx, out_offsets_d,
+                        out_offsets_h, _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def fold_norm(handle: int, out_features: int, hidden: int, w, gamma, w_folded, stream=None) -> None:
@@ -210,38 +228,44 @@ def rope_table(handle: int, max_positions: int, head_dim: int, rope_base: float,
 
 def project(handle: int, rows: int, hidden: int, out_features: int, x, w_folded, bias, eps: float, head_dim: int,
             positions, table, max_positions: int, y, stream=None, out_scale: float = 0.0) -> None:
-    _check(LIB.litevlm_select_project(handle, rows, hidden, out_features, _ptr(x), _ptr(w_folded), _ptr(bias), eps,
-                                      head_dim, _ptr(positions), _ptr(table), max_positions, out_scale, _ptr(y),
-                                      _stream_ptr(stream)), handle)
+    rc = _FC.project(handle, rows, hidden, out_features, x, w_folded, bias, eps, head_dim, positions, table,
+                     max_positions, out_scale, y, _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def topk(handle: int, batch: int, scores, seq_offsets_d, seq_offsets_h, keep_k_d, keep_k_h, keep_ratio: float,
          kept_idx, out_offsets_d, out_offsets_h: Optional[np.ndarray] = None, stream=None) -> None:
-    so_h, kk_h = _host_i32(seq_offsets_h), _host_i32(keep_k_h)
-    _check(LIB.litevlm_select_topk(handle, batch, _ptr(scores), _ptr(seq_offsets_d), _ptr(so_h), _ptr(keep_k_d),
-                                   _ptr(kk_h), keep_ratio, _ptr(kept_idx), _ptr(out_offsets_d),
-                                   _ptr(out_offsets_h), _stream_ptr(stream)), handle)
+    rc = _FC.topk(handle, batch, scores, seq_offsets_d, seq_offsets_h, keep_k_d, keep_k_h, keep_ratio, kept_idx,
+                  out_offsets_d, out_offsets_h, _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def compact(handle: int, total_kept: int, kept_idx, src_rows: int, srcs: Sequence, dsts: Sequence,
             row_bytes: Sequence[int], stream=None) -> None:
     n = len(srcs)
-    src_arr = (ctypes.c_void_p * n)(*[_ptr(s) for s in srcs])
-    dst_arr = (ctypes.c_void_p * n)(*[_ptr(d) for d in dsts])
-    rb_arr = (ctypes.c_int64 * n)(*[int(r) for r in row_bytes])
-    _check(LIB.litevlm_select_compact(handle, total_kept, _ptr(kept_idx), src_rows, n, src_arr, dst_arr, rb_arr,
-                                      _stream_ptr(stream)), handle)
+    if 1 <= n <= 8:
+        rc = _FC.compact(handle, total_kept, kept_idx, src_rows, list(srcs), list(dsts), [int(r) for r in row_bytes],
+                         _stream_ptr(stream))
+    else:  # an error of the C call's
+        src_arr = (ctypes.c_void_p * n)(*[_ptr(s) for s in srcs])
+        dst_arr = (ctypes.c_void_p * n)(*[_ptr(d) for d in dsts])
+        rb_arr = (ctypes.c_int64 * n)(*[int(r) for r in row_bytes])
+        rc = LIB.litevlm_select_compact(handle, total_kept, _ptr(kept_idx), src_rows, n, src_arr, dst_arr, rb_arr,
+                                        _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def splice(handle: int, batch: int, sys_rows, sys_offsets_d, sys_offsets_h, vis_rows, seq_offsets_d, seq_offsets_h,
            kept_idx, kept_offsets_d, kept_offsets_h, txt_rows, text_offsets_d, text_offsets_h, row_bytes: int,
            out_rows, out_offsets_d, position_ids, out_offsets_h: Optional[np.ndarray] = None, stream=None) -> None:
-    so, vo, ko, to = (_host_i32(a) for a in (sys_offsets_h, seq_offsets_h, kept_offsets_h, text_offsets_h))
-    _check(LIB.litevlm_select_splice(handle, batch, _ptr(sys_rows), _ptr(sys_offsets_d), _ptr(so), _ptr(vis_rows),
-                                     _ptr(seq_offsets_d), _ptr(vo), _ptr(kept_idx), _ptr(kept_offsets_d), _ptr(ko),
-                                     _ptr(txt_rows), _ptr(text_offsets_d), _ptr(to), int(row_bytes), _ptr(out_rows),
-                                     _ptr(out_offsets_d), _ptr(out_offsets_h), _ptr(position_ids),
-                                     _stream_ptr(stream)), handle)
+    rc = _FC.splice(handle, batch, sys_rows, sys_offsets_d, sys_offsets_h, vis_rows, seq_offsets_d, seq_offsets_h,
+                    kept_idx, kept_offsets_d, kept_offsets_h, txt_rows, text_offsets_d, text_offsets_h,
+                    int(row_bytes), out_rows, out_offsets_d, out_offsets_h, position_ids, _stream_ptr(stream))
+    if rc:
+        _check(rc, handle)
 
 
 def host_view(handle: int, host_ptr: int) -> int:
@@ -262,6 +286,14 @@ def keep_offsets(seq_offsets_h, keep_k_h=None, keep_ratio: float = 0.0) -> np.nd
     out = np.zeros(len(so), np.int32)
     _check(LIB.litevlm_select_keep_offsets(len(so) - 1, _ptr(so), _ptr(kk), keep_ratio, _ptr(out)), None)
     return out
+
+
+def _keep_total(seq_offsets_h, keep_k_h, keep_ratio: float) -> int:
+    """Kept tokens of a batch (the last of keep_offsets)."""
+    total = _FC.keep_total(seq_offsets_h, keep_k_h, keep_ratio)
+    if total < 0:
+        _check(-total, None)
+    return total
 
 
 def set_wait_budget(handle: int, cycles: int) -> None:
@@ -378,15 +410,17 @@ class Selector:
         if kk_h is not None:
             kk_d = keep_k if isinstance(keep_k, torch.Tensor) and keep_k.is_cuda else \
                 torch.from_numpy(kk_h).to(k.device)
-        total = int(keep_offsets(so_h, kk_h, keep_ratio)[-1])
-        scores = out if out is not None else torch.empty(max(1, int(so_h[-1])), dtype=torch.float32, device=k.device)
-        kept = kept_idx if kept_idx is not None else torch.empty(max(total, 1), dtype=torch.int32, device=k.device)
-        off_d = out_offsets if out_offsets is not None else torch.empty(batch + 1, dtype=torch.int32, device=k.device)
+        total, n, dev = _keep_total(so_h, kk_h, keep_ratio), int(so_h[-1]), k.device
+        scores = out if out is not None else torch.empty(max(1, n), dtype=torch.float32, device=dev)
+        kept = kept_idx if kept_idx is not None else torch.empty(max(total, 1), dtype=torch.int32, device=dev)
+        off_d = out_offsets if out_offsets is not None else torch.empty(batch + 1, dtype=torch.int32, device=dev)
         off_h = np.zeros(batch + 1, np.int32)
         score_topk(self.handle, batch, q, text_offsets, to_h, k, seq_offsets, so_h, q_scale, k_scale, scores, kk_d,
                    kk_h, keep_ratio, kept, off_d, off_h, stream)
         self._keep_alive = kk_d
-        return scores[:int(so_h[-1])], kept[:int(off_h[-1])], off_d, off_h
+        # (a buffer made here already has its length, unless that is 0)
+        return (scores if out is None and n else scores[:n], kept if kept_idx is None and total else kept[:total],
+                off_d, off_h)
 
     def fold_norm(self, w, gamma, stream=None):
         """bf16 W * gamma (per input column) for project()."""
@@ -427,7 +461,8 @@ class Selector:
             kk_d = keep_k if isinstance(keep_k, torch.Tensor) and keep_k.is_cuda else \
                 torch.from_numpy(kk_h).to(scores.device)
         off_h = np.zeros(batch + 1, dtype=np.int32)
-        total = int(keep_offsets(so_h, kk_h, keep_ratio)[-1])
+        total = _keep_total(so_h, kk_h, keep_ratio)
+        made = kept_idx is None and total > 0
         if kept_idx is None:
             kept_idx = torch.empty(max(total, 1), dtype=torch.int32, device=scores.device)
         if out_offsets is None:
@@ -435,7 +470,7 @@ class Selector:
         topk(self.handle, batch, scores, seq_offsets, so_h, kk_d, kk_h, keep_ratio, kept_idx, out_offsets, off_h,
              stream)
         self._keep_alive = kk_d
-        return kept_idx[:int(off_h[-1])], out_offsets, off_h
+        return kept_idx if made else kept_idx[:total], out_offsets, off_h
 
     def compact(self, kept_idx, total_kept: int, srcs: Sequence, dsts: Optional[List] = None, stream=None):
         """Gathers the kept rows of each source into the device. A source in
@@ -444,10 +479,10 @@ class Selector:
         import torch
         rows = [s.shape[0] for s in srcs]
         if dsts is None:
-            dsts = [torch.empty((max(total_kept, 0),) + tuple(s.shape[1:]), dtype=s.dtype, device=kept_idx.device)
-                    for s in srcs]
-        rb = [s[0].numel() * s.element_size() if s.shape[0] else 1 for s in srcs]
-        src_ptrs = [self.host_view(s) if s.device.type == "cpu" else s for s in srcs]
+            dev, n = kept_idx.device, max(total_kept, 0)
+            dsts = [torch.empty((n, *s.shape[1:]), dtype=s.dtype, device=dev) for s in srcs]
+        rb = [s.nbytes // r if r else 1 for s, r in zip(srcs, rows)]
+        src_ptrs = [s if s.is_cuda else self.host_view(s) for s in srcs]
         compact(self.handle, total_kept, kept_idx, min(rows) if rows else 0, src_ptrs, dsts, rb, stream)
         return dsts
 
