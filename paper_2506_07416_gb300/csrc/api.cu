@@ -30,7 +30,6 @@ struct litevlm_select {
     size_t n_counters = 0;
     int32_t* err_d = nullptr;   // device error word (bits lvs::kErr*)
     float* ctx_stats = nullptr; // [max_total_text][Hq]: normaliser terms of system + causal text keys
-    float* row_scale = nullptr; // [kProjChunkRows]: RMSNorm scales of a projection's rows (behind the tickets)
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     int res_capacity[2][17];  // resident score kernel: CTAs at once per cluster size, by pass-1 rows (64/128); -1 unknown
     int tc_capacity[2][17];   // the same for the re-read score kernel
@@ -442,12 +441,8 @@ litevlm_status_t litevlm_select_create(const litevlm_select_config_t* c, litevlm
         e = cudaMalloc(&h->partials, sizeof(float) * (size_t)c->num_q_heads * (size_t)c->max_total_visual);
     // one fold ticket per 128-token tile: index floor(n0 / 128) + t + b < total / 128 + 2 * batch + 1
     h->n_counters = (size_t)(c->max_total_visual / lvs::kTileRows) + 2 * (size_t)c->max_batch + 2;
-    // (the row scales share the allocation, which stays below the 1 MB from which on
-    // cudaMalloc maps a block of its own, 0.13 ms)
-    const size_t ticket_bytes = (sizeof(int32_t) * h->n_counters + 255) & ~(size_t)255;
-    if (e == cudaSuccess) e = cudaMalloc(&h->counters, ticket_bytes + sizeof(float) * (size_t)lvs::kProjChunkRows);
+    if (e == cudaSuccess) e = cudaMalloc(&h->counters, sizeof(int32_t) * h->n_counters);
     if (e == cudaSuccess) e = cudaMemset(h->counters, 0, sizeof(int32_t) * h->n_counters);
-    if (e == cudaSuccess) h->row_scale = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(h->counters) + ticket_bytes);
     if (e == cudaSuccess)
         e = cudaMalloc(&h->ctx_stats, sizeof(float) * (size_t)c->num_q_heads * (size_t)c->max_total_text);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -1100,32 +1095,28 @@ litevlm_status_t litevlm_select_project(litevlm_select_t h, int64_t rows, int32_
         return fail(h, LITEVLM_ERR_INVALID_ARG, "positions, rope_table and max_positions are required with RoPE");
     const int bn = lvs::proj_tile_cols(out_features);
     CUtensorMap tm_x, tm_w;
-    litevlm_status_t s = encode_rows_map(h, &tm_w, w_folded, hidden, 1, out_features, bn / 2, false, "w_folded");
+    litevlm_status_t s = encode_rows_map(h, &tm_x, x, hidden, 1, rows, 128, false, "x");
+    if (s != LITEVLM_OK) return s;
+    s = encode_rows_map(h, &tm_w, w_folded, hidden, 1, out_features, bn / 2, false, "w_folded");
     if (s != LITEVLM_OK) return s;
     lvs::ProjArgs p{};
+    p.rows = rows;
     p.hidden = hidden;
     p.out_features = out_features;
     p.head_dim = head_dim;
     p.max_positions = max_positions;
     p.eps = eps;
-    p.scale = h->row_scale;
     p.bias = bias;
+    p.positions = positions;
     p.rope = reinterpret_cast<const float2*>(rope_table);
+    p.y = out_scale > 0.f ? nullptr : static_cast<__nv_bfloat16*>(y);
+    p.y8 = out_scale > 0.f ? static_cast<uint8_t*>(y) : nullptr;
     p.out_inv_scale = out_scale > 0.f ? 1.f / out_scale : 0.f;
     p.err = h->err_d;
     p.wait_budget = h->wait_budget;
-    for (int64_t r0 = 0; r0 < rows; r0 += lvs::kProjChunkRows) {
-        p.rows = rows - r0 < lvs::kProjChunkRows ? rows - r0 : lvs::kProjChunkRows;
-        const uint8_t* xr = static_cast<const uint8_t*>(x) + r0 * hidden * 2;
-        s = encode_rows_map(h, &tm_x, xr, hidden, 1, p.rows, 128, false, "x");
-        if (s != LITEVLM_OK) return s;
-        p.positions = head_dim > 0 ? positions + r0 : nullptr;
-        p.y = out_scale > 0.f ? nullptr : static_cast<__nv_bfloat16*>(y) + r0 * out_features;
-        p.y8 = out_scale > 0.f ? static_cast<uint8_t*>(y) + r0 * out_features : nullptr;
-        const cudaError_t e = lvs::launch_proj(tm_x, tm_w, p, xr, h->num_sms, (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(h, e, "project launch");
-        h->last_launches += 2;
-    }
+    const cudaError_t e = lvs::launch_proj(tm_x, tm_w, p, h->num_sms, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "project launch");
+    h->last_launches = 1;
     return LITEVLM_OK;
 }
 

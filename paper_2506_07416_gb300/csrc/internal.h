@@ -102,7 +102,6 @@ struct ProjArgs {
     int64_t rows;
     int32_t hidden, out_features, head_dim, max_positions;
     float eps;
-    float* scale;             // [rows] row scales (workspace)
     const float* bias;        // [O] or null
     const int32_t* positions; // [rows] (head_dim > 0)
     const float2* rope;       // [max_positions][head_dim / 2] (cos, sin)
@@ -118,10 +117,8 @@ struct RopeArgs {
     float inv_freq[128];      // rope_base^(-2j / head_dim), rounded to fp32
 };
 int proj_tile_cols(int out_features);
-constexpr int64_t kProjChunkRows = int64_t(1) << 16;  // rows per launch (row scales kept in the handle's workspace)
-// x [rows, hidden]: the row scales, then the contraction
-cudaError_t launch_proj(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, const void* x,
-                        int num_sms, cudaStream_t stream);
+cudaError_t launch_proj(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, int num_sms,
+                        cudaStream_t stream);
 cudaError_t launch_fold_norm(const __nv_bfloat16* w, const float* gamma, __nv_bfloat16* out, int64_t total,
                              int hidden, int num_sms, cudaStream_t stream);
 cudaError_t launch_rope_table(const RopeArgs& a, int num_sms, cudaStream_t stream);

@@ -7,30 +7,29 @@
 // cos / sin from a table indexed by the row's position.
 //
 // The RMSNorm weight is folded into W once (fold kernel below), so the
-// contraction reads the raw hidden rows, and the per-row scale s_r is applied in
-// the epilogue with the bias and the rotation.
+// contraction reads the raw hidden rows; the per-row scale s_r is a sum of
+// squares taken from the A tiles while they sit in shared memory for the tensor
+// core, and is applied in the epilogue with the bias and the rotation.
 //
-// Row scales: a small kernel launched just before (one warp per row). The
-// contraction kernel starts under it (programmatic dependent launch) and only its
-// epilogue waits for it, so the second read of x overlaps the first tiles. Summing
-// the squares from the A tiles in shared memory instead, as this kernel used to,
-// took a quarter of the shared-memory bandwidth that the contraction needs.
-//
-// Contraction: pairs of CTAs (clusters of two, cta_group::2) work through output
-// tiles of 256 rows x BN columns (BN = 256, or 128 where the columns leave no
-// choice), N tiles fastest, so that the tiles in flight share their rows of x and
-// W' stays in L2. Each CTA stages its 128 rows of x and half of the tile's rows of
-// W' (64 hidden values a stage); one thread of the first CTA issues the
-// tcgen05.mma (M = 256, N = BN, K = 16) for both. A CTA's operands then take
-// 64 bytes a clock out of shared memory and 64 in, its limit of 128; one CTA alone
-// on 128 x 256 needs 96 and 96. Accumulators alternate between two TMEM buffers:
-// the epilogue of a tile runs under the contraction of the next. Against one-CTA
-// tiles of 256 x 256 with the sums taken from shared memory: 27648 x 4096 -> 4096
-// 755 -> 625 us (1.48 PFLOP/s), 6157 x 3584 -> 512 34.3 -> 28 us, 1536 x 2048 ->
-// 2048 25.5 -> 20.3 us (48 tiles on 76 pairs, 10 us of it launch, set-up and the
-// single epilogue).
+// Pairs of CTAs (clusters of two, cta_group::2) work through output tiles of 256
+// rows x BN columns (BN = 256, or 128 where the columns leave no choice), N tiles
+// fastest, so that the tiles in flight share their rows of x and W' stays in L2.
+// Each CTA stages its 128 rows of x and half of the tile's rows of W' (64 hidden
+// values a stage); one thread of the first CTA issues the tcgen05.mma (M = 256,
+// N = BN, K = 16) for both, so a CTA's operands take 64 bytes a clock out of shared
+// memory and 64 in (one CTA alone on 128 x 256: 96 and 96; its limit is 128).
+// Accumulators alternate between two TMEM buffers: the epilogue of a tile runs
+// under the contraction of the next.
 //   warp 0: TMA producer; warp 1: TMEM, and in the first CTA the MMA issuer; warps
-//   2-9: epilogue, two warpgroups that split a tile's columns by whole heads.
+//   6-9: row sums, each stage after its contraction and before it is given back;
+//   warps 2-5: epilogue (TMEM lane = row); warps 6-9 take half of a pair's last
+//   tile, after which there is nothing left to sum.
+// Against one-CTA tiles of 256 x 256 with a single accumulator, whose sums shared
+// the tile's stages with the contraction: 27648 x 4096 -> 4096 755 -> 617 us, 6157
+// x 3584 -> 512 (e4m3) 34.3 -> 26.6 us, 1536 x 2048 -> 2048 25.5 -> 19.4 us (48 tiles
+// on 76 pairs: 10 us of it are launch, set-up and the one epilogue). A kernel of
+// its own for the row scales, overlapping the first tiles, was slower on all of
+// them (623, 29 and 21 us): its loads compete with the copies.
 // Every wait is bounded.
 
 #include <math.h>
@@ -58,8 +57,10 @@ struct ProjLayout {
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + STAGES * A_BYTES;
     static constexpr int OFF_ROPE = OFF_B + STAGES * B_BYTES;  // 4 KB per epilogue warp
-    static constexpr int OFF_BAR = OFF_ROPE + 8 * 4096;        // full[S], empty[S], acc_full[2], acc_empty[2], drain
-    static constexpr int OFF_MISC = OFF_BAR + (2 * STAGES + 5) * 8;
+    // full[S], done[S], empty[S], acc_full[2], acc_empty[2], sc_full[2], sc_empty[2], drain
+    static constexpr int OFF_BAR = OFF_ROPE + 8 * 4096;
+    static constexpr int OFF_SC = OFF_BAR + (3 * STAGES + 9) * 8;  // [2][128] row scales
+    static constexpr int OFF_MISC = OFF_SC + 2 * kProjRows * 4;
     static constexpr int ALLOC = OFF_MISC + 16 + 1024;
     static constexpr int TMEM_COLS = 2 * BN;
 };
@@ -139,19 +140,21 @@ struct RopeWindow {
     }
 };
 
-// scale, bias, rotation and store (bf16 or e4m3) of columns [c_begin, c_end) of one
-// accumulator row (this thread's); the range holds whole heads. With a rotation the
-// warp's window holds the pairs of chunk 0 on entry (and may be left at another).
-__device__ __forceinline__ void proj_store_row(const ProjArgs& p, uint32_t ta, int64_t grow, int n0, int c_begin,
-                                               int c_end, bool live, float sc, RopeWindow& w)
+// scale, bias, rotation and store (bf16 or e4m3) of part `part` of `parts` of the BN
+// columns of one accumulator row (this thread's): with a rotation, of every head's
+// chunks of 16 pairs, the warp's window holding the part's first chunk in flight
+// (fetched); without, of the columns.
+template <int BN>
+__device__ __forceinline__ void proj_store_row(const ProjArgs& p, uint32_t ta, int64_t grow, int n0, int part, int parts,
+                                               bool live, float sc, RopeWindow& w)
 {
     const int64_t row0 = grow * (int64_t)p.out_features + n0;  // element index of this tile's first column
     if (p.head_dim > 0) {
-        const int half = p.head_dim / 2, nc = half / 16;
-        for (int c = 0; c < nc; ++c) {
+        const int half = p.head_dim / 2, nc = half / 16 / parts * (part + 1);
+        for (int c = half / 16 / parts * part; c < nc; ++c) {
             w.put();
             if (c + 1 < nc) w.fetch(c + 1);
-            for (int h0 = c_begin; h0 < c_end; h0 += p.head_dim) {
+            for (int h0 = 0; h0 < BN; h0 += p.head_dim) {
                 float v1[16], v2[16];
                 tmem_ld16(ta + (uint32_t)(h0 + 16 * c), v1);
                 tmem_ld16(ta + (uint32_t)(h0 + half + 16 * c), v2);
@@ -175,7 +178,7 @@ __device__ __forceinline__ void proj_store_row(const ProjArgs& p, uint32_t ta, i
             }
         }
     } else {
-        for (int c = c_begin; c < c_end; c += 32) {
+        for (int c = BN / parts * part; c < BN / parts * (part + 1); c += 32) {
             float v[32];
             tmem_ld32(ta + (uint32_t)c, v);
             tmem_wait_ld();
@@ -212,21 +215,28 @@ __global__ void __launch_bounds__(kProjThreads, 1)
 
     const uint32_t bar0 = base + L::OFF_BAR;
     auto FULL = [&](int s) -> uint32_t { return bar0 + 8u * (uint32_t)s; };
-    auto EMPTY = [&](int s) -> uint32_t { return bar0 + 8u * (uint32_t)(S + s); };
-    auto ACC_FULL = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(2 * S + b); };
-    auto ACC_EMPTY = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(2 * S + 2 + b); };
-    const uint32_t DRAIN = bar0 + 8u * (uint32_t)(2 * S + 4);
+    auto DONE = [&](int s) -> uint32_t { return bar0 + 8u * (uint32_t)(S + s); };
+    auto EMPTY = [&](int s) -> uint32_t { return bar0 + 8u * (uint32_t)(2 * S + s); };
+    auto ACC_FULL = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + b); };
+    auto ACC_EMPTY = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + 2 + b); };
+    auto SC_FULL = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + 4 + b); };
+    auto SC_EMPTY = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + 6 + b); };
+    const uint32_t DRAIN = bar0 + 8u * (uint32_t)(3 * S + 8);
+    float* sc_s = reinterpret_cast<float*>(smem + L::OFF_SC);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 4);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(FULL(s), 1);   // first CTA: its arming arrival; both CTAs' copies complete bytes on it
-            mbar_init(EMPTY(s), 1);  // the commit, in both CTAs
+            mbar_init(DONE(s), 1);   // the commit of the stage's contractions, in both CTAs
+            mbar_init(EMPTY(s), 4);  // the summing warps
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(ACC_FULL(b), 1);
-            mbar_init(ACC_EMPTY(b), 16);  // first CTA: the epilogue warps of both
+            mbar_init(ACC_EMPTY(b), 8);  // first CTA: the epilogue warps of both
+            mbar_init(SC_FULL(b), 4);
+            mbar_init(SC_EMPTY(b), 4);
         }
         mbar_init(DRAIN, 1);
         *abort_flag = 0;
@@ -248,8 +258,7 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     const Ctl ctl{abort_flag, p.err, p.wait_budget};
     volatile int no_abort = 0;
     const Ctl drain{&no_abort, p.err, kWaitBudgetCycles};
-    // x and W' come from kernels that had completed before the row-scale kernel
-    // passed its own wait, so only the readers of the scales wait for that one
+    griddep_wait();
     griddep_launch_dependents();
 
     if (warp == 0) {
@@ -269,8 +278,8 @@ __global__ void __launch_bounds__(kProjThreads, 1)
                     tma_load_3d_pair(base + L::OFF_B + s * L::B_BYTES, &tm_w, full, kc * kProjK, 0, n0);
                 }
             }
-            // every stage's last contraction has completed (and with it its copies)
-            // and its commit has arrived here before this CTA may leave
+            // every stage's last contraction has completed (and with it its copies),
+            // its commit has arrived here and its rows are summed before this CTA leaves
             for (int s = 0; s < S && s < it && ok; ++s)
                 ok = wait_phase(EMPTY(s), (uint32_t)((it - 1 - s) / S) & 1u, ctl);
             if (!ok) {  // after an abort: time enough for the copies in flight to land
@@ -298,7 +307,7 @@ __global__ void __launch_bounds__(kProjThreads, 1)
 #pragma unroll
                     for (int st = 0; st < 4; ++st)
                         mma_f16_pair(d, ad + (uint64_t)st * 2, bd + (uint64_t)st * 2, idesc, (kc | st) != 0);
-                    mma_commit_pair(EMPTY(s));
+                    mma_commit_pair(DONE(s));
                 }
                 if (ok) mma_commit_pair(ACC_FULL(a & 1));
             }
@@ -307,49 +316,75 @@ __global__ void __launch_bounds__(kProjThreads, 1)
         }
         __syncwarp();
     } else {
-        // ---------------------------------------------------------------- epilogue
+        // ---------------------------------------------------------------- row sums (wg 1), epilogue
         const int quad = warp & 3;
         const int wg = (warp - 2) >> 2;
         const int r = quad * 32 + lane;  // row of this CTA's half = TMEM lane
-        const int unit = p.head_dim > 32 ? p.head_dim : 32;
-        int c_begin = 0, c_end = BN;
-        if ((BN / 2) % unit == 0) {
-            c_begin = wg * (BN / 2);
-            c_end = c_begin + BN / 2;
-        } else if (wg == 1) {
-            c_end = 0;  // the columns cannot be split by whole heads: warpgroup 0 takes all
-        }
         RopeWindow w;
         w.table = p.rope;
         w.buf = smem + L::OFF_ROPE + (warp - 2) * 4096;
         w.half = p.head_dim / 2;
         w.lane = lane;
-        bool waited = false;
-        int a = 0;
-        for (int t = pair; t < ntiles; t += npairs, ++a) {
+        // part `part` of `parts` of tile t, the a-th of this pair
+        auto store_tile = [&](int t, int a, int part, int parts) -> bool {
             const int64_t grow = (int64_t)(t / ntn) * (2 * kProjRows) + rank * kProjRows + r;
-            const int n0 = t % ntn * BN;
-            if (p.head_dim > 0 && c_begin < c_end) {
-                // positions and table come from kernels before the row-scale kernel
+            if (p.head_dim > 0) {
                 w.pos = grow < p.rows ? p.positions[grow] : 0;
                 if (w.pos < 0 || w.pos >= p.max_positions) {
                     atomicOr(p.err, kErrBounds);
                     w.pos = 0;
                 }
-                w.fetch(0);
+                w.fetch(w.half / 16 / parts * part);
             }
-            if (!waited) griddep_wait();  // the row scales
-            waited = true;
-            const float sc = grow < p.rows ? p.scale[grow] : 0.f;
-            const bool ok = wait_phase(ACC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl);
-            tc_fence_after();
-            if (c_begin < c_end)
-                proj_store_row(p, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a & 1) * BN), grow, n0, c_begin,
-                               c_end, ok && grow < p.rows, sc, w);
-            tc_fence_before();
+            bool ok = wait_phase(SC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl);
+            const float sc = sc_s[(a & 1) * kProjRows + r];
             __syncwarp();
-            if (lane == 0) mbar_arrive_remote(mapa_shared(ACC_EMPTY(a & 1), 0));
-            if (!ok) break;
+            if (wg == 0 && lane == 0) mbar_arrive(SC_EMPTY(a & 1));
+            ok = wait_phase(ACC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl) && ok;
+            tc_fence_after();
+            proj_store_row<BN>(p, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a & 1) * BN), grow, t % ntn * BN,
+                               part, parts, ok && grow < p.rows, sc, w);
+            return ok;
+        };
+        int it = 0, a = 0;
+        bool ok = true;
+        for (int t = pair; t < ntiles && ok; t += npairs, ++a) {
+            const bool last = t + npairs >= ntiles;
+            if (wg == 0) {
+                ok = store_tile(t, a, 0, last ? 2 : 1);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(mapa_shared(ACC_EMPTY(a & 1), 0));
+                continue;
+            }
+            // four packed accumulators: two chains of 32 dependent adds a stage would
+            // take as long as the stage's contraction
+            float2 ss[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ss[q] = make_float2(0.f, 0.f);
+            for (int kc = 0; kc < nk; ++kc, ++it) {
+                const int s = it % S;
+                if (!wait_phase(DONE(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
+                const uint8_t* row = smem + L::OFF_A + s * L::A_BYTES + r * 128;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(row + ((j ^ (r & 7)) << 4));
+                    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 x = make_float2(__uint_as_float(w4[q] << 16), __uint_as_float(w4[q] & 0xFFFF0000u));
+                        ss[q] = ffma2(x, x, ss[q]);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(EMPTY(s));
+            }
+            if (!ok || !wait_phase(SC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl)) break;
+            const float2 s01 = fadd2(ss[0], ss[1]), s23 = fadd2(ss[2], ss[3]);
+            sc_s[(a & 1) * kProjRows + r] = rsqrtf(((s01.x + s01.y) + (s23.x + s23.y)) / (float)p.hidden + p.eps);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(SC_FULL(a & 1));
+            if (last) store_tile(t, a, 1, 2);
         }
     }
     tc_fence_before();
@@ -358,43 +393,6 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem, L::TMEM_COLS);
-    }
-    griddep_wait();  // returns at once for threads that already waited
-}
-
-// scale[r] = 1 / sqrt(mean x_r^2 + eps), one warp per row; x rows are 16-byte
-// aligned (hidden a multiple of 8)
-constexpr int kScaleThreads = 384;
-
-__global__ void __launch_bounds__(kScaleThreads) row_scale_kernel(const uint4* __restrict__ x, float* __restrict__ scale,
-                                                                  int64_t rows, int hidden, float eps)
-{
-    griddep_wait();
-    griddep_launch_dependents();
-    const int lane = threadIdx.x & 31, n16 = hidden / 8;
-    const int64_t nw = (int64_t)gridDim.x * (kScaleThreads / 32);
-    for (int64_t r = (int64_t)blockIdx.x * (kScaleThreads / 32) + (threadIdx.x >> 5); r < rows; r += nw) {
-        const uint4* row = x + r * n16;
-        float ss0 = 0.f, ss1 = 0.f;
-        for (int c = lane; c < n16; c += 128) {  // up to four vectors per lane in flight
-            uint4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = c + 32 * u < n16 ? row[c + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t w4[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float lo = __uint_as_float(w4[q] << 16), hi = __uint_as_float(w4[q] & 0xFFFF0000u);
-                    ss0 = fmaf(lo, lo, ss0);
-                    ss1 = fmaf(hi, hi, ss1);
-                }
-            }
-        }
-        float ss = ss0 + ss1;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) scale[r] = rsqrtf(ss / (float)hidden + eps);
     }
 }
 
@@ -467,17 +465,10 @@ cudaError_t launch_proj_variant(const CUtensorMap& tm_x, const CUtensorMap& tm_w
 
 int proj_tile_cols(int out_features) { return out_features % 256 == 0 ? 256 : 128; }
 
-cudaError_t launch_proj(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, const void* x,
-                        int num_sms, cudaStream_t stream)
+cudaError_t launch_proj(const CUtensorMap& tm_x, const CUtensorMap& tm_w, const ProjArgs& p, int num_sms,
+                        cudaStream_t stream)
 {
     if (p.rows <= 0) return cudaSuccess;
-    // one CTA per SM at most, with registers left for a CTA of the contraction
-    // kernel beside it: all start at once, and that kernel starts with them
-    const int64_t want = (p.rows + kScaleThreads / 32 - 1) / (kScaleThreads / 32);
-    const unsigned grid = (unsigned)(want < num_sms ? want : num_sms);
-    cudaError_t e = launch_plain(row_scale_kernel, grid, kScaleThreads, 0, stream, static_cast<const uint4*>(x),
-                                 p.scale, p.rows, (int)p.hidden, p.eps);
-    if (e != cudaSuccess) return e;
     return proj_tile_cols(p.out_features) == 256 ? launch_proj_variant<256>(tm_x, tm_w, p, num_sms, stream)
                                                  : launch_proj_variant<128>(tm_x, tm_w, p, num_sms, stream);
 }

@@ -68,7 +68,7 @@ def test_project_matches_oracle(sel, rows, hidden, out_f, head_dim, bias):
 
 
 @pytest.mark.parametrize("rows,hidden,out_f,head_dim,bias", [
-    (127, 64, 128, 128, False),      # one 128-column tile: warpgroup 0 takes the whole head; the pair's second half empty
+    (127, 64, 128, 128, False),      # one 128-column tile: one warpgroup takes the whole head; the pair's second half empty
     (129, 8, 256, 64, True),         # the smallest hidden; one row in the pair's second half
     (256, 72, 640, 0, True),         # 128-column tiles, a stage that is almost all padding
     (257, 1000, 512, 128, False),    # a second row tile with one row
@@ -76,27 +76,6 @@ def test_project_matches_oracle(sel, rows, hidden, out_f, head_dim, bias):
 ])
 def test_project_tile_edges(sel, rows, hidden, out_f, head_dim, bias):
     _run(sel, rows, hidden, out_f, head_dim, bias)
-
-
-@pytest.mark.parametrize("rows", [65535, 65536 + 130])
-def test_project_rows_beyond_one_launch(sel, rows):
-    """Rows are projected 65536 at a time; against fp64 torch on the rows around the
-    seam and the ends (the bar of the module's docstring)."""
-    gen = torch.Generator(device="cuda").manual_seed(5)
-    x = torch.randn(rows, 128, generator=gen, device="cuda").to(torch.bfloat16)
-    w = (torch.randn(256, 128, generator=gen, device="cuda") / 11.3).to(torch.bfloat16)
-    pos = torch.randint(0, 512, (rows,), generator=gen, device="cuda", dtype=torch.int32)
-    table = sel.rope_table(512, 64, 1e4)
-    y = sel.project(x, w, None, 1e-6, 64, pos, table)
-    sel.check_device()
-    pick = torch.cat([torch.arange(300), torch.arange(65536 - 200, min(rows, 65536 + 100)),
-                      torch.arange(rows - 300, rows)]).cuda()
-    xd = x[pick].double()
-    z = torch.rsqrt((xd * xd).mean(dim=1, keepdim=True) + 1e-6) * (xd @ w.double().t())
-    z = z.view(-1, 4, 2, 32)
-    c, s = table[pos[pick].long()].double()[:, None].unbind(dim=-1)
-    o = torch.stack([z[:, :, 0] * c - z[:, :, 1] * s, z[:, :, 1] * c + z[:, :, 0] * s], dim=2).reshape(-1, 256)
-    _close(y[pick].double().cpu().numpy(), o.cpu().numpy())
 
 
 def test_project_fold_is_w_times_gamma(sel):
