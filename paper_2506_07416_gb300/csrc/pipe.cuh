@@ -76,6 +76,17 @@ __device__ __forceinline__ bool poll_phase(uint32_t bar, uint32_t parity, const 
     }
 }
 
+// both by a whole warp, which agrees on the result
+__device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, const Ctl& c)
+{
+    return __all_sync(0xffffffffu, wait_phase(bar, parity, c));
+}
+
+__device__ __forceinline__ bool poll_phase_warp(uint32_t bar, uint32_t parity, const Ctl& c)
+{
+    return __all_sync(0xffffffffu, poll_phase(bar, parity, c));
+}
+
 // Online (max, sum 2^(x*c - max*c)) update of one row over NV columns.
 template <int NV>
 __device__ __forceinline__ void row_stats_update(const float* v, int valid, float cl, float& m, float& l)

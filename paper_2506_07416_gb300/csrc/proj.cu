@@ -15,7 +15,7 @@
 // rows x BN columns (BN = 256, or 128 where the columns leave no choice), N tiles
 // fastest, so that the tiles in flight share their rows of x and W' stays in L2.
 // Each CTA stages its 128 rows of x and half of the tile's rows of W' (64 hidden
-// values a stage); one thread of the first CTA issues the tcgen05.mma (M = 256,
+// values a stage); warp 1 of the first CTA issues the tcgen05.mma (M = 256,
 // N = BN, K = 16) for both, so a CTA's operands take 64 bytes a clock out of shared
 // memory and 64 in (one CTA alone on 128 x 256: 96 and 96; its limit is 128).
 // Accumulators alternate between two TMEM buffers: the epilogue of a tile runs
@@ -27,9 +27,11 @@
 // Against one-CTA tiles of 256 x 256 with a single accumulator, whose sums shared
 // the tile's stages with the contraction: 27648 x 4096 -> 4096 755 -> 617 us, 6157
 // x 3584 -> 512 (e4m3) 34.3 -> 26.6 us, 1536 x 2048 -> 2048 25.5 -> 19.4 us (48 tiles
-// on 76 pairs: 10 us of it are launch, set-up and the one epilogue). A kernel of
-// its own for the row scales, overlapping the first tiles, was slower on all of
-// them (623, 29 and 21 us): its loads compete with the copies.
+// on 76 pairs: 10 us of it are launch, set-up and the one epilogue); with the
+// contractions issued from uniform registers (elect_one) 588, 24.9 and 18.5 us. A
+// kernel of its own for the row scales, overlapping the first tiles, was slower on
+// all of them (623, 29 and 21 us against 617, 26.6 and 19.4): its loads compete with
+// the copies.
 // Every wait is bounded.
 
 #include <math.h>
@@ -206,8 +208,8 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = (int)cluster_ctarank();
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+    const int rank = uniform((int)cluster_ctarank());
     const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
     const int nk = (p.hidden + kProjK - 1) / kProjK;
     const int ntn = p.out_features / BN;
@@ -254,7 +256,7 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     __syncthreads();
     tc_fence_after();
     cluster_sync_all();  // both CTAs' barriers and TMEM exist
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     const Ctl ctl{abort_flag, p.err, p.wait_budget};
     volatile int no_abort = 0;
     const Ctl drain{&no_abort, p.err, kWaitBudgetCycles};
@@ -290,29 +292,34 @@ __global__ void __launch_bounds__(kProjThreads, 1)
         __syncwarp();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (first CTA)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc = idesc_make(256, BN, 1u);
             int it = 0, a = 0;
             bool ok = true;
             for (int t = pair; t < ntiles && ok; t += npairs, ++a) {
                 const uint32_t d = tmem + (uint32_t)((a & 1) * BN);
-                if (!wait_phase_cluster(ACC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl)) break;
+                if (!__all_sync(0xffffffffu, wait_phase_cluster(ACC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl))) break;
                 tc_fence_after();
                 for (int kc = 0; kc < nk; ++kc, ++it) {
                     const int s = it % S;
-                    if (!wait_phase(FULL(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
+                    if (!wait_phase_warp(FULL(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t ad = sdesc_k_sw128(base + L::OFF_A + s * L::A_BYTES);
                     const uint64_t bd = sdesc_k_sw128(base + L::OFF_B + s * L::B_BYTES);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int st = 0; st < 4; ++st)
-                        mma_f16_pair(d, ad + (uint64_t)st * 2, bd + (uint64_t)st * 2, idesc, (kc | st) != 0);
-                    mma_commit_pair(DONE(s));
+                        for (int st = 0; st < 4; ++st)
+                            mma_f16_pair(d, ad + (uint64_t)st * 2, bd + (uint64_t)st * 2, idesc, (kc | st) != 0);
+                        mma_commit_pair(DONE(s));
+                    }
+                    __syncwarp();
                 }
-                if (ok) mma_commit_pair(ACC_FULL(a & 1));
+                if (ok && elect_one()) mma_commit_pair(ACC_FULL(a & 1));
+                __syncwarp();
             }
-            mma_commit_pair(DRAIN);  // every contraction above has landed once this arrives
-            wait_phase(DRAIN, 0, drain);
+            if (elect_one()) mma_commit_pair(DRAIN);  // every contraction above has landed once this arrives
+            __syncwarp();
+            wait_phase_warp(DRAIN, 0, drain);
         }
         __syncwarp();
     } else {

@@ -337,6 +337,28 @@ __device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t a_desc, uint64_
         : "memory");
 }
 
+// One thread of the (converged) warp, always the same. Contractions are issued
+// from loops that the whole warp runs, inside `if (elect_one())` and on values
+// the compiler can prove equal over the warp (kernel parameters, loop counters,
+// uniform()): their operands then stay in uniform registers, and an instruction
+// issues at the tensor cores' rate (a 128 x 128 x 128 bf16 unit 516 cycles, e4m3
+// 260). From `if (lane == 0)` on per-thread values each instruction took 157
+// cycles (1255 and 732 a unit), whatever its N.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// lane 0's value, known to be the same over the warp
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 // arrive (once) on an mbarrier when all prior tcgen05 async ops of this thread complete
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {

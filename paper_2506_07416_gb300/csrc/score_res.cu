@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t csize = cluster_nctarank();
     // This cluster's work: one (request, head group), or with a flattened
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
     // is released by fence.mbarrier_init above, and no other write of this CTA
     // is read by a peer.
     cluster_arrive_relaxed();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     const Ctl ctl{abort_flag, p.err, p.wait_budget};
 
     const ResShape shp = res_shape<L::RECV_COLS, L::ACC_TILES, QS>(p, n0, n1, tq, t1, rank, csize, MROWS);
@@ -376,52 +376,55 @@ __global__ void __launch_bounds__(kResThreads, 1)
         cluster_wait();
     } else if (warp <= 2) {
         // ------------------------------------------------------------ MMA issuers
-        // Two issuing threads (lane 0 of warps 1 and 2) take alternate tiles:
-        // issuing a tile (two barrier waits, the contractions, two commits)
-        // costs more time than the tensor core needs to run it, so one thread's
-        // waits and commits overlap the other thread's contractions. Each
-        // thread follows the global tile sequence for the ring's stage and
-        // phase and commits its own contractions. The operand descriptors are
-        // made once (per head for Q, per tile for K) and each K step adds a
-        // constant to the start-address field (shared-memory offsets stay below
-        // 256 KB, so the 14-bit field never carries).
-        if (lane == 0) {
-            const int who = warp - 1;  // 0: even tiles, 1: odd tiles
-            if (mt > 0) {
-                const uint32_t idesc = idesc_make(128, (uint32_t)n2, FMT);
-                // A stage's consecutive loads can belong to different threads
-                // (tiles gt and gt - kStages of opposite parity within their
-                // heads). The K_FULL parity test is only sound once the stage's
-                // previous load has landed, which a thread knows of its own tiles
-                // but not of the other thread's: for those tiles it first waits
-                // for the release of the previous load (its contraction done, so
-                // its data had landed). `cross` marks them by tile.
-                uint32_t cross = 0;
-                for (int tl = who; tl < mt; tl += 2) {
-                    const int ptl = ((tl - kStages) % mt + mt) % mt;
-                    if ((ptl ^ tl) & 1) cross |= 1u << tl;
-                }
-                bool ok = true;
-                for (int s = 0; s < nheads && ok; ++s) {
-                    const int qb = s & 1;
-                    const int buf = nb == 2 ? (s & 1) : 0;
-                    const uint32_t use = nb == 2 ? (uint32_t)(s >> 1) : (uint32_t)s;  // earlier heads in this buffer
-                    if (!wait_phase(BAR(Q_FULL + qb), (s >> 1) & 1, ctl)) break;
+        // Two issuing warps (1 and 2; the whole warp runs the loop and an elected
+        // thread issues) take alternate tiles: issuing a tile (two barrier waits,
+        // the contractions, two commits) costs more time than the tensor core
+        // needs to run it, so one warp's waits and commits overlap the other's
+        // contractions. Each warp follows the global tile sequence for the ring's
+        // stage and phase and commits its own contractions. The operand
+        // descriptors are made once (per head for Q, per tile for K) and each K
+        // step adds a constant to the start-address field (shared-memory offsets
+        // stay below 256 KB, so the 14-bit field never carries). Issued from one
+        // lane on per-thread registers (ptx.cuh, elect_one) the scores of 128
+        // requests of 3456 tokens, T = 64, 32 heads took 734 us, this way 680.
+        const int who = warp - 1;  // 0: even tiles, 1: odd tiles
+        const int umt = uniform(mt), unb = uniform(nb), uheads = uniform(nheads);
+        if (umt > 0) {
+            const uint32_t idesc = idesc_make(128, (uint32_t)uniform(n2), FMT);
+            // A stage's consecutive loads can belong to different warps
+            // (tiles gt and gt - kStages of opposite parity within their
+            // heads). The K_FULL parity test is only sound once the stage's
+            // previous load has landed, which a warp knows of its own tiles
+            // but not of the other warp's: for those tiles it first waits
+            // for the release of the previous load (its contraction done, so
+            // its data had landed). `cross` marks them by tile.
+            uint32_t cross = 0;
+            for (int tl = who; tl < umt; tl += 2) {
+                const int ptl = ((tl - kStages) % umt + umt) % umt;
+                if ((ptl ^ tl) & 1) cross |= 1u << tl;
+            }
+            bool ok = true;
+            for (int s = 0; s < uheads && ok; ++s) {
+                const int qb = s & 1;
+                const int buf = unb == 2 ? (s & 1) : 0;
+                const uint32_t use = unb == 2 ? (uint32_t)(s >> 1) : (uint32_t)s;  // earlier heads in this buffer
+                if (!wait_phase_warp(BAR(Q_FULL + qb), (s >> 1) & 1, ctl)) break;
+                tc_fence_after();
+                const uint64_t qdesc = sdesc_k_sw128(base + L::OFF_Q + qb * L::Q_BYTES);
+                for (int tl = who; tl < umt; tl += 2) {
+                    const int sl = buf * kBufSlots + tl;
+                    const int gt = s * umt + tl;  // the ring runs over the tiles of all heads in order
+                    const uint32_t ks = (uint32_t)(gt % kStages), kph = (uint32_t)(gt / kStages) & 1u;
+                    if (((cross >> tl) & 1u) && gt >= kStages && !wait_phase_warp(BAR(K_EMPTY + ks), kph ^ 1u, ctl)) {
+                        ok = false;
+                        break;
+                    }
+                    if (!wait_phase_warp(BAR(K_FULL + ks), kph, ctl)) { ok = false; break; }
+                    if (!wait_phase_warp(BAR(S_EMPTY + sl), (use & 1u) ^ 1u, ctl)) { ok = false; break; }
                     tc_fence_after();
-                    const uint64_t qdesc = sdesc_k_sw128(base + L::OFF_Q + qb * L::Q_BYTES);
-                    for (int tl = who; tl < mt; tl += 2) {
-                        const int sl = buf * kBufSlots + tl;
-                        const int gt = s * mt + tl;  // the ring runs over the tiles of all heads in order
-                        const uint32_t ks = (uint32_t)(gt % kStages), kph = (uint32_t)(gt / kStages) & 1u;
-                        if (((cross >> tl) & 1u) && gt >= kStages && !wait_phase(BAR(K_EMPTY + ks), kph ^ 1u, ctl)) {
-                            ok = false;
-                            break;
-                        }
-                        if (!wait_phase(BAR(K_FULL + ks), kph, ctl)) { ok = false; break; }
-                        if (!wait_phase(BAR(S_EMPTY + sl), (use & 1u) ^ 1u, ctl)) { ok = false; break; }
-                        tc_fence_after();
-                        const uint64_t kdesc = sdesc_k_sw128(base + L::OFF_K + ks * L::TILE_BYTES);
-                        const uint32_t d = tmem + (uint32_t)(buf * kBufCols + tl * scols);
+                    const uint64_t kdesc = sdesc_k_sw128(base + L::OFF_K + ks * L::TILE_BYTES);
+                    const uint32_t d = tmem + (uint32_t)(buf * kBufCols + tl * scols);
+                    if (elect_one()) {
 #pragma unroll
                         for (int st = 0; st < KSTEPS; ++st) {
                             constexpr uint64_t kQ16 = MROWS * 128 / 16, kK16 = kTileRows * 128 / 16;
@@ -433,17 +436,19 @@ __global__ void __launch_bounds__(kResThreads, 1)
                         mma_commit(BAR(S_FULL + sl));
                         mma_commit(BAR(K_EMPTY + ks));
                     }
-                    // Q(s) is free once both threads' contractions of head s are done
-                    // (one arrival each; a thread without tiles in this head arrives at once)
-                    if (ok) mma_commit(BAR(Q_EMPTY + qb));
+                    __syncwarp();
                 }
+                // Q(s) is free once both warps' contractions of head s are done
+                // (one arrival each; a warp without tiles in this head arrives at once)
+                if (ok && elect_one()) mma_commit(BAR(Q_EMPTY + qb));
+                __syncwarp();
             }
-            mma_commit(BAR(DRAIN));
-            volatile int no_abort = 0;
-            const Ctl drain_ctl{&no_abort, p.err, kWaitBudgetCycles};
-            wait_phase(BAR(DRAIN), 0, drain_ctl);
         }
+        if (elect_one()) mma_commit(BAR(DRAIN));
         __syncwarp();
+        volatile int no_abort = 0;
+        const Ctl drain_ctl{&no_abort, p.err, kWaitBudgetCycles};
+        wait_phase_warp(BAR(DRAIN), 0, drain_ctl);
         cluster_wait();
     } else {
         // ------------------------------------------------------------ epilogue (kResWG warpgroups)
