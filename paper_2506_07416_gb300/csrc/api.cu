@@ -170,22 +170,22 @@ bool uniform_batch(int batch, const int32_t* seq_offsets_h, const int32_t* text_
 
 // Picks the score kernel and its launch shape by modelled time (microseconds,
 // fitted on GB300 to launches of 1 to 128 requests; KernelCosts below).
-//   Resident kernel: a CTA takes 8 to start and leave (2 more with a fold of
-// several head groups); a head with one TMEM buffer takes 0.8 a tile plus 0.8 for
+//   Resident kernel: a CTA takes 7.5 to start and leave (2 more with a fold of
+// several head groups); a head with one TMEM buffer takes 0.75 a tile plus 0.75 for
 // the cluster exchange, with two buffers (MMAs and exchange under the epilogue)
-// 0.6 a tile plus 2.1, and at least the time its K tiles need at the CTA's share
+// 0.56 a tile plus 2.0, and at least the time its K tiles need at the CTA's share
 // of HBM bandwidth. Waves of CTAs come from the measured cluster occupancy.
 //   Re-read kernel: 6 to start (launch, set-up, first copies and contractions
-// from cold memory) and leave; per head two passes over the tiles, 1.2 a tile for
-// 256-byte rows with more than 64 query rows (the contractions' operands come out
-// of shared memory at its full rate beside the copies coming in), 1.0 up to 64,
-// 0.75 for 128-byte rows; 1.5 for the exchange over a cluster, 0.5 within one CTA;
-// the fold is a launch of its own, 2. It computes every contraction twice but has
+// from cold memory) and leave, 1 from one item to the next in a CTA without a
+// cluster; per head two passes over the tiles, 1.12 a tile for 256-byte rows with
+// more than 64 query rows, 0.86 up to 64 (the epilogue's time), 0.65 for 128-byte
+// rows; 1.5 for the exchange over a cluster, 0.5 within one CTA; the fold is a
+// launch of its own, 2 and its bytes. It computes every contraction twice but has
 // no phases that wait for one another and no clusters to place; it is taken where
 // its model is more than 10% below: ragged batches (12 requests of 2 to 20 tiles,
-// T up to 127, 32 / 8 heads: 47 against 108 us), not large uniform ones (128 x 27
-// tiles, T = 64: 1000 against 734 us) nor short single requests, where both take
-// the time of a launch (12 tiles, 16 heads: 11.4 and 11.9 us).
+// T up to 127, 32 / 8 heads: 38 against 100 us), not large uniform ones (32 x 27
+// tiles, T = 64, 32 heads: 251 against 188 us) nor short single requests, where both
+// take the time of a launch (12 tiles, 16 heads: 11.4 us).
 //   limit_rule: the older model by which the no-alloc entry point decides whether
 // a batch is within its static scratch (so that what it takes does not move with
 // the plans); in units of 1.17 us, the re-read kernel's times 1.6.
@@ -233,12 +233,12 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     for (int cl = 1; cl <= lvs::kMaxCluster; ++cl)
         if (tcap[cl] < 0) tcap[cl] = lvs::tc_cluster_capacity(row_bytes, fp8, hp * max_t <= 64 ? 64 : 128, cl);
     const double u = 1.17;
-    const lvs::KernelCosts res_costs = limit_rule ? lvs::KernelCosts{6.0 * u, u, u, 0.25 * u, 2.0 * u, false}
-                                                  : lvs::KernelCosts{8.0, 0.8, 0.8, 0.25, 2.0, false};
-    const double two_tile = limit_rule ? 0.6 * u : 0.6, two_head = limit_rule ? 2.1 * u : 2.1;
+    const lvs::KernelCosts res_costs = limit_rule ? lvs::KernelCosts{6.0 * u, 6.0 * u, u, u, 0.25 * u, 2.0 * u, false}
+                                                  : lvs::KernelCosts{7.5, 7.5, 0.75, 0.75, 0.25, 2.0, false};
+    const double two_tile = limit_rule ? 0.6 * u : 0.56, two_head = limit_rule ? 2.1 * u : 2.0;
     const lvs::KernelCosts tc_costs =
-        limit_rule ? lvs::KernelCosts{9.6 * u, 1.6 * u, 1.6 * u, 0.4 * u, 3.2 * u, false}
-                   : lvs::KernelCosts{6.0, row_bytes == 256 ? (hp * max_t > 64 ? 1.2 : 1.0) : 0.75, 1.5, 0.5, 2.0, true};
+        limit_rule ? lvs::KernelCosts{9.6 * u, 9.6 * u, 1.6 * u, 1.6 * u, 0.4 * u, 3.2 * u, false}
+                   : lvs::KernelCosts{6.0, 1.0, row_bytes == 256 ? (hp * max_t > 64 ? 1.12 : 0.86) : 0.65, 1.5, 0.5, 2.0, true};
     ScoreChoice best{false, lvs::plan_score(bt, hq / hp, c.num_kv_heads, row_bytes, tcap, tc_costs,
                                             limit_rule ? 2.0 : 1.0, &tc_cost)};
     best.plan.hp = hp;
@@ -440,7 +440,8 @@ litevlm_status_t litevlm_select_create(const litevlm_select_config_t* c, litevlm
     if (e == cudaSuccess && c->num_q_heads > 1)
         e = cudaMalloc(&h->partials, sizeof(float) * (size_t)c->num_q_heads * (size_t)c->max_total_visual);
     // one fold ticket per 128-token tile: index floor(n0 / 128) + t + b < total / 128 + 2 * batch + 1
-    h->n_counters = (size_t)(c->max_total_visual / lvs::kTileRows) + 2 * (size_t)c->max_batch + 2;
+    // (and behind them the two counts of the re-read kernel's claims)
+    h->n_counters = (size_t)(c->max_total_visual / lvs::kTileRows) + 2 * (size_t)c->max_batch + 2 + 2;
     if (e == cudaSuccess) e = cudaMalloc(&h->counters, sizeof(int32_t) * h->n_counters);
     if (e == cudaSuccess) e = cudaMemset(h->counters, 0, sizeof(int32_t) * h->n_counters);
     if (e == cudaSuccess)
@@ -607,6 +608,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     p.out = scores;
     p.partials = h->partials;
     p.counters = h->counters;
+    p.claims = h->counters + (h->n_counters - 2);
     p.err = h->err_d;
     p.total_vis = tot_n;
     p.hq = c.num_q_heads;
@@ -673,6 +675,9 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     if (clear_tickets > 0 && choice.resident && plan.groups > 1) {
         const cudaError_t ce = cudaMemsetAsync(h->counters, 0, sizeof(int32_t) * clear_tickets, (cudaStream_t)stream);
         if (ce != cudaSuccess) return cuda_fail(h, ce, "clearing the fold tickets");
+    } else if (clear_tickets > 0 && !choice.resident && plan.cluster == 1 && plan.ctas < plan.groups * batch) {
+        const cudaError_t ce = cudaMemsetAsync(p.claims, 0, 2 * sizeof(int32_t), (cudaStream_t)stream);
+        if (ce != cudaSuccess) return cuda_fail(h, ce, "clearing the claims");
     }
     const cudaError_t e =
         choice.resident
@@ -1231,7 +1236,7 @@ constexpr int64_t kNoAllocTickets = int64_t(1) << 14;        // 64 KiB of fold t
 constexpr int kNoAllocMaxDevices = 64;
 
 static __device__ __align__(256) float g_noalloc_partials[kNoAllocPartialFloats];
-static __device__ __align__(256) int32_t g_noalloc_tickets[kNoAllocTickets];
+static __device__ __align__(256) int32_t g_noalloc_tickets[kNoAllocTickets + 2];  // and the claims
 
 struct NoAllocDevice {
     bool ready = false;
@@ -1340,7 +1345,7 @@ extern "C" litevlm_status_t litevlm_select_score_noalloc(int32_t num_q_heads, in
         h.num_sms = d.num_sms;
         h.partials = d.partials;
         h.counters = d.tickets;
-        h.n_counters = (size_t)kNoAllocTickets;
+        h.n_counters = (size_t)kNoAllocTickets + 2;
         h.encode = d.encode;
         for (int r = 0; r < 2; ++r)
             for (int c = 0; c < 17; ++c) {

@@ -31,6 +31,11 @@ struct ScoreLaunch {
     // re-read kernel: query heads of one key head whose text rows share a
     // contraction (a head block), and text rows per Q tile (instance rows / hp)
     int32_t hp, box_rows;
+    // re-read kernel without clusters: its CTAs share `items` (request, head
+    // group) items; claims[0] counts those taken beyond a CTA's first, claims[1]
+    // the CTAs that are done (zero between launches, workspace)
+    int32_t items;
+    int32_t* claims;
     int32_t ctas_per_request; // cluster size * groups
     int32_t slot_cols;        // resident kernel: TMEM columns per slot (query rows per head, rounded up to 16)
     // resident kernel: 1, or 2 when each query head's text rows run as two
@@ -75,6 +80,7 @@ struct ScorePlan {
     int res_nb = 1;           // resident kernel: TMEM head buffers
     int flat = 0;             // resident kernel: clusters of the flattened (request, head) schedule, 0: none
     int qsplit = 1;           // resident kernel: 2 = each head's text rows as two pseudo-heads (64-row kernel)
+    int ctas = 0;             // re-read kernel without clusters: CTAs that run at once
     int hp = 1;               // re-read kernel: query heads per head block
 };
 
@@ -140,11 +146,12 @@ double makespan(const BatchTiles& bt, int g, int slots, const Cost& cost)
     return mx;
 }
 
-// Modelled times of the planners, in microseconds: a CTA's start and end, a tile
-// of a head, a head's statistics exchange over a cluster / within one CTA, and a
-// fold of several head groups (per CTA, or once when it is a launch of its own).
+// Modelled times of the planners, in microseconds: a CTA's start and end, the step
+// from one item to the next in a CTA that works through several, a tile of a head,
+// a head's statistics exchange over a cluster / within one CTA, and a fold of
+// several head groups (per CTA, or once when it is a launch of its own).
 struct KernelCosts {
-    double start, tile, exchange, exchange_one, fold;
+    double start, next, tile, exchange, exchange_one, fold;
     bool fold_once;
 };
 // cap_by_cluster[c]: CTAs of the re-read kernel resident at once with clusters of c (<= 0: unusable)

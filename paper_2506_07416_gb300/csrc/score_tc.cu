@@ -26,6 +26,11 @@
 // tile being text row i of head h. "Head" below means such a block: it streams
 // the key head's tiles once instead of hp times (last-token queries of 64
 // requests, 32 / 8 heads: 314 -> 106 us).
+// A CTA without a cluster works through several (request, head group) items,
+// claimed largest first: its set-up and teardown (5 us) are paid once, and the
+// groups can be finer. Scores of 12 requests of 322 to 2491 tokens, 32 / 8 heads: 45
+// -> 38 us; 16 requests of 636 to 2586, 16 heads: 36.5 -> 33.9; 32 requests of 629 to
+// 3404 in e4m3, 32 heads: 109 -> 106.
 // Software pipeline with one head of look-ahead: pass 1 of head s+1 runs while
 // the statistics of head s travel across the cluster, then pass 2 of head s
 // (a CTA that is its own cluster has nothing to wait for and runs the two
@@ -50,7 +55,10 @@
 // lane quadrant = warp % 4). A contraction unit is one tile of one pass; the
 // units cycle through four 128-column TMEM buffers in issue order, and unit u
 // belongs to issuer u & 1 and to warpgroup u & 1: two independent pipelines,
-// each with one buffer being read and one being filled. Eight epilogue warps keep
+// each with one buffer being read and one being filled. Both issuers elect a thread
+// of a uniform warp (ptx.cuh, elect_one): from one lane on per-thread registers the
+// contractions set the pace at 740 cycles a unit (bf16; e4m3 470), now the epilogue
+// does at 800 for 128 query rows, 500 for 32 (e4m3 item above: 121 -> 109 us). Eight epilogue warps keep
 // the exponential unit as busy as sixteen do (4.8 cycles per 2^x and SM quarter
 // against 4.0 at best) and leave 168 registers a thread for straight-line blocks
 // of 64 columns: a branch per 32 columns (the reference check, the column count)
@@ -106,12 +114,27 @@ struct SmemLayout {
     static constexpr int OFF_B2 = OFF_STATS + kStatSlots * kMaxText * 8;
     static constexpr int OFF_XS = OFF_B2 + 2 * kMaxText * 4;  // [head & 1][kEpiWG - 1][128] float2: other warpgroups' row stats
     static constexpr int OFF_BAR = OFF_XS + 2 * (kEpiWG - 1) * kMaxText * 8;
-    // k_full[S], k_empty[S], q_full[QBUF], q_empty[QBUF], t1_full[2], t1_empty[2],
-    // t2_full[2], t2_empty[2], stats[4], drain
-    static constexpr int NBAR = 2 * kStages + 2 * QBUF + 2 * 4 + kStatSlots + 2;
-    static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
+    // k_full[S], k_empty[S], q_full[QBUF], q_empty[QBUF], u_full[4], u_empty[4],
+    // stats[4], drain, stall, item_full[2], item_empty[2]
+    static constexpr int NBAR = 2 * kStages + 2 * QBUF + 2 * 4 + kStatSlots + 2 + 4;
+    static constexpr int OFF_ITEMS = OFF_BAR + NBAR * 8;  // [3][5] int: the items in work, the epilogue's
+    static constexpr int OFF_MISC = OFF_ITEMS + 3 * 5 * 4;
     static constexpr int BYTES = OFF_MISC + 16;
     static constexpr int ALLOC = BYTES + 1024;  // slack for 1024-byte alignment
+};
+
+// An item as claimed, and what a CTA of its cluster serves of it.
+struct TcItem {
+    int hg, n0, N, t0, T;
+};
+struct TcWork {
+    int hg, n0, N, t0, T;
+    int R, n2;                     // query rows of a head block, rounded up to 16
+    int tile_begin, tile_end, mt;
+    // pass 1 runs with M = 64 for a request of at most 64 query rows, also in the
+    // 128-row instance: its rows then lie in 16 lanes of each of the four lane
+    // quadrants, so all SM sub-partitions work on them
+    bool m64;
 };
 
 template <int ROW_BYTES, bool FP8, int MROWS>
@@ -134,14 +157,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t csize = cluster_nctarank();
-    const int item = (int)(blockIdx.x / csize);  // this cluster's (request, head group)
-    const int req_i = item / p.groups;
-    const int b = p.order_n > 0 ? (int)p.order[req_i] : req_i;
-    const int hg = item - req_i * p.groups;
-
     // With the full-key-set terms (p.extra, written by the kernel launched just
     // before this one) only the threads that read them wait for that kernel,
     // right before the read: this kernel's other inputs come from kernels that
@@ -150,35 +168,62 @@ __global__ void __launch_bounds__(kThreads, 1)
     // completes ahead of that one.
     if (!p.extra) griddep_wait();
     griddep_launch_dependents();
-    // the request's offsets: by value for small batches (no global load)
-    const bool byv = p.nv > 0;
-    const int n0 = byv ? p.so_v[b] : p.seq_off[b];
-    const int N = (byv ? p.so_v[b + 1] : p.seq_off[b + 1]) - n0;
-    const int tq = byv ? p.to_v[b] : p.text_off[b];
-    const int t1 = byv ? p.to_v[b + 1] : p.text_off[b + 1];
-    const int t0 = p.query_last && t1 > tq ? t1 - 1 : tq;  // last-token queries: one row
-    const int T = t1 - t0;
     const bool multi = p.groups > 1;
-    const int hp = p.hp, R = T * hp;  // query heads and rows of a head block
-    // Uniform for the whole cluster (same request).
-    if (R > MROWS || (N > 0 && T <= 0) || N <= 0) {
-        if (p.extra) griddep_wait();
-        if (N > 0 && threadIdx.x == 0 && rank == 0 && hg == 0) atomicOr(p.err, kErrShape);
-        return;
-    }
-    const int n_tiles = (N + kTileRows - 1) / kTileRows;
-    const int tpc = (n_tiles + (int)csize - 1) / (int)csize;
-    const int tile_begin = min(n_tiles, (int)rank * tpc);
-    const int tile_end = min(n_tiles, tile_begin + tpc);
-    const int mt = tile_end - tile_begin;
-    const int n2 = (R + 15) & ~15;
-    // pass 1 runs with M = 64 for a request of at most 64 query rows, also in the
-    // 128-row instance: its rows then lie in 16 lanes of each of the four lane
-    // quadrants, so all SM sub-partitions work on them
-    const bool m64 = MROWS == 64 || R <= 64;
+    const int hp = p.hp;  // query heads of a head block
     const int G = p.hq / p.hkv;
     const int hpg = p.heads_per_group;
     const float cl = p.c_log2;
+    // An item is a (request, head group); without a cluster a CTA works through
+    // several, claimed in order of size (p.claims), and its roles run on from one
+    // to the next: the copies and contractions of an item's first tiles lie under
+    // the end of the one before.
+    const bool shared = csize == 1 && (int)gridDim.x < p.items;  // items beyond each CTA's first
+    auto make_work = [&](const TcItem& i) -> TcWork {
+        TcWork w;
+        w.hg = i.hg;
+        w.n0 = i.n0;
+        w.N = i.N;
+        w.t0 = i.t0;
+        w.T = i.T;
+        w.R = i.T * hp;
+        const int n_tiles = (i.N + kTileRows - 1) / kTileRows;
+        const int tpc = (n_tiles + (int)csize - 1) / (int)csize;
+        w.tile_begin = min(n_tiles, (int)rank * tpc);
+        w.tile_end = min(n_tiles, w.tile_begin + tpc);
+        w.mt = w.tile_end - w.tile_begin;
+        w.n2 = (w.R + 15) & ~15;
+        w.m64 = MROWS == 64 || w.R <= 64;
+        return w;
+    };
+    // N = 0 for an item without work; shape errors are caught on the host, this
+    // only keeps the kernel within its buffers
+    auto get_item = [&](int item) -> TcItem {
+        const int req_i = item / p.groups;
+        const int b = p.order_n > 0 ? (int)p.order[req_i] : req_i;
+        // the request's offsets: by value for small batches (no global load)
+        const bool byv = p.nv > 0;
+        TcItem i;
+        i.hg = item - req_i * p.groups;
+        i.n0 = byv ? p.so_v[b] : p.seq_off[b];
+        i.N = (byv ? p.so_v[b + 1] : p.seq_off[b + 1]) - i.n0;
+        const int tq = byv ? p.to_v[b] : p.text_off[b];
+        const int t1 = byv ? p.to_v[b + 1] : p.text_off[b + 1];
+        i.t0 = p.query_last && t1 > tq ? t1 - 1 : tq;  // last-token queries: one row
+        i.T = t1 - i.t0;
+        if (i.N > 0 && (i.T <= 0 || i.T * hp > MROWS || (i.N + kTileRows - 1) / kTileRows > kMaxTilesPerCta * (int)csize)) {
+            atomicOr(p.err, kErrShape);
+            i.N = 0;
+        }
+        return i;
+    };
+    TcWork mine{};  // the one item of a cluster
+    if (csize > 1) {
+        mine = make_work(get_item((int)(blockIdx.x / csize)));
+        if (mine.N <= 0) {  // uniform for the whole cluster
+            if (p.extra) griddep_wait();
+            return;
+        }
+    }
     // Pass 2 of a head follows pass 1 of the next head (lag 1), so the
     // statistics exchange of the cluster overlaps a contraction; a CTA without
     // peers needs no exchange and runs both passes of a head in turn (lag 0),
@@ -191,7 +236,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // contractions of both passes, in issue order (unit u uses buffer u % 4)
     const int K_FULL = 0, K_EMPTY = kStages, Q_FULL = 2 * kStages, Q_EMPTY = Q_FULL + QBUF, U_FULL = Q_EMPTY + QBUF,
               U_EMPTY = U_FULL + 4, STATS = U_EMPTY + 4,
-              DRAIN = STATS + kStatSlots, STALL = DRAIN + 1;
+              DRAIN = STATS + kStatSlots, STALL = DRAIN + 1, IT_FULL = STALL + 1, IT_EMPTY = IT_FULL + 2;
+    volatile int* items_s = reinterpret_cast<volatile int*>(smem + L::OFF_ITEMS);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 4);
     float* acc_s = reinterpret_cast<float*>(smem + L::OFF_ACC);
@@ -215,6 +261,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = 0; i < kStatSlots; ++i) mbar_init(BAR(STATS + i), csize);
         mbar_init(BAR(DRAIN), 2);
         mbar_init(BAR(STALL), 1);  // nothing ever arrives (the debug stall below)
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(BAR(IT_FULL + i), 1);
+            mbar_init(BAR(IT_EMPTY + i), 3);  // the issuers and the epilogue
+        }
         *abort_flag = 0;
         fence_mbar_init_cluster();
     }
@@ -244,13 +294,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     // needs no release: the barriers' set-up is released by fence.mbarrier_init
     // above, and the statistics peers read are released by their own arrivals.
     cluster_arrive_relaxed();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     const Ctl ctl{abort_flag, p.err, p.wait_budget};
 
-    // Pipeline step s (0..hpg): pass 1 of head s (s < hpg), then pass 2 of head s-1 (s >= 1).
+    // the k-th item of this CTA, for one thread of each role that follows the
+    // producer; N = 0 when there is none, or after an abort
+    auto take_item = [&](int k) -> TcItem {
+        TcItem i{0, 0, 0, 0, 0};
+        if (poll_phase(BAR(IT_FULL + (k & 1)), (uint32_t)(k >> 1) & 1u, ctl)) {
+            const volatile int* q = items_s + (k & 1) * 5;
+            i = TcItem{q[0], q[1], q[2], q[3], q[4]};
+            mbar_arrive(BAR(IT_EMPTY + (k & 1)));
+        }
+        return i;
+    };
+
+    // Pipeline step s of an item (0..hpg): pass 1 of head s (s < hpg), then pass 2 of
+    // head s - lag. hc counts the heads of the items before.
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0 && mt > 0) {
+        if (lane == 0) {
             uint32_t ks = 0, kph = 0;
             int k_issued[kStages];
             int q_issued[QBUF];
@@ -261,33 +324,56 @@ __global__ void __launch_bounds__(kThreads, 1)
             // of budget and every other wait of the launch runs out or sees the
             // abort flag, with no copy or contraction in flight.
             bool ok = !p.stall || poll_phase(BAR(STALL), 0, ctl);
-            auto load_tiles = [&](int g) {
-                for (int t = tile_begin; t < tile_end && ok; ++t) {
-                    if (!poll_phase(BAR(K_EMPTY + ks), kph ^ 1, ctl)) { ok = false; break; }
-                    mbar_arrive_expect_tx(BAR(K_FULL + ks), L::TILE_BYTES);
-                    const uint32_t kdst = base + L::OFF_K + ks * L::TILE_BYTES;
-#pragma unroll
-                    for (int kb = 0; kb < L::KB; ++kb)
-                        tma_load_3d(kdst + kb * kTileRows * 128, &tm_k, BAR(K_FULL + ks), kb * ELEMS_PER_KB, g,
-                                    n0 + t * kTileRows);
-                    ++k_issued[ks];
-                    if (++ks == kStages) { ks = 0; kph ^= 1; }
+            int item = (int)blockIdx.x, hc = 0;
+            for (int k = 0; ok; ++k, hc += hpg) {
+                TcWork w;
+                if (csize > 1) {
+                    if (k > 0 || mine.mt == 0) break;
+                    w = mine;
+                } else {
+                    TcItem i{0, 0, 0, 0, 0};
+                    if (k > 0) item = shared ? (int)gridDim.x + atomicAdd(p.claims, 1) : p.items;
+                    while (item < p.items && (i = get_item(item)).N <= 0)
+                        item = shared ? (int)gridDim.x + atomicAdd(p.claims, 1) : p.items;
+                    if (!poll_phase(BAR(IT_EMPTY + (k & 1)), ((uint32_t)(k >> 1) & 1u) ^ 1u, ctl)) break;
+                    volatile int* q = items_s + (k & 1) * 5;
+                    q[0] = i.hg;
+                    q[1] = i.n0;
+                    q[2] = i.N;
+                    q[3] = i.t0;
+                    q[4] = i.T;
+                    mbar_arrive(BAR(IT_FULL + (k & 1)));
+                    if (i.N <= 0) break;  // the end, for every role
+                    w = make_work(i);
                 }
-            };
-            for (int s = 0; s < hpg + lag && ok; ++s) {
-                if (s < hpg) {
-                    const int h = (hg * hpg + s) * hp;
-                    const int qb = s % QBUF;
-                    if (!poll_phase(BAR(Q_EMPTY + qb), ((s / QBUF) & 1) ^ 1, ctl)) break;
-                    mbar_arrive_expect_tx(BAR(Q_FULL + qb), (uint32_t)(L::KB * 128 * hp * p.box_rows));
-                    const uint32_t qdst = base + L::OFF_Q + qb * L::Q_BYTES;
+                auto load_tiles = [&](int g) {
+                    for (int t = w.tile_begin; t < w.tile_end && ok; ++t) {
+                        if (!poll_phase(BAR(K_EMPTY + ks), kph ^ 1, ctl)) { ok = false; break; }
+                        mbar_arrive_expect_tx(BAR(K_FULL + ks), L::TILE_BYTES);
+                        const uint32_t kdst = base + L::OFF_K + ks * L::TILE_BYTES;
 #pragma unroll
-                    for (int kb = 0; kb < L::KB; ++kb)
-                        tma_load_3d(qdst + kb * MROWS * 128, &tm_q, BAR(Q_FULL + qb), kb * ELEMS_PER_KB, h, t0);
-                    ++q_issued[qb];
-                    load_tiles(h / G);
+                        for (int kb = 0; kb < L::KB; ++kb)
+                            tma_load_3d(kdst + kb * kTileRows * 128, &tm_k, BAR(K_FULL + ks), kb * ELEMS_PER_KB, g,
+                                        w.n0 + t * kTileRows);
+                        ++k_issued[ks];
+                        if (++ks == kStages) { ks = 0; kph ^= 1; }
+                    }
+                };
+                for (int s = 0; s < hpg + lag && ok; ++s) {
+                    if (s < hpg) {
+                        const int h = (w.hg * hpg + s) * hp;
+                        const int qb = (hc + s) % QBUF;
+                        if (!poll_phase(BAR(Q_EMPTY + qb), ((uint32_t)((hc + s) / QBUF) & 1u) ^ 1u, ctl)) { ok = false; break; }
+                        mbar_arrive_expect_tx(BAR(Q_FULL + qb), (uint32_t)(L::KB * 128 * hp * p.box_rows));
+                        const uint32_t qdst = base + L::OFF_Q + qb * L::Q_BYTES;
+#pragma unroll
+                        for (int kb = 0; kb < L::KB; ++kb)
+                            tma_load_3d(qdst + kb * MROWS * 128, &tm_q, BAR(Q_FULL + qb), kb * ELEMS_PER_KB, h, w.t0);
+                        ++q_issued[qb];
+                        load_tiles(h / G);
+                    }
+                    if (s >= lag && ok) load_tiles((w.hg * hpg + s - lag) * hp / G);
                 }
-                if (s >= lag && ok) load_tiles((hg * hpg + s - lag) * hp / G);
             }
             // drain: the last load of every slot lands before the CTA leaves
             // (these waits ignore the abort flag)
@@ -302,70 +388,84 @@ __global__ void __launch_bounds__(kThreads, 1)
         cluster_wait();
     } else if (warp <= 2) {
         // ------------------------------------------------------------ MMA issuers
-        // Lane 0 of warps 1 and 2; issuer `who` takes the units u with (u & 1)
-        // == who, their stages and TMEM buffers (both counts are even). The
-        // operand descriptors are made once per head (Q) and unit (K); each K
-        // step adds a constant to the start-address field (shared-memory
-        // offsets stay below 256 KB, so the 14-bit field never carries).
-        if (lane == 0) {
-            const uint32_t who = (uint32_t)(warp - 1);
-            if (mt > 0) {
-                const uint32_t idesc1 = idesc_make(m64 ? 64 : 128, 128, FMT);
-                const uint32_t idesc2 = idesc_make(128, (uint32_t)n2, FMT);
-                uint32_t ks = 0, kph = 0, ui = 0;
-                bool ok = true;
-                for (int s = 0; s < hpg + lag && ok; ++s) {
-                    for (int pass = 0; pass < 2 && ok; ++pass) {
-                        if (pass == 0 && s >= hpg) continue;
-                        if (pass == 1 && s < lag) continue;
-                        const int hs = pass == 0 ? s : s - lag;  // head of these units
-                        const int qb = hs % QBUF;
-                        if (pass == 0) {
-                            if (!poll_phase(BAR(Q_FULL + qb), (hs / QBUF) & 1, ctl)) { ok = false; break; }
-                            tc_fence_after();
+        // Warps 1 and 2; issuer `who` takes the units u with (u & 1) == who, their
+        // stages and TMEM buffers (both counts are even). The whole warp runs the
+        // loop and an elected thread issues (elect_one). The operand descriptors
+        // are made once per head (Q) and unit (K); each K step adds a constant to
+        // the start-address field (shared-memory offsets stay below 256 KB, so the
+        // 14-bit field never carries).
+        const uint32_t who = (uint32_t)(warp - 1);
+        const uint32_t idesc_r64 = idesc_make(64, 128, FMT), idesc_r128 = idesc_make(128, 128, FMT);
+        uint32_t ks = 0, kph = 0, ui = 0;
+        bool ok = true;
+        int hc = 0;
+        for (int k = 0; ok; ++k, hc += hpg) {
+            if (csize > 1 && k > 0) break;
+            TcItem item{mine.hg, mine.n0, mine.N, mine.t0, mine.T};
+            if (csize == 1) {
+                if (lane == 0) item = take_item(k);
+                __syncwarp();
+            }
+            item = TcItem{uniform(item.hg), uniform(item.n0), uniform(item.N), uniform(item.t0), uniform(item.T)};
+            const TcWork w = make_work(item);
+            if (w.N <= 0 || w.mt == 0) break;
+            const uint32_t idesc1 = w.m64 ? idesc_r64 : idesc_r128;
+            const uint32_t idesc2 = idesc_make(128, (uint32_t)w.n2, FMT);
+            for (int s = 0; s < hpg + lag && ok; ++s) {
+                for (int pass = 0; pass < 2 && ok; ++pass) {
+                    if (pass == 0 && s >= hpg) continue;
+                    if (pass == 1 && s < lag) continue;
+                    const int hs = hc + (pass == 0 ? s : s - lag);  // head of these units
+                    const int qb = hs % QBUF;
+                    if (pass == 0) {
+                        if (!poll_phase_warp(BAR(Q_FULL + qb), (uint32_t)(hs / QBUF) & 1u, ctl)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+                    const uint64_t qdesc = sdesc_k_sw128(base + L::OFF_Q + qb * L::Q_BYTES);
+                    for (int t = w.tile_begin; t < w.tile_end; ++t, ++ui) {
+                        const uint32_t st_ks = ks, st_ph = kph;
+                        if (++ks == kStages) { ks = 0; kph ^= 1; }
+                        if ((ui & 1u) != who) continue;
+                        const uint32_t ub = ui & 3, uph = (ui >> 2) & 1;
+                        if (!poll_phase_warp(BAR(K_FULL + st_ks), st_ph, ctl) ||
+                            !poll_phase_warp(BAR(U_EMPTY + ub), uph ^ 1, ctl)) {
+                            ok = false;
+                            break;
                         }
-                        const uint64_t qdesc = sdesc_k_sw128(base + L::OFF_Q + qb * L::Q_BYTES);
-                        for (int t = tile_begin; t < tile_end; ++t, ++ui) {
-                            const uint32_t st_ks = ks, st_ph = kph;
-                            if (++ks == kStages) { ks = 0; kph ^= 1; }
-                            if ((ui & 1u) != who) continue;
-                            const uint32_t ub = ui & 3, uph = (ui >> 2) & 1;
-                            if (!poll_phase(BAR(K_FULL + st_ks), st_ph, ctl) ||
-                                !poll_phase(BAR(U_EMPTY + ub), uph ^ 1, ctl)) {
-                                ok = false;
-                                break;
-                            }
-                            tc_fence_after();
-                            const uint64_t kdesc = sdesc_k_sw128(base + L::OFF_K + st_ks * L::TILE_BYTES);
-                            const uint32_t d = tmem + ub * 128u;
+                        tc_fence_after();
+                        const uint64_t kdesc = sdesc_k_sw128(base + L::OFF_K + st_ks * L::TILE_BYTES);
+                        const uint32_t d = tmem + ub * 128u;
+                        const uint64_t adesc = pass == 0 ? qdesc : kdesc, bdesc = pass == 0 ? kdesc : qdesc;
+                        constexpr uint64_t kQ16 = MROWS * 128 / 16, kK16 = kTileRows * 128 / 16;
+                        const uint64_t ablk = pass == 0 ? kQ16 : kK16, bblk = pass == 0 ? kK16 : kQ16;
+                        const uint32_t idesc = pass == 0 ? idesc1 : idesc2;
+                        if (elect_one()) {
 #pragma unroll
                             for (int st = 0; st < KSTEPS; ++st) {
-                                constexpr uint64_t kQ16 = MROWS * 128 / 16, kK16 = kTileRows * 128 / 16;
-                                const uint64_t qd = qdesc + (uint64_t)(st >> 2) * kQ16 + (uint64_t)(st & 3) * 2;
-                                const uint64_t kd = kdesc + (uint64_t)(st >> 2) * kK16 + (uint64_t)(st & 3) * 2;
-                                if (pass == 0) {
-                                    if (FP8) mma_f8(d, qd, kd, idesc1, st > 0);
-                                    else mma_f16(d, qd, kd, idesc1, st > 0);
-                                } else {
-                                    if (FP8) mma_f8(d, kd, qd, idesc2, st > 0);
-                                    else mma_f16(d, kd, qd, idesc2, st > 0);
-                                }
+                                const uint64_t ad = adesc + (uint64_t)(st >> 2) * ablk + (uint64_t)(st & 3) * 2;
+                                const uint64_t bd = bdesc + (uint64_t)(st >> 2) * bblk + (uint64_t)(st & 3) * 2;
+                                if (FP8) mma_f8(d, ad, bd, idesc, st > 0);
+                                else mma_f16(d, ad, bd, idesc, st > 0);
                             }
                             mma_commit(BAR(U_FULL + ub));
                             mma_commit(BAR(K_EMPTY + st_ks));
                         }
-                        // Q(hs) is free once both issuers' contractions of its pass 2 are done
-                        if (pass == 1 && ok) mma_commit(BAR(Q_EMPTY + qb));
+                        __syncwarp();
+                    }
+                    // Q(hs) is free once both issuers' contractions of its pass 2 are done
+                    if (pass == 1 && ok) {
+                        if (elect_one()) mma_commit(BAR(Q_EMPTY + qb));
+                        __syncwarp();
                     }
                 }
             }
-            // drain: every MMA issued by this thread has completed
-            mma_commit(BAR(DRAIN));
-            volatile int no_abort = 0;
-            const Ctl drain_ctl{&no_abort, p.err, kWaitBudgetCycles};
-            poll_phase(BAR(DRAIN), 0, drain_ctl);
         }
+        // drain: every MMA issued by this warp's thread has completed
+        if (elect_one()) mma_commit(BAR(DRAIN));
         __syncwarp();
+        volatile int no_abort = 0;
+        const Ctl drain_ctl{&no_abort, p.err, kWaitBudgetCycles};
+        poll_phase_warp(BAR(DRAIN), 0, drain_ctl);
         cluster_wait();
     } else {
         // ------------------------------------------------------------ epilogue
@@ -379,11 +479,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int et = threadIdx.x - 96;                      // 0 .. kEpiThreads - 1
         const int vrow = quad * 32 + lane;                    // pass 2: TMEM lane = visual token in tile
         const uint32_t tcol = tmem + ((uint32_t)(quad * 32) << 16);
-        // pass 1 row of this thread: M = 128 -> lane; M = 64 -> lanes 16q..16q+15, two
-        // column halves
-        const int prow = !m64 ? quad * 32 + lane : quad * 16 + (lane & 15);
-        const bool p1_live = !m64 ? (quad * 32 < R) : (quad * 16 < R);
-        for (int tl = wg; tl < mt; tl += kEpiWG) acc_s[tl * kTileRows + vrow] = 0.f;
         const float2 cl2 = make_float2(cl, cl);
         // this warp has read buffer ub: hand it back
         auto release = [&](uint32_t ub) {
@@ -392,6 +487,34 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == 0) mbar_arrive(BAR(U_EMPTY + ub));
         };
         uint32_t ui = 0;  // contraction units in issue order (both passes)
+        int hc = 0;
+        // One thread takes the next item for all of them, so that every warp agrees on
+        // it also when a wait gives up. It writes between two barriers of the
+        // warpgroups that all readers of the item before have passed.
+        volatile int* cur = items_s + 2 * 5;
+        auto next_item = [&](int k) {
+            if (csize == 1 && et == 0) {
+                const TcItem i = take_item(k);
+                cur[0] = i.hg;
+                cur[1] = i.n0;
+                cur[2] = i.N;
+                cur[3] = i.t0;
+                cur[4] = i.T;
+            }
+            named_bar_sync(1, kEpiThreads);
+        };
+        next_item(0);
+        for (int k = 0;; hc += hpg) {
+        const TcWork w = csize > 1 ? mine : make_work(TcItem{cur[0], cur[1], cur[2], cur[3], cur[4]});
+        if (w.N <= 0) break;
+        const int n0 = w.n0, N = w.N, t0 = w.t0, T = w.T, R = w.R, n2 = w.n2, mt = w.mt, hg = w.hg;
+        const int tile_begin = w.tile_begin, tile_end = w.tile_end;
+        const bool m64 = w.m64;
+        // pass 1 row of this thread: M = 128 -> lane; M = 64 -> lanes 16q..16q+15, two
+        // column halves
+        const int prow = !m64 ? quad * 32 + lane : quad * 16 + (lane & 15);
+        const bool p1_live = !m64 ? (quad * 32 < R) : (quad * 16 < R);
+        for (int tl = wg; tl < mt; tl += kEpiWG) acc_s[tl * kTileRows + vrow] = 0.f;
         for (int s = 0; s < hpg + lag; ++s) {
             if (s < hpg) {
                 // ---- pass 1 of head s: row sums over this warpgroup's tiles
@@ -486,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const bool writer = !m64 || lane < 16;
                 // (double-buffered by head: the other warpgroups may publish head s + 1
                 // while the first one is still reading head s)
-                float2* xs = xs_s + (s & 1) * (kEpiWG - 1) * kMaxText;
+                float2* xs = xs_s + ((hc + s) & 1) * (kEpiWG - 1) * kMaxText;
                 if (wg > 0 && writer) xs[(wg - 1) * kMaxText + prow] = make_float2(m, l);
                 named_bar_sync(1, kEpiThreads);
                 if (wg == 0) {
@@ -496,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             const float2 o = xs[(o_wg - 1) * kMaxText + prow];
                             merge_row(m, l, o.x, o.y, cl);
                         }
-                        stats_s[(s % kStatSlots) * kMaxText + prow] = make_float2(m, l);
+                        stats_s[((hc + s) % kStatSlots) * kMaxText + prow] = make_float2(m, l);
                     }
                     named_bar_sync(2, 128);
                     // one release arrival per CTA of the cluster, each from its own
@@ -511,8 +634,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (s >= lag) {
                 // ---- merge the cluster's statistics of head s - lag
                 const int hs = s - lag;
-                const int slot = hs % kStatSlots;
-                float* b2 = b2_s + (hs & 1) * kMaxText;
+                const int slot = (hc + hs) % kStatSlots;
+                float* b2 = b2_s + ((hc + hs) & 1) * kMaxText;
                 if (wg == 0) {
                     // (a CTA that is its own cluster reads its own rows, ordered by the named barrier above)
                     if (csize > 1) poll_phase<true>(BAR(STATS + slot), (uint32_t)(hs / kStatSlots) & 1u, ctl);
@@ -569,7 +692,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
-        named_bar_sync(1, kEpiThreads);  // every tile's sums are in acc_s
+        next_item(++k);  // (with its barrier every tile's sums are in acc_s)
         // ---- results
         const float denom = (float)p.hq * (float)T;
         for (int tl = wg; tl < mt; tl += kEpiWG) {
@@ -579,6 +702,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!multi) p.out[n0 + j] = a / denom;
                 else p.partials[(int64_t)hg * p.total_vis + n0 + j] = a;
             }
+        }
+        if (csize > 1) break;
         }
         tc_fence_before();
     }
@@ -591,6 +716,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (p.extra) griddep_wait();  // returns at once for threads that already waited
     cluster_sync_all();  // peers are done reading this CTA's statistics
+    // the last CTA to leave clears the claims for the next launch
+    if (shared && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(p.claims + 1, 1) == (int)gridDim.x - 1) p.claims[0] = p.claims[1] = 0;
+    }
 }
 
 // scores = sum over the head groups' partial rows, in group order, / (Hq * T):
@@ -667,7 +797,10 @@ cudaError_t launch_variant(const CUtensorMap& tm_q, const CUtensorMap& tm_k, con
     cudaError_t e = tc_prepare<ROW_BYTES, FP8, MROWS>(plan.cluster);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(plan.cluster * plan.groups * batch), 1, 1);
+    // clusters: one per item; without, as many CTAs as run at once, which share the items
+    const int items = plan.groups * batch;
+    const int ctas = plan.cluster > 1 ? plan.cluster * items : items < plan.ctas ? items : plan.ctas;
+    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -711,6 +844,8 @@ ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int row_bytes, const
     }
     const int G = hq / hkv;
     const double tile_bytes = (double)kTileRows * row_bytes;
+    double rows = 0.0;
+    for (int i = 0; i < bt.n; ++i) rows += (double)bt.desc[i] * kTileRows;
     for (int pass = 0; pass < 2 && best_cost >= 1e299; ++pass) {
         for (int c = 1; c <= kMaxCluster; ++c) {
             const int tpc = (max_tiles + c - 1) / c;
@@ -733,16 +868,22 @@ ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int row_bytes, const
                 const int share = hpg >= G ? 1 : G / hpg;
                 const double window = (c > 1 ? 2.0 : window_one) * tpc * tile_bytes * (double)active / share;
                 if (pass == 0 && window > 160.0 * 1024 * 1024) continue;
+                // beyond 110 MB some of the re-read comes from HBM: 32 requests of 27
+                // tiles, 32 heads (134 MB) took 264 us where the tiles alone make 190
+                const double miss = costs.fold_once && window > 110e6 ? 1.0 + (window - 110e6) / 110e6 : 1.0;
                 auto item_cost = [&](int tiles) {
                     const int t = (tiles + c - 1) / c;
-                    return tiles <= 0 ? 1.0
-                                      : costs.start + (g > 1 && !costs.fold_once ? costs.fold : 0.0) +
-                                            hpg * (t * costs.tile + (c > 1 ? costs.exchange : costs.exchange_one));
+                    return tiles <= 0 ? 0.1
+                                      : (c > 1 ? costs.start : costs.next) + (g > 1 && !costs.fold_once ? costs.fold : 0.0) +
+                                            hpg * (t * costs.tile * miss + (c > 1 ? costs.exchange : costs.exchange_one));
                 };
-                const double cost = makespan(bt, g, cap / c, item_cost) + (g > 1 && costs.fold_once ? costs.fold : 0.0);
+                // a fold of its own also moves the partial rows once out and in
+                const double cost = makespan(bt, g, cap / c, item_cost) + (c > 1 ? 0.0 : costs.start - costs.next) +
+                                    (g > 1 && costs.fold_once ? costs.fold + g * rows * 8.0 / 4e6 : 0.0);
                 if (cost < best_cost - 1e-9) {
                     best_cost = cost;
                     best = ScorePlan{c, tpc, g};
+                    best.ctas = cap;
                 }
             }
         }
@@ -773,6 +914,8 @@ cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const
     q.box_rows = mrows / plan.hp;
     q.heads_per_group = p.hq / plan.hp / plan.groups;
     q.ctas_per_request = plan.cluster * plan.groups;
+    q.items = plan.groups * batch;
+    if (plan.cluster == 1 && plan.ctas < 1) return cudaErrorInvalidValue;
     if (fp8) {
         return mrows == 64 ? launch_variant<128, true, 64>(tm_q, tm_k, q, plan, batch, stream)
                            : launch_variant<128, true, 128>(tm_q, tm_k, q, plan, batch, stream);

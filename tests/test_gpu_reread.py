@@ -143,3 +143,33 @@ def test_no_alloc_limit_does_not_follow_the_plan(sel):
     # two kernels, sums in another order: 32-bit rounding over at most 128 * 32 terms a score
     assert float(((out - ref).abs() / ref).max()) < 1e-5
     s.close()
+
+
+@pytest.mark.parametrize("n,t,hq,hkv,d", [
+    ([130, 64, 0, 257, 1] * 40, [3, 64, 5, 20, 65], 4, 4, 128),  # five sizes, empty requests among them
+    ([128] * 180, [16] * 5, 2, 1, 64),                            # one tile, one head block each
+    ([900, 129] * 60, [100, 70, 30, 9, 128], 8, 2, 128),
+], ids=["mixed_empty", "one_tile", "two_sizes"])
+def test_more_items_than_ctas(sel, n, t, hq, hkv, d):
+    """More (request, head group) items than CTAs run at once: the CTAs claim the
+    rest among themselves, and the claims are back at zero for the next launch."""
+    t = [t[i % len(t)] for i in range(len(n))]
+    w = _w("claims", n, t, hq, hkv, d)
+    x = inputs.make_numpy(w)
+    xd = to_device(x, w)
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel="reread")
+    plan = s.score_plan(x["text_offsets"], x["seq_offsets"])
+    assert plan[0] == 1 and plan[1] == 1
+    assert plan[3] * w.batch > torch.cuda.get_device_properties(0).multi_processor_count
+    o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, w.head_dim, w.dtype,
+                     x["q_scale"], x["k_scale"])
+    for _ in range(3):
+        assert_scores_close(_scores(s, x, xd), o, w.dtype)
+    s.close()
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        out = torch.full((w.total_vis,), float("nan"), device="cuda")
+        sel.score_noalloc(w.hq, w.hkv, w.head_dim, w.dtype, w.batch, xd["q"], xd["text_offsets"], x["text_offsets"],
+                          xd["k"], xd["seq_offsets"], x["seq_offsets"], x["q_scale"], x["k_scale"], out, err)
+        assert_scores_close(out.cpu().numpy(), o, w.dtype)
+        assert int(err.item()) == 0
