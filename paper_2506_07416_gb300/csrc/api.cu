@@ -195,7 +195,6 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     const litevlm_select_config_t& c = h->cfg;
     const int hq = c.num_q_heads;
     const int mrows = max_t <= 64 ? 64 : 128;
-    const int slot_cols = (max_t + 15) & ~15;
     // the batch's tiles per request, largest first; the memo key hashes them
     int td_small[4096];
     int* td = td_small;
@@ -220,7 +219,6 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
         if (m.used && m.key == key) return ScoreChoice{m.resident, m.plan};
     const lvs::BatchTiles bt{td, batch};
 
-    const int cmax = lvs::res_max_cluster(row_bytes, slot_cols);
     const double hbm_bytes_per_us = 6.8e6;
     const double tile_bytes = (double)lvs::kTileRows * row_bytes;
     double tc_cost = 0.0;
@@ -255,10 +253,18 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     // partial-row workspace holds Hq rows, so a request's rows come in at most
     // Hq parts.
     const bool split = split_queries && max_t > 64 && !(c.flags & LITEVLM_FLAG_QUERY_LAST_TOKEN);
-    for (int qs = split ? 2 : 1; qs <= (split ? 2 : 1) && kflags != LITEVLM_FLAG_SCORE_REREAD; ++qs) {
+    // Head blocks as in the re-read kernel, up to the 64 rows that the costs were
+    // fitted on: a block streams its key head's tiles once (64 requests of 2309 to
+    // 3068 tokens, last-token queries, 32 / 8 heads: 251 -> 81 us; the re-read kernel,
+    // which takes the tiles twice, 98).
+    int hp_res = 1;
+    for (int d = 2; d <= hp; ++d)
+        if (G % d == 0 && d * max_t <= 64) hp_res = d;
+    const int qs = split ? 2 : 1;
+    for (int hr = 1; hr <= hp_res && kflags != LITEVLM_FLAG_SCORE_REREAD; hr = hr < hp_res ? hp_res : hp_res + 1) {
         const int mrows_r = qs == 2 ? 64 : mrows;
-        const int slot_r = qs == 2 ? (((max_t + 1) / 2 + 15) & ~15) : slot_cols;
-        const int hq_r = hq * qs;
+        const int slot_r = ((qs == 2 ? (max_t + 1) / 2 : hr * max_t) + 15) & ~15;
+        const int hq_r = hq * qs / hr;
         const int cmax = lvs::res_max_cluster(row_bytes, slot_r);
         int* rcap = h->res_capacity[mrows_r == 64 ? 0 : 1];
         for (int nb = 1; nb <= 2; ++nb) {
@@ -273,7 +279,7 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
                 int& cap = rcap[cl];
                 if (cap < 0) cap = lvs::res_cluster_capacity(row_bytes, fp8, mrows_r, cl);
                 if (cap <= 0) continue;
-                for (int g = 1; g <= hq; ++g) {
+                for (int g = 1; g <= hq_r && g <= hq; ++g) {
                     if (hq_r % g) continue;
                     const int hpg = hq_r / g;
                     if (nb == 2 && hpg < 2) continue;  // nothing to overlap
@@ -298,6 +304,7 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
                         lvs::ScorePlan pl{cl, tpc, g};
                         pl.res_nb = nb;
                         pl.qsplit = qs;
+                        pl.hp = hr;
                         best = ScoreChoice{true, pl};
                     }
                 }
@@ -343,6 +350,7 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
                     pl.res_nb = 1;
                     pl.flat = (int)nclu;
                     pl.qsplit = qs;
+                    pl.hp = hr;
                     best = ScoreChoice{true, pl};
                 }
             }
@@ -616,7 +624,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     p.c_log2 = (float)((double)q_scale * (double)k_scale / sqrt((double)c.head_dim) * 1.4426950408889634);
     p.wait_budget = h->wait_budget;
     p.stall = (h->debug_flags & LITEVLM_DEBUG_STALL_SCORE) != 0;
-    p.slot_cols = ((qsplit ? (max_t + 1) / 2 : max_t) + 15) & ~15;
+    p.slot_cols = ((qsplit ? (max_t + 1) / 2 : max_t * plan.hp) + 15) & ~15;
     p.qsplit = qsplit ? 2 : 1;
     p.query_last = (c.flags & LITEVLM_FLAG_QUERY_LAST_TOKEN) != 0;
     p.extra = nullptr;

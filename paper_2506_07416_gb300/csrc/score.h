@@ -26,11 +26,12 @@ struct ScoreLaunch {
     int32_t* err;
     int64_t total_vis;        // partial-row stride
     int32_t hq, hkv;
-    int32_t heads_per_group;  // (re-read kernel: head blocks)
+    int32_t heads_per_group;  // as scheduled (head blocks, pseudo-heads)
     int32_t groups;
-    // re-read kernel: query heads of one key head whose text rows share a
-    // contraction (a head block), and text rows per Q tile (instance rows / hp)
+    // query heads of one key head whose text rows share a contraction (a head
+    // block), and text rows per Q tile (instance rows / hp)
     int32_t hp, box_rows;
+    int32_t hqe;  // resident kernel: heads of a request as scheduled (pseudo-heads, head blocks)
     // re-read kernel without clusters: its CTAs share `items` (request, head
     // group) items; claims[0] counts those taken beyond a CTA's first, claims[1]
     // the CTAs that are done (zero between launches, workspace)
@@ -81,7 +82,7 @@ struct ScorePlan {
     int flat = 0;             // resident kernel: clusters of the flattened (request, head) schedule, 0: none
     int qsplit = 1;           // resident kernel: 2 = each head's text rows as two pseudo-heads (64-row kernel)
     int ctas = 0;             // re-read kernel without clusters: CTAs that run at once
-    int hp = 1;               // re-read kernel: query heads per head block
+    int hp = 1;               // query heads per head block
 };
 
 // The head groups' partial rows added up (re-read kernel with several groups).

@@ -146,7 +146,7 @@ __device__ __forceinline__ ResShape res_shape(const ScoreLaunch& p, int n0, int 
     r.N = n1 - n0;
     r.t0 = p.query_last && t1 > tq ? t1 - 1 : tq;  // last-token queries: one row
     r.T = t1 - r.t0;
-    r.Th = QS ? (r.T + 1) >> 1 : r.T;  // rows of the first (largest) pseudo-head
+    r.Th = QS ? (r.T + 1) >> 1 : r.T * p.hp;  // rows of the first (largest) pseudo-head; of a head block
     r.n2 = (r.Th + 15) & ~15;
     r.n_tiles = (r.N + kTileRows - 1) / kTileRows;
     const int tpc = r.N > 0 ? (r.n_tiles + (int)csize - 1) / (int)csize : 0;
@@ -196,10 +196,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const int fr0 = flat ? p.flat_r[item] : 0;
     const int nheads = flat ? p.flat_r[item + 1] - fr0 : p.heads_per_group;
     const int req_i = flat ? 0 : item / p.groups;
-    // heads of a request as scheduled (pseudo-heads with the query split); read
-    // from the parameters where it is used rather than held in a register
-#define LVS_HQE (QS ? 2 * p.hq : p.hq)
-    const int b = flat ? fr0 / LVS_HQE : (p.order_n > 0 ? (int)p.order[req_i] : req_i);
+    const int b = flat ? fr0 / p.hqe : (p.order_n > 0 ? (int)p.order[req_i] : req_i);
     const int hg = flat ? 0 : item - req_i * p.groups;
 
     // With the full-key-set terms (p.extra, written by the kernel launched just
@@ -259,6 +256,14 @@ __global__ void __launch_bounds__(kResThreads, 1)
         *abort_flag = 0;
         fence_mbar_init_cluster();
     }
+    // Q rows past the copied box (MROWS not a multiple of hp) are columns of weight
+    // 0: they must be numbers
+    for (int x = threadIdx.x; x < 2 * L::KB * (MROWS - p.hp * p.box_rows) * 8; x += kResThreads) {
+        const int rows = MROWS - p.hp * p.box_rows, blk = x / (rows * 8), o = x - blk * (rows * 8);
+        *reinterpret_cast<uint4*>(smem + L::OFF_Q + blk * MROWS * 128 + p.hp * p.box_rows * 128 + o * 16) =
+            make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async_shared();
+    }
     if (warp == 0 && lane == 0) {
         tma_prefetch_desc(&tm_q);
         tma_prefetch_desc(&tm_k);
@@ -300,9 +305,9 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const int tile_begin = shp.tile_begin;
     const int tile_end = tile_begin + shp.mt;
     const int mt = shp.mt;
-    // request, scheduled head (pseudo-head with the query split), query head,
-    // first visual row, first query row and query rows of head s of this CTA's
-    // sequence (with a flattened schedule the requests' rows follow one another
+    // request, scheduled head (pseudo-head with the query split, block of p.hp
+    // heads), (first) query head, first visual row, first text row and text rows of
+    // head s of this CTA's sequence (with a flattened schedule the requests' rows follow one another
     // at equal strides). With the query split, pseudo-head 2h + u of a request
     // holds the query rows [u * Th, min((u + 1) * Th, T)) of head h.
     struct HeadRef {
@@ -311,15 +316,15 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const int t_stride = t1 - tq;
     auto head_of = [&](int s_) -> HeadRef {
         if constexpr (!QS) {
-            if (!flat) return HeadRef{b, hg * hpg + s_, hg * hpg + s_, n0, t0, T};
-            const int rh = fr0 + s_, bb = rh / p.hq;
-            return HeadRef{bb, rh - bb * p.hq, rh - bb * p.hq, n0 + (bb - b) * N, t0 + (bb - b) * t_stride, T};
+            if (!flat) return HeadRef{b, hg * hpg + s_, (hg * hpg + s_) * p.hp, n0, t0, T};
+            const int rh = fr0 + s_, bb = rh / p.hqe, ph = rh - bb * p.hqe;
+            return HeadRef{bb, ph, ph * p.hp, n0 + (bb - b) * N, t0 + (bb - b) * t_stride, T};
         } else {
             int bb = b, ph = hg * hpg + s_, nn0 = n0, tt0 = t0;
             if (flat) {
                 const int rh = fr0 + s_;
-                bb = rh / LVS_HQE;
-                ph = rh - bb * LVS_HQE;
+                bb = rh / p.hqe;
+                ph = rh - bb * p.hqe;
                 nn0 = n0 + (bb - b) * N;
                 tt0 = t0 + (bb - b) * t_stride;
             }
@@ -347,7 +352,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 const int g = h / G;
                 const int qb = s & 1;
                 if (!wait_phase(BAR(Q_EMPTY + qb), ((s >> 1) & 1) ^ 1, ctl)) break;
-                mbar_arrive_expect_tx(BAR(Q_FULL + qb), L::Q_BYTES);
+                mbar_arrive_expect_tx(BAR(Q_FULL + qb), (uint32_t)(L::KB * 128 * p.hp * p.box_rows));
                 const uint32_t qdst = base + L::OFF_Q + qb * L::Q_BYTES;
 #pragma unroll
                 for (int kb = 0; kb < L::KB; ++kb)
@@ -660,7 +665,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
             // query rows of head s (with the query split, pseudo-heads alternate
             // halves: the parity of the request's pseudo-head index, which is the
             // parity of its index in the schedule since a request has an even count)
-            const int Ts = !QS ? T : ((((flat ? fr0 : hg * hpg) + s) & 1) ? T - Th : Th);
+            const int Ts = !QS ? Th : ((((flat ? fr0 : hg * hpg) + s) & 1) ? T - Th : Th);
             if (wt < WGC) {
                 const int col = c_begin + wt;
                 float wval = 0.f;
@@ -677,7 +682,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
                     if (p.extra) {
                         griddep_wait();
                         const HeadRef hs = head_of(s);
-                        b = log2_add(b, p.extra[(int64_t)(hs.t0 + col) * p.hq + hs.h]);
+                        b = log2_add(b, QS ? p.extra[(int64_t)(hs.t0 + col) * p.hq + hs.h]
+                                           : p.extra[(int64_t)(hs.t0 + col / p.hp) * p.hq + hs.h + col % p.hp]);
                     }
                     float mloc = smax[wt];  // this CTA's column max: the e values' reference
 #pragma unroll
@@ -737,7 +743,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
         // final scores; otherwise this cluster's partial rows, folded by the last
         // of the request's clusters to finish each tile (fixed part order).
         auto flush = [&](const HeadRef& hr) {
-            const int first = hr.b * LVS_HQE, last = first + LVS_HQE - 1;
+            const int first = hr.b * p.hqe, last = first + p.hqe - 1;
             const bool whole = first >= fr0 && last < fr0 + nheads;
             auto cluster_of = [&](int pair) {  // the cluster whose range holds the pair
                 int lo = 0, hi = p.flat_n - 1;
@@ -778,7 +784,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 back(s);
                 if (flat) {
                     const HeadRef hr = head_of(s);
-                    if (s == nheads - 1 || hr.ph == LVS_HQE - 1) flush(hr);
+                    if (s == nheads - 1 || hr.ph == p.hqe - 1) flush(hr);
                 }
             }
         }
@@ -811,7 +817,6 @@ __global__ void __launch_bounds__(kResThreads, 1)
     // has completed on this CTA's barriers before its epilogue ends; no peer
     // reads this CTA's memory, so the arrival needs no release.
     cluster_sync_relaxed();
-#undef LVS_HQE
 }
 
 template <int ROW_BYTES, bool FP8, int MROWS, bool COMPACT, bool QS>
@@ -913,12 +918,15 @@ cudaError_t launch_score_resident(const CUtensorMap& tm_q, const CUtensorMap& tm
     q.res_nb = plan.res_nb;
     q.groups = plan.groups;
     q.qsplit = plan.qsplit;
-    q.heads_per_group = p.hq * plan.qsplit / plan.groups;
+    q.hp = plan.hp;
+    q.box_rows = mrows / plan.hp;
+    q.hqe = p.hq * plan.qsplit / plan.hp;
+    q.heads_per_group = q.hqe / plan.groups;
     q.ctas_per_request = plan.cluster * plan.groups;
     q.flat_n = 0;
     if (plan.flat > 0) {  // equal shares of the batch's (request, head) pairs, in request-major order
         if (plan.flat > kFlatMax || plan.res_nb != 1) return cudaErrorInvalidValue;
-        const long long pairs = (long long)batch * p.hq * plan.qsplit;
+        const long long pairs = (long long)batch * q.hqe;
         q.flat_n = plan.flat;
         for (int k = 0; k <= plan.flat; ++k) q.flat_r[k] = (int32_t)(pairs * k / plan.flat);
         q.order_n = 0;

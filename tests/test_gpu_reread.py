@@ -63,9 +63,35 @@ def test_rows_tiles_and_groups(sel, w):
     s.close()
 
 
+RESIDENT = [
+    (_w("rows_63", [300, 129], [9, 4], 7, 1), "resident"),          # hp 7: one row of the 64 is no head's
+    (_w("rows_64", [513, 40, 1200], [16, 7, 1], 16, 4), "resident"),
+    (_w("rows_64_uniform", [1500] * 9, [16] * 9, 8, 2), "resident_flat"),
+    (_w("rows_8_d64", [700, 128], [1, 1], 16, 2, d=64), "resident_1buf"),
+    (_w("rows_60_two_buffers", [900, 257, 1], [15, 8, 3], 16, 4), "resident_2buf"),
+    (_w("rows_48_e4m3", [400, 1290], [16, 3], 12, 4, dtype="e4m3"), "resident"),
+    (_w("not_packed", [400, 1290], [33, 3], 12, 4), "resident"),
+]
+
+
+@pytest.mark.parametrize("w,kernel", RESIDENT, ids=[w.name for w, _ in RESIDENT])
+def test_packed_heads_in_the_resident_kernel(sel, w, kernel):
+    x = inputs.make_numpy(w)
+    xd = to_device(x, w)
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel=kernel)
+    assert s.score_plan(x["text_offsets"], x["seq_offsets"])[0] >= 2
+    o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, w.head_dim, w.dtype,
+                     x["q_scale"], x["k_scale"])
+    g = _scores(s, x, xd)
+    assert_scores_close(g, o, w.dtype)
+    np.testing.assert_array_equal(g, _scores(s, x, xd))
+    s.close()
+
+
+@pytest.mark.parametrize("kernel", ["reread", "resident"])
 @pytest.mark.parametrize("query", ["all", "last"])
-@pytest.mark.parametrize("t", [[18, 7], [30, 11]])
-def test_packed_heads_with_the_full_key_set(sel, t, query):
+@pytest.mark.parametrize("t", [[18, 7], [30, 11], [9, 3]])
+def test_packed_heads_with_the_full_key_set(sel, t, query, kernel):
     w = _w("packed_full", [300, 150], t, 14, 2)
     x = inputs.make_numpy(w)
     xd = to_device(x, w)
@@ -73,7 +99,7 @@ def test_packed_heads_with_the_full_key_set(sel, t, query):
     c = inputs.context_keys_numpy(w, n_sys, seed=24)
     dev = lambda a: torch.from_numpy(a.view(np.int16).copy()).view(torch.bfloat16).cuda()
     sys_off = np.concatenate([[0], np.cumsum(n_sys)]).astype(np.int32)
-    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel="reread",
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel=kernel,
                      query=query)
     out = s.score_full_keys(xd["q"], xd["text_offsets"], xd["k"], xd["seq_offsets"], dev(c["k_sys"]),
                             torch.from_numpy(sys_off).cuda(), dev(c["k_txt"]), seq_offsets_h=x["seq_offsets"],
