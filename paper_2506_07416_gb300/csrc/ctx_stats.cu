@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kCtxThreads) ctx_stats_kernel(const CtxArgs a)
     const int b = (int)blockIdx.x / a.hq;
     const int h = (int)blockIdx.x - b * a.hq;
     const int g = h / (a.hq / a.hkv);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
 
     griddep_wait();
     griddep_launch_dependents();
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kCtxThreads) ctx_stats_kernel(const CtxArgs a)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
     const Ctl ctl{abort_flag, a.err, a.wait_budget};
     const float cl = a.c_log2;
 
@@ -154,17 +154,20 @@ __global__ void __launch_bounds__(kCtxThreads) ctx_stats_kernel(const CtxArgs a)
         cp_async_wait_all();
         fence_proxy_async_shared();  // the copies' writes -> visible to the tensor core
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
             tc_fence_after();
-            const uint32_t idesc = idesc_make(kCtxQRows, (uint32_t)N, FMT);
+            const uint32_t idesc = idesc_make(kCtxQRows, (uint32_t)uniform(N), FMT);
+            if (elect_one()) {
 #pragma unroll
-            for (int st = 0; st < KSTEPS; ++st) {
-                const uint64_t ad = sdesc_k_sw128(sA + (st >> 2) * (kCtxQRows * 128) + (st & 3) * 32);
-                const uint64_t bd = sdesc_k_sw128(sB + (st >> 2) * (kCtxKeys * 128) + (st & 3) * 32);
-                if (FP8) mma_f8(tmem, ad, bd, idesc, st > 0);
-                else mma_f16(tmem, ad, bd, idesc, st > 0);
+                for (int st = 0; st < KSTEPS; ++st) {
+                    const uint64_t ad = sdesc_k_sw128(sA + (st >> 2) * (kCtxQRows * 128) + (st & 3) * 32);
+                    const uint64_t bd = sdesc_k_sw128(sB + (st >> 2) * (kCtxKeys * 128) + (st & 3) * 32);
+                    if (FP8) mma_f8(tmem, ad, bd, idesc, st > 0);
+                    else mma_f16(tmem, ad, bd, idesc, st > 0);
+                }
+                mma_commit(bar);
             }
-            mma_commit(bar);
+            __syncwarp();
         }
         ++issued;
         wait_phase(bar, (uint32_t)kt & 1u, ctl);
