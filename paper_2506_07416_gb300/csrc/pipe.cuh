@@ -185,12 +185,13 @@ __device__ __forceinline__ void col_sum_exp16(const float* v, float2 cl2, const 
     }
 }
 
-// (m, l) += (mo, lo): two sums of 2^((s - reference) * c) of one row under the larger reference
-__device__ __forceinline__ void merge_row(float& m, float& l, float mo, float lo, float cl)
+// (m, l) += (mo, lo): two sums of 2^(s * c - m) of one row, references m in units of log2,
+// under the larger reference
+__device__ __forceinline__ void merge_row(float& m, float& l, float mo, float lo)
 {
     const float mm = fmaxf(m, mo);
     if (mm != -INFINITY) {
-        l = (l > 0.f ? l * ex2((m - mm) * cl) : 0.f) + (lo > 0.f ? lo * ex2((mo - mm) * cl) : 0.f);
+        l = (l > 0.f ? l * ex2(m - mm) : 0.f) + (lo > 0.f ? lo * ex2(mo - mm) : 0.f);
         m = mm;
     }
 }
@@ -203,10 +204,10 @@ __device__ __forceinline__ float log2_add(float x, float y)
     return mx + __log2f(1.f + ex2(mn - mx));
 }
 
-// Merges the (max, sum) partials of one row from every CTA of the cluster in
-// rank order and returns b = M * c + log2(L). All remote loads are issued
+// Merges the (reference, sum) partials of one row from every CTA of the cluster in
+// rank order and returns b = M + log2(L). All remote loads are issued
 // before any is used, so their latencies overlap.
-__device__ __forceinline__ float merge_cluster_row(uint32_t my_addr, uint32_t csize, float cl)
+__device__ __forceinline__ float merge_cluster_row(uint32_t my_addr, uint32_t csize)
 {
     float2 st[kMaxCluster];
 #pragma unroll
@@ -219,8 +220,8 @@ __device__ __forceinline__ float merge_cluster_row(uint32_t my_addr, uint32_t cs
     float L = 0.f;
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r)
-        if (r < (int)csize && st[r].y > 0.f) L += st[r].y * ex2((st[r].x - M) * cl);
-    return fmaf(M, cl, __log2f(L));
+        if (r < (int)csize && st[r].y > 0.f) L += st[r].y * ex2(st[r].x - M);
+    return M + __log2f(L);
 }
 
 // Ticket slot of tile t of the request starting at row n0 (request b): unique

@@ -569,9 +569,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                             ld_masked(c, v);
                             m = fmaxf(m, row_max<32>(v));
                         }
-                        const float f = ref == -INFINITY ? 0.f : ex2((ref - m) * cl);
+                        const float nr = m == -INFINITY ? 0.f : -(m * cl);
+                        const float f = ref == -INFINITY ? 0.f : ex2(nr - nrc);
                         ref = m;
-                        nrc = m == -INFINITY ? 0.f : -(m * cl);
+                        nrc = nr;
                         s01 = make_float2(o01.x * f, o01.y * f);
                         s23 = make_float2(o23.x * f, o23.y * f);
                         sum_masked();
@@ -598,12 +599,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tile([&](int c, float* v) { tmem_ld16x2_32<64>(ta + (uint32_t)c, v); }, Blocks<1>{}, ub,
                              left - (lane >> 4) * 64, first, full);
                 }
-                float m = ref, l = (s01.x + s01.y) + (s23.x + s23.y);
+                // the statistics' maximum in units of log2, as the sums used it: rounded once
+                float m = ref == -INFINITY ? ref : -nrc, l = (s01.x + s01.y) + (s23.x + s23.y);
                 if (m64) {
                     // merge the two column parts of each row (threads t and t ^ 16)
                     const float mo = __shfl_xor_sync(0xffffffffu, m, 16);
                     const float lo = __shfl_xor_sync(0xffffffffu, l, 16);
-                    merge_row(m, l, mo, lo, cl);
+                    merge_row(m, l, mo, lo);
                 }
                 // ---- merge the warpgroups, publish (m, l) of head s to the cluster
                 const bool writer = !m64 || lane < 16;
@@ -617,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                         for (int o_wg = 1; o_wg < kEpiWG; ++o_wg) {  // fixed order: deterministic
                             const float2 o = xs[(o_wg - 1) * kMaxText + prow];
-                            merge_row(m, l, o.x, o.y, cl);
+                            merge_row(m, l, o.x, o.y);
                         }
                         stats_s[((hc + s) % kStatSlots) * kMaxText + prow] = make_float2(m, l);
                     }
@@ -642,10 +644,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (et < R) {
                         float bm;
                         if (csize > 1) {
-                            bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + et) * 8u, csize, cl);
+                            bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + et) * 8u, csize);
                         } else {
                             const float2 st = stats_s[slot * kMaxText + et];
-                            bm = fmaf(st.x, cl, __log2f(st.y));
+                            bm = st.x + __log2f(st.y);
                         }
                         if (p.extra) {
                             griddep_wait();
