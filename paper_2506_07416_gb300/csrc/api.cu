@@ -240,6 +240,15 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     ScoreChoice best{false, lvs::plan_score(bt, hq / hp, c.num_kv_heads, row_bytes, tcap, tc_costs,
                                             limit_rule ? 2.0 : 1.0, &tc_cost)};
     best.plan.hp = hp;
+    // Four epilogue warpgroups for e4m3 without clusters from 12 tiles a request on:
+    // its contractions leave the epilogue's latency as the pace (32 requests of 5 to 27
+    // tiles, 32 heads: 105.6 -> 98.7 us; 8 of 4 to 25: 31.9 -> 30.9; 64 of 18 to 24,
+    // last token: 68.5 -> 67.0), while on shorter requests the wider barriers cost more (64
+    // of 4 to 10 tiles: 75.7 against 79.3 us; 1 to 6: 51.1 against 58.3) and bf16 gains
+    // nothing (12 of 3 to 20: 37.5 against 38.6).
+    long long tiles = 0;
+    for (int b = 0; b < batch; ++b) tiles += td[b];
+    best.plan.wide = fp8 && best.plan.cluster == 1 && tiles >= 12ll * batch;
     double best_cost = limit_rule ? tc_cost : tc_cost / 0.9;
     const int max_tiles = batch > 0 ? td[0] : 0;
     const bool split_queries = (c.flags & LITEVLM_FLAG_SCORE_SPLIT_QUERIES) != 0;

@@ -83,6 +83,7 @@ struct ScorePlan {
     int qsplit = 1;           // resident kernel: 2 = each head's text rows as two pseudo-heads (64-row kernel)
     int ctas = 0;             // re-read kernel without clusters: CTAs that run at once
     int hp = 1;               // query heads per head block
+    bool wide = false;        // re-read kernel, e4m3: four epilogue warpgroups
 };
 
 // The head groups' partial rows added up (re-read kernel with several groups).

@@ -65,6 +65,9 @@
 // kept a warp from overlapping one block's sums with the next one's exponents and
 // cost 40% (P1 work per tile of two warps of an SM quarter: 1900 cycles, 1230 is
 // the exponential unit's share).
+// For e4m3 on long requests (choose_score_kernel has the line) an instance with four
+// warpgroups, blocks of 32 columns and 96 registers: its contractions take half as
+// long, and more warps hide the epilogue's latency (105.6 -> 98.7 us).
 // Every wait is bounded (clock budget); on expiry the kernel sets the error
 // word, drains its own copies and MMAs, frees TMEM and returns.
 
@@ -78,9 +81,6 @@ namespace lvs {
 
 namespace {
 
-constexpr int kEpiWG = 2;                    // epilogue warpgroups
-constexpr int kEpiThreads = 128 * kEpiWG;
-constexpr int kThreads = 96 + kEpiThreads;
 constexpr int kStatSlots = 4;  // stats of heads s-3..s may be live across the cluster
 template <int N>
 struct Blocks {
@@ -92,7 +92,7 @@ constexpr float kSumLimit = 7.9e28f;  // about 2^96: a pass-1 sum beyond moves i
 // Q double buffer and the bookkeeping; every variant needs more than half of
 // the SM's shared memory, so a single CTA (and a single 512-column TMEM
 // allocation) lives on an SM at a time.
-template <int ROW_BYTES, int MROWS>
+template <int ROW_BYTES, int MROWS, int kEpiWG>
 struct SmemLayout {
     static constexpr int KB = ROW_BYTES / 128;             // 128-byte swizzle blocks along d
     static constexpr int TILE_BYTES = kTileRows * ROW_BYTES;
@@ -137,12 +137,16 @@ struct TcWork {
     bool m64;
 };
 
-template <int ROW_BYTES, bool FP8, int MROWS>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int kEpiWG>
+constexpr int kThreadsOf = 96 + 128 * kEpiWG;
+
+template <int ROW_BYTES, bool FP8, int MROWS, int kEpiWG>
+__global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
     score_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ ScoreLaunch p)
 {
-    using L = SmemLayout<ROW_BYTES, MROWS>;
+    using L = SmemLayout<ROW_BYTES, MROWS, kEpiWG>;
+    constexpr int kEpiThreads = 128 * kEpiWG, kThreads = kThreadsOf<kEpiWG>;
     constexpr int KSTEPS = ROW_BYTES / 32;                 // one MMA consumes 32 bytes of d
     constexpr int ELEMS_PER_KB = FP8 ? 128 : 64;           // elements in 128 bytes
     constexpr uint32_t FMT = FP8 ? 0u : 1u;
@@ -477,6 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int quad = warp & 3;
         const int wg = (warp - 3) >> 2;                       // 0 .. kEpiWG - 1
         const int et = threadIdx.x - 96;                      // 0 .. kEpiThreads - 1
+        const int wt = et & 127;
         const int vrow = quad * 32 + lane;                    // pass 2: TMEM lane = visual token in tile
         const uint32_t tcol = tmem + ((uint32_t)(quad * 32) << 16);
         const float2 cl2 = make_float2(cl, cl);
@@ -510,6 +515,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int n0 = w.n0, N = w.N, t0 = w.t0, T = w.T, R = w.R, n2 = w.n2, mt = w.mt, hg = w.hg;
         const int tile_begin = w.tile_begin, tile_end = w.tile_end;
         const bool m64 = w.m64;
+        // The units of an item come in pairs, so with four warpgroups its first may
+        // belong to warpgroup 2: roles and the order of the merge below follow the
+        // item's first unit, and its scores do not depend on the items before it.
+        const int lead = kEpiWG == 4 ? (int)(ui & 3u) : 0;
+        const int rwg = (wg - lead) & (kEpiWG - 1);
         // pass 1 row of this thread: M = 128 -> lane; M = 64 -> lanes 16q..16q+15, two
         // column halves
         const int prow = !m64 ? quad * 32 + lane : quad * 16 + (lane & 15);
@@ -548,7 +558,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float2 o01 = s01, o23 = s23;
                     if (full) {
 #pragma unroll
-                        for (int k = 0; k < NB; ++k) {
+                        for (int k = 0; k < (kEpiWG == 4 ? 2 * NB : 0); ++k) {
+                            float v[32];
+                            ld(k * 32, v);
+                            tmem_wait_ld();
+                            row_sum_exp<32>(v, cl2, make_float2(nrc, nrc), s01, s23);
+                        }
+#pragma unroll
+                        for (int k = 0; k < (kEpiWG == 4 ? 0 : NB); ++k) {
                             float va[32], vb[32];
                             ld(k * 64, va);
                             ld(k * 64 + 32, vb);
@@ -612,9 +629,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // (double-buffered by head: the other warpgroups may publish head s + 1
                 // while the first one is still reading head s)
                 float2* xs = xs_s + ((hc + s) & 1) * (kEpiWG - 1) * kMaxText;
-                if (wg > 0 && writer) xs[(wg - 1) * kMaxText + prow] = make_float2(m, l);
+                if (rwg > 0 && writer) xs[(rwg - 1) * kMaxText + prow] = make_float2(m, l);
                 named_bar_sync(1, kEpiThreads);
-                if (wg == 0) {
+                if (rwg == 0) {
                     if (writer) {
 #pragma unroll
                         for (int o_wg = 1; o_wg < kEpiWG; ++o_wg) {  // fixed order: deterministic
@@ -629,8 +646,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // threads wrote before the named barrier, and the arrivals'
                     // fences (each waits for this SM's memory traffic to settle)
                     // overlap instead of running one after another
-                    if (csize > 1 && et < (int)csize)
-                        mbar_arrive_remote(mapa_shared(BAR(STATS + s % kStatSlots), (uint32_t)et));
+                    if (csize > 1 && wt < (int)csize)
+                        mbar_arrive_remote(mapa_shared(BAR(STATS + s % kStatSlots), (uint32_t)wt));
                 }
             }
             if (s >= lag) {
@@ -638,24 +655,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int hs = s - lag;
                 const int slot = (hc + hs) % kStatSlots;
                 float* b2 = b2_s + ((hc + hs) & 1) * kMaxText;
-                if (wg == 0) {
+                if (rwg == 0) {
                     // (a CTA that is its own cluster reads its own rows, ordered by the named barrier above)
                     if (csize > 1) poll_phase<true>(BAR(STATS + slot), (uint32_t)(hs / kStatSlots) & 1u, ctl);
-                    if (et < R) {
+                    if (wt < R) {
                         float bm;
                         if (csize > 1) {
-                            bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + et) * 8u, csize);
+                            bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + wt) * 8u, csize);
                         } else {
-                            const float2 st = stats_s[slot * kMaxText + et];
+                            const float2 st = stats_s[slot * kMaxText + wt];
                             bm = st.x + __log2f(st.y);
                         }
                         if (p.extra) {
                             griddep_wait();
-                            bm = log2_add(bm, p.extra[(int64_t)(t0 + et / hp) * p.hq + (hg * hpg + hs) * hp + et % hp]);
+                            bm = log2_add(bm, p.extra[(int64_t)(t0 + wt / hp) * p.hq + (hg * hpg + hs) * hp + wt % hp]);
                         }
-                        b2[et] = -bm;  // stored negated: the fma addend of pass 2
+                        b2[wt] = -bm;  // stored negated: the fma addend of pass 2
                     } else {
-                        b2[et] = -INFINITY;
+                        b2[wt] = -INFINITY;
                     }
                 }
                 named_bar_sync(1, kEpiThreads);
@@ -668,7 +685,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float2 a01 = make_float2(0.f, 0.f), a23 = make_float2(0.f, 0.f);
                     const uint32_t ta = tcol + ub * 128u;
 #pragma unroll
-                    for (int c0 = 0; c0 < MROWS; c0 += 64) {
+                    for (int c0 = 0; c0 < (kEpiWG == 4 ? MROWS : 0); c0 += 32) {
+                        if (n2 >= c0 + 32) {
+                            float v[32];
+                            tmem_ld32(ta + (uint32_t)c0, v);
+                            tmem_wait_ld();
+                            if (n2 == c0 + 32) release(ub);
+                            col_sum_exp16(v, cl2, b2 + c0, a01, a23);
+                            col_sum_exp16(v + 16, cl2, b2 + c0 + 16, a01, a23);
+                        } else if (n2 > c0) {  // the last 16
+                            float v[16];
+                            tmem_ld16(ta + (uint32_t)c0, v);
+                            tmem_wait_ld();
+                            release(ub);
+                            col_sum_exp16(v, cl2, b2 + c0, a01, a23);
+                        }
+                    }
+#pragma unroll
+                    for (int c0 = 0; c0 < (kEpiWG == 4 ? 0 : MROWS); c0 += 64) {
                         if (n2 >= c0 + 64) {  // a straight-line block of 64 columns
                             float va[32], vb[32];
                             tmem_ld32(ta + (uint32_t)c0, va);
@@ -753,28 +787,28 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const __grid_constan
     }
 }
 
-template <int ROW_BYTES, bool FP8, int MROWS>
+template <int ROW_BYTES, bool FP8, int MROWS, int kEpiWG = 2>
 cudaError_t tc_prepare(int cluster)
 {
-    auto kern = score_tc_kernel<ROW_BYTES, FP8, MROWS>;
+    auto kern = score_tc_kernel<ROW_BYTES, FP8, MROWS, kEpiWG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SmemLayout<ROW_BYTES, MROWS>::ALLOC);
+                                         SmemLayout<ROW_BYTES, MROWS, kEpiWG>::ALLOC);
     if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
 // CTAs resident at once with clusters of `cluster` CTAs (occupancy query)
-template <int ROW_BYTES, bool FP8, int MROWS>
+template <int ROW_BYTES, bool FP8, int MROWS, int kEpiWG = 2>
 int tc_capacity(int cluster)
 {
-    if (tc_prepare<ROW_BYTES, FP8, MROWS>(cluster) != cudaSuccess) {
+    if (tc_prepare<ROW_BYTES, FP8, MROWS, kEpiWG>(cluster) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster * 64, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = SmemLayout<ROW_BYTES, MROWS>::ALLOC;
+    cfg.blockDim = dim3(kThreadsOf<kEpiWG>, 1, 1);
+    cfg.dynamicSmemBytes = SmemLayout<ROW_BYTES, MROWS, kEpiWG>::ALLOC;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cluster;
@@ -783,27 +817,27 @@ int tc_capacity(int cluster)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, score_tc_kernel<ROW_BYTES, FP8, MROWS>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, score_tc_kernel<ROW_BYTES, FP8, MROWS, kEpiWG>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return n * cluster;
 }
 
-template <int ROW_BYTES, bool FP8, int MROWS>
+template <int ROW_BYTES, bool FP8, int MROWS, int kEpiWG = 2>
 cudaError_t launch_variant(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const ScoreLaunch& p,
                            const ScorePlan& plan, int batch, cudaStream_t stream)
 {
-    auto kern = score_tc_kernel<ROW_BYTES, FP8, MROWS>;
-    const int smem = SmemLayout<ROW_BYTES, MROWS>::ALLOC;
-    cudaError_t e = tc_prepare<ROW_BYTES, FP8, MROWS>(plan.cluster);
+    auto kern = score_tc_kernel<ROW_BYTES, FP8, MROWS, kEpiWG>;
+    const int smem = SmemLayout<ROW_BYTES, MROWS, kEpiWG>::ALLOC;
+    cudaError_t e = tc_prepare<ROW_BYTES, FP8, MROWS, kEpiWG>(plan.cluster);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     // clusters: one per item; without, as many CTAs as run at once, which share the items
     const int items = plan.groups * batch;
     const int ctas = plan.cluster > 1 ? plan.cluster * items : items < plan.ctas ? items : plan.ctas;
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(kThreadsOf<kEpiWG>, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -919,6 +953,9 @@ cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const
     q.items = plan.groups * batch;
     if (plan.cluster == 1 && plan.ctas < 1) return cudaErrorInvalidValue;
     if (fp8) {
+        if (plan.wide)
+            return mrows == 64 ? launch_variant<128, true, 64, 4>(tm_q, tm_k, q, plan, batch, stream)
+                               : launch_variant<128, true, 128, 4>(tm_q, tm_k, q, plan, batch, stream);
         return mrows == 64 ? launch_variant<128, true, 64>(tm_q, tm_k, q, plan, batch, stream)
                            : launch_variant<128, true, 128>(tm_q, tm_k, q, plan, batch, stream);
     }

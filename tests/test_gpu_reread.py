@@ -144,6 +144,29 @@ def test_logits_far_from_the_first_tiles_reference(sel, t, later):
     s.close()
 
 
+@pytest.mark.parametrize("n,t,hq,hkv", [
+    ([1537, 1700, 1410, 1664] * 8, [128, 33, 16, 65, 1], 16, 16),   # 128-row instance, all row counts in one batch
+    ([1537, 1700, 1410, 1664] * 10, [16, 9, 31], 64, 16),            # packed heads, 124 rows
+    ([1664, 3000, 129] * 10, [64, 17], 16, 16),                      # 64-row instance, 2-tile requests among them
+], ids=["rows_128", "packed", "rows_64"])
+def test_long_e4m3_requests(sel, n, t, hq, hkv):
+    """From 12 tiles a request on, e4m3 runs on four epilogue warpgroups."""
+    t = [t[i % len(t)] for i in range(len(n))]
+    w = _w("long_e4m3", n, t, hq, hkv, dtype="e4m3")
+    assert sum((x + 127) // 128 for x in n) >= 12 * len(n)
+    x = inputs.make_numpy(w)
+    xd = to_device(x, w)
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel="reread")
+    assert tuple(s.score_plan(x["text_offsets"], x["seq_offsets"])[:2]) == (1, 1)
+    o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, w.head_dim, w.dtype,
+                     x["q_scale"], x["k_scale"])
+    g = _scores(s, x, xd)
+    assert_scores_close(g, o, w.dtype)
+    for _ in range(4):  # whichever CTA takes an item, and behind whichever items, its scores are the same
+        np.testing.assert_array_equal(g, _scores(s, x, xd))
+    s.close()
+
+
 def test_no_alloc_limit_does_not_follow_the_plan(sel):
     """A batch whose chosen launch would need more partial rows than the static scratch holds, but whose fixed
     shape does not, is still taken."""
@@ -189,8 +212,10 @@ def test_more_items_than_ctas(sel, n, t, hq, hkv, d):
     assert plan[3] * w.batch > torch.cuda.get_device_properties(0).multi_processor_count
     o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, w.head_dim, w.dtype,
                      x["q_scale"], x["k_scale"])
-    for _ in range(3):
-        assert_scores_close(_scores(s, x, xd), o, w.dtype)
+    g = _scores(s, x, xd)
+    assert_scores_close(g, o, w.dtype)
+    for _ in range(2):  # whichever CTA takes an item, its scores are the same
+        np.testing.assert_array_equal(g, _scores(s, x, xd))
     s.close()
     err = torch.zeros(1, dtype=torch.int32, device="cuda")
     for _ in range(2):
