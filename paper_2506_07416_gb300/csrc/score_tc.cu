@@ -47,7 +47,8 @@
 // and the reference cancels in b. A thread takes the largest of the first 32
 // columns it sees, and moves it (to the larger maximum, rescaling its sum) only
 // when a sum passes 2^96, checked once per tile while the logits are still in
-// tensor memory. The loop is then one fused multiply-add (packed in
+// tensor memory. In units of log2 it is rounded to a whole number, so that sums
+// under two references are merged by a power of two, without error. The loop is then one fused multiply-add (packed in
 // pairs), one 2^x and one add (packed) per logit, in both passes.
 //
 // Warp roles (352 threads): warp 0 = TMA producer, warps 1 and 2 = MMA issuers
@@ -528,7 +529,7 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
         for (int s = 0; s < hpg + lag; ++s) {
             if (s < hpg) {
                 // ---- pass 1 of head s: row sums over this warpgroup's tiles
-                float ref = -INFINITY, nrc = 0.f;           // reference logit and -(ref * c)
+                float ref = -INFINITY, nrc = 0.f;           // reference logit and -(ref * c), a whole number
                 float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
                 // One tile: a row's columns (128; 64 with M = 64, the other 64 with the
                 // thread 16 lanes on), in blocks of 64; `ld` reads 32 columns from c.
@@ -553,7 +554,7 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
                         float v[32];
                         ld_masked(0, v);
                         ref = row_max<32>(v);
-                        nrc = ref == -INFINITY ? 0.f : -(ref * cl);
+                        nrc = ref == -INFINITY ? 0.f : -rintf(ref * cl);
                     }
                     const float2 o01 = s01, o23 = s23;
                     if (full) {
@@ -586,7 +587,7 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
                             ld_masked(c, v);
                             m = fmaxf(m, row_max<32>(v));
                         }
-                        const float nr = m == -INFINITY ? 0.f : -(m * cl);
+                        const float nr = m == -INFINITY ? 0.f : -rintf(m * cl);
                         const float f = ref == -INFINITY ? 0.f : ex2(nr - nrc);
                         ref = m;
                         nrc = nr;
@@ -616,7 +617,7 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
                         tile([&](int c, float* v) { tmem_ld16x2_32<64>(ta + (uint32_t)c, v); }, Blocks<1>{}, ub,
                              left - (lane >> 4) * 64, first, full);
                 }
-                // the statistics' maximum in units of log2, as the sums used it: rounded once
+                // the reference in units of log2, as the sums used it
                 float m = ref == -INFINITY ? ref : -nrc, l = (s01.x + s01.y) + (s23.x + s23.y);
                 if (m64) {
                     // merge the two column parts of each row (threads t and t ^ 16)
