@@ -364,11 +364,7 @@ __global__ void __launch_bounds__(kProjThreads, 1)
                 if (lane == 0) mbar_arrive_remote(mapa_shared(ACC_EMPTY(a & 1), 0));
                 continue;
             }
-            // four packed accumulators: two chains of 32 dependent adds a stage would
-            // take as long as the stage's contraction
-            float2 ss[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) ss[q] = make_float2(0.f, 0.f);
+            float2 ss = make_float2(0.f, 0.f);  // even and odd hidden values, each in order
             for (int kc = 0; kc < nk; ++kc, ++it) {
                 const int s = it % S;
                 if (!wait_phase(DONE(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
@@ -380,15 +376,22 @@ __global__ void __launch_bounds__(kProjThreads, 1)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const float2 x = make_float2(__uint_as_float(w4[q] << 16), __uint_as_float(w4[q] & 0xFFFF0000u));
-                        ss[q] = ffma2(x, x, ss[q]);
+                        ss = ffma2(x, x, ss);
                     }
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(EMPTY(s));
+                // Only this arrival keeps the next copy (async proxy) out of the stage
+                // while the loads above (generic proxy) read it. An arrival orders no
+                // proxies, and a load that has been issued but waits behind the stores of
+                // the epilogue warps would read the copy's bytes. So every lane orders its
+                // loads before the async proxy, and the arrival depends on a vote that
+                // needs every lane's sums, hence the values of all its loads (a sum of
+                // squares is never negative: the vote is always 0).
+                fence_proxy_async_shared();
+                const bool bad = __any_sync(0xffffffffu, ss.x < 0.f || ss.y < 0.f);
+                if (lane == 0 && !bad) mbar_arrive(EMPTY(s));
             }
             if (!ok || !wait_phase(SC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl)) break;
-            const float2 s01 = fadd2(ss[0], ss[1]), s23 = fadd2(ss[2], ss[3]);
-            sc_s[(a & 1) * kProjRows + r] = rsqrtf(((s01.x + s01.y) + (s23.x + s23.y)) / (float)p.hidden + p.eps);
+            sc_s[(a & 1) * kProjRows + r] = rsqrtf((ss.x + ss.y) / (float)p.hidden + p.eps);
             __syncwarp();
             if (lane == 0) mbar_arrive(SC_FULL(a & 1));
             if (last) store_tile(t, a, 1, 2);

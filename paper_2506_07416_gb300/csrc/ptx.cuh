@@ -75,8 +75,9 @@ __device__ __forceinline__ void fence_mbar_init_cluster()
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// orders this thread's earlier shared-memory writes (generic proxy) before its
-// later bulk-copy operations (async proxy)
+// orders this thread's earlier shared-memory accesses (generic proxy) before later
+// operations of the async proxy (bulk copies, contractions), its own and those that
+// a barrier orders behind it
 __device__ __forceinline__ void fence_proxy_async_shared()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -78,6 +78,43 @@ def test_project_tile_edges(sel, rows, hidden, out_f, head_dim, bias):
     _run(sel, rows, hidden, out_f, head_dim, bias)
 
 
+@pytest.mark.parametrize("rows,hidden,out_f,head_dim", [
+    (9001, 3584, 4096, 0),     # 8 tiles a pair, no rotation: the stores of a tile run beside the sums of the next
+    (2810, 4096, 3584, 128),   # 3 tiles a pair
+    (6000, 1024, 640, 64),     # 128-column tiles
+])
+def test_project_row_scales_over_several_tiles(sel, rows, hidden, out_f, head_dim):
+    """Pairs that work through several tiles, each of more stages than the ring holds: runs agree bit for bit, and no
+    row scale of any (row, tile) is off. The factor between a row's outputs in a tile (N of them) and their fp64
+    values is 1 but for the rounding to bf16, which spreads it by 0.8e-3 / sqrt(N / 3) (relative rounding errors of
+    0.8e-3 rms, weights y^2 of a normal y): 9e-5 for 256 columns and 1.2e-4 for 128. The bound is 6 times that; one
+    stage of 64 hidden values replaced by others in a sum of 4096 squares moves the factor by 1.4e-3 rms."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows)
+    x = torch.randn(rows, hidden, generator=gen, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(out_f, hidden, generator=gen, device="cuda") / math.sqrt(hidden)).to(torch.bfloat16)
+    pos = torch.randint(0, 4096, (rows,), generator=gen, device="cuda", dtype=torch.int32) if head_dim else None
+    table = sel.rope_table(4096, head_dim, 1e4) if head_dim else None
+    ys = [sel.project(x, w, None, 1e-6, head_dim, pos, table) for _ in range(4)]
+    sel.check_device()
+    for y in ys[1:]:
+        assert torch.equal(y, ys[0])
+    cols = 256 if out_f % 256 == 0 else 128
+    worst = 0.0
+    for r0 in range(0, rows, 3000):
+        xd = x[r0:r0 + 3000].double()
+        z = torch.rsqrt((xd * xd).mean(dim=1, keepdim=True) + 1e-6) * (xd @ w.double().t())
+        if head_dim:
+            cs = table[pos[r0:r0 + 3000].long()].double()
+            c, s = cs[:, None, :, 0], cs[:, None, :, 1]
+            z = z.view(-1, out_f // head_dim, 2, head_dim // 2)
+            z = torch.stack([z[:, :, 0] * c - z[:, :, 1] * s, z[:, :, 1] * c + z[:, :, 0] * s], dim=2)
+        z = z.reshape(-1, out_f // cols, cols)
+        y = ys[0][r0:r0 + 3000].double().view_as(z)
+        worst = max(worst, float(((z * y).sum(dim=2) / (z * z).sum(dim=2) - 1).abs().max()))
+    assert worst < 6 * 0.8e-3 / math.sqrt(cols / 3), worst
+
+
 def test_project_fold_is_w_times_gamma(sel):
     """fold_norm alone: bit-exact bf16(w * gamma) (one fp32 product, rounded once)."""
     rng = np.random.Generator(np.random.PCG64(3))
