@@ -317,7 +317,9 @@ __global__ void __launch_bounds__(kProjThreads, 1)
                 if (ok && elect_one()) mma_commit_pair(ACC_FULL(a & 1));
                 __syncwarp();
             }
-            if (elect_one()) mma_commit_pair(DRAIN);  // every contraction above has landed once this arrives
+            // Every contraction above has landed once this arrives. It arrives here alone:
+            // nobody in the other CTA would wait for it before leaving.
+            if (elect_one()) mma_commit_pair(DRAIN, 1);
             __syncwarp();
             wait_phase_warp(DRAIN, 0, drain);
         }

@@ -399,12 +399,13 @@ __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, u
         : "memory");
 }
 
-// arrive (once) on the mbarrier at this offset in both CTAs when all prior pair contractions of this thread complete
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar)
+// arrive (once) on the mbarrier at this offset in the CTAs of the mask (both of the
+// pair) when all prior pair contractions of this thread complete
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t ctas = 3)
 {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-        "h"((uint16_t)3)
+        "h"(ctas)
         : "memory");
 }
 
