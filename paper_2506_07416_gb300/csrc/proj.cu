@@ -346,7 +346,9 @@ __global__ void __launch_bounds__(kProjThreads, 1)
         w.buf = smem + L::OFF_ROPE + (warp - 2) * 4096;
         w.half = p.head_dim / 2;
         w.lane = lane;
-        // part `part` of `parts` of tile t, the a-th of this pair
+        // part `part` of `parts` of tile t, the a-th of this pair. A warp agrees on what
+        // its waits found, here and below: a lane that gave up alone would leave the
+        // others at their shuffles and aligned loads.
         auto store_tile = [&](int t, int a, int part, int parts) -> bool {
             const int64_t grow = (int64_t)(t / ntn) * (2 * kProjRows) + rank * kProjRows + r;
             if (p.head_dim > 0) {
@@ -357,22 +359,22 @@ __global__ void __launch_bounds__(kProjThreads, 1)
                 }
                 w.fetch(w.half / 16 / parts * part);
             }
-            bool ok = wait_phase(SC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl);
+            if (!wait_phase_warp(SC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl)) return false;
             const float sc = sc_s[(a & 1) * kProjRows + r];
             __syncwarp();
             if (wg == 0 && lane == 0) mbar_arrive(SC_EMPTY(a & 1));
-            ok = wait_phase(ACC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl) && ok;
+            if (!wait_phase_warp(ACC_FULL(a & 1), (uint32_t)(a >> 1) & 1u, ctl)) return false;
             tc_fence_after();
             proj_store_row<BN>(p, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((a & 1) * BN), grow, t % ntn * BN,
-                               part, parts, ok && grow < p.rows, sc, w);
-            return ok;
+                               part, parts, grow < p.rows, sc, w);
+            return true;
         };
         int it = 0, a = 0;
         bool ok = true;
         for (int t = pair; t < ntiles && ok; t += npairs, ++a) {
             const bool last = t + npairs >= ntiles;
             if (wg == 0) {
-                ok = store_tile(t, a, 0, last ? 2 : 1);
+                if (!store_tile(t, a, 0, last ? 2 : 1)) break;
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_remote(mapa_shared(ACC_EMPTY(a & 1), 0));
@@ -381,7 +383,7 @@ __global__ void __launch_bounds__(kProjThreads, 1)
             float2 ss = make_float2(0.f, 0.f);  // even and odd hidden values, each in order
             for (int kc = 0; kc < nk; ++kc, ++it) {
                 const int s = it % S;
-                if (!wait_phase(DONE(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
+                if (!wait_phase_warp(DONE(s), (uint32_t)(it / S) & 1u, ctl)) { ok = false; break; }
                 const uint8_t* row = smem + L::OFF_A + s * L::A_BYTES + r * 128;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
@@ -404,7 +406,7 @@ __global__ void __launch_bounds__(kProjThreads, 1)
                 const bool bad = __any_sync(0xffffffffu, ss.x < 0.f || ss.y < 0.f);
                 if (lane == 0 && !bad) mbar_arrive(EMPTY(s));
             }
-            if (!ok || !wait_phase(SC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl)) break;
+            if (!ok || !wait_phase_warp(SC_EMPTY(a & 1), ((uint32_t)(a >> 1) & 1u) ^ 1u, ctl)) break;
             sc_s[(a & 1) * kProjRows + r] = rsqrtf((ss.x + ss.y) / (float)p.hidden + p.eps);
             __syncwarp();
             if (lane == 0) mbar_arrive(SC_FULL(a & 1));
