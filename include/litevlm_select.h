@@ -457,11 +457,16 @@ litevlm_status_t litevlm_select_set_wait_budget(litevlm_select_t handle, int64_t
  * wait runs out of the wait budget before any copy or contraction is issued;
  * every other wait of the launch then gives up as well. The launch writes
  * invalid scores, and litevlm_select_check_device reports LITEVLM_ERR_TIMEOUT.
+ * LITEVLM_DEBUG_STALL_PROJECT: in the projection launches, the copies of every
+ * second CTA stop after three stages in the same way, so that the launch gives
+ * up with copies and contractions in flight and its CTAs at different stages;
+ * rows are invalid, and check_device reports LITEVLM_ERR_TIMEOUT.
  * Nothing faults, traps or hangs: each wait is bounded by the budget. flags = 0
  * restores normal operation. Errors: INVALID_ARG for a NULL handle or an
  * unknown flag.
  */
 #define LITEVLM_DEBUG_STALL_SCORE 1
+#define LITEVLM_DEBUG_STALL_PROJECT 4
 litevlm_status_t litevlm_select_set_debug_flags(litevlm_select_t handle, int32_t flags);
 
 /*

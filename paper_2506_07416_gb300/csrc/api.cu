@@ -1137,6 +1137,7 @@ litevlm_status_t litevlm_select_project(litevlm_select_t h, int64_t rows, int32_
     p.y = out_scale > 0.f ? nullptr : static_cast<__nv_bfloat16*>(y);
     p.y8 = out_scale > 0.f ? static_cast<uint8_t*>(y) : nullptr;
     p.out_inv_scale = out_scale > 0.f ? 1.f / out_scale : 0.f;
+    p.stall = (h->debug_flags & LITEVLM_DEBUG_STALL_PROJECT) != 0;
     p.err = h->err_d;
     p.wait_budget = h->wait_budget;
     const cudaError_t e = lvs::launch_proj(tm_x, tm_w, p, h->num_sms, (cudaStream_t)stream);
@@ -1217,7 +1218,7 @@ litevlm_status_t litevlm_select_set_debug_flags(litevlm_select_t h, int32_t flag
     const CallRange range_(__func__);
     if (!h) return LITEVLM_ERR_INVALID_ARG;
     h->last_error.clear();
-    if (flags & ~LITEVLM_DEBUG_STALL_SCORE) return fail(h, LITEVLM_ERR_INVALID_ARG, "unknown debug flag");
+    if (flags & ~(LITEVLM_DEBUG_STALL_SCORE | LITEVLM_DEBUG_STALL_PROJECT)) return fail(h, LITEVLM_ERR_INVALID_ARG, "unknown debug flag");
     h->debug_flags = flags;
     return LITEVLM_OK;
 }

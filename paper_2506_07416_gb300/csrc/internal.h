@@ -108,6 +108,7 @@ struct ProjArgs {
     __nv_bfloat16* y;         // [rows, O] bf16 output, or
     uint8_t* y8;              // [rows, O] e4m3 codes of y * out_inv_scale (null: bf16 output)
     float out_inv_scale;
+    int32_t stall;            // debug: a pair's second CTA stops after three stages
     int32_t* err;
     long long wait_budget;
 };

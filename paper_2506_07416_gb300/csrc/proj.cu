@@ -59,12 +59,20 @@ struct ProjLayout {
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + STAGES * A_BYTES;
     static constexpr int OFF_ROPE = OFF_B + STAGES * B_BYTES;  // 4 KB per epilogue warp
-    // full[S], done[S], empty[S], acc_full[2], acc_empty[2], sc_full[2], sc_empty[2], drain
+    // full[S], done[S], empty[S], acc_full[2], acc_empty[2], sc_full[2], sc_empty[2], drain, stall
     static constexpr int OFF_BAR = OFF_ROPE + 8 * 4096;
-    static constexpr int OFF_SC = OFF_BAR + (3 * STAGES + 9) * 8;  // [2][128] row scales
+    static constexpr int OFF_SC = OFF_BAR + (3 * STAGES + 10) * 8;  // [2][128] row scales
     static constexpr int OFF_MISC = OFF_SC + 2 * kProjRows * 4;
-    static constexpr int ALLOC = OFF_MISC + 16 + 1024;
+    // TMEM address, abort flag, the other CTA's; ProjCounts of this CTA and of the other
+    static constexpr int OFF_COUNTS = OFF_MISC + 16;
+    static constexpr int ALLOC = OFF_COUNTS + 2 * 16 + 1024;
     static constexpr int TMEM_COLS = 2 * BN;
+};
+
+// What a CTA of a pair had started when its roles ended: stages it copied, and (first
+// CTA) stages contracted and accumulators committed.
+struct ProjCounts {
+    int copied, contracted, tiles, unused;
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
@@ -235,10 +243,12 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     auto ACC_EMPTY = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + 2 + b); };
     auto SC_FULL = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + 4 + b); };
     auto SC_EMPTY = [&](int b) -> uint32_t { return bar0 + 8u * (uint32_t)(3 * S + 6 + b); };
-    const uint32_t DRAIN = bar0 + 8u * (uint32_t)(3 * S + 8);
+    const uint32_t DRAIN = bar0 + 8u * (uint32_t)(3 * S + 8), STALL = DRAIN + 8u;
     float* sc_s = reinterpret_cast<float*>(smem + L::OFF_SC);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 4);
+    volatile int* peer_abort = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 8);
+    volatile ProjCounts* counts = reinterpret_cast<volatile ProjCounts*>(smem + L::OFF_COUNTS);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -253,7 +263,10 @@ __global__ void __launch_bounds__(kProjThreads, 1)
             mbar_init(SC_EMPTY(b), 4);
         }
         mbar_init(DRAIN, 1);
+        mbar_init(STALL, 1);  // nothing ever arrives (the debug stall below)
         *abort_flag = 0;
+        *peer_abort = 0;
+        counts[0].copied = counts[0].contracted = counts[0].tiles = 0;
         fence_mbar_init_cluster();
     }
     if (warp == 0 && lane == 0) {
@@ -275,38 +288,46 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     griddep_wait();
     griddep_launch_dependents();
 
+    // this CTA's first rows of x and W' of tile t, and the copies of the tile's stage kc
+    // from there into slot s of the ring
+    auto x_row = [&](int t) { return t / ntn * (2 * kProjRows) + rank * kProjRows; };
+    auto w_row = [&](int t) { return t % ntn * BN + rank * (BN / 2); };
+    auto load_stage = [&](int s, int kc, int m0, int n0) {
+        const uint32_t full = mapa_shared(FULL(s), 0);
+        if (rank == 0) mbar_arrive_expect_tx(FULL(s), 2u * (uint32_t)L::STAGE);
+        tma_load_3d_pair(base + L::OFF_A + s * L::A_BYTES, &tm_x, full, kc * kProjK, 0, m0);
+        tma_load_3d_pair(base + L::OFF_B + s * L::B_BYTES, &tm_w, full, kc * kProjK, 0, n0);
+    };
+
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
             int it = 0;
             bool ok = true;
             for (int t = pair; t < ntiles && ok; t += npairs) {
-                const int m0 = t / ntn * (2 * kProjRows) + rank * kProjRows;
-                const int n0 = t % ntn * BN + rank * (BN / 2);
+                const int m0 = x_row(t), n0 = w_row(t);
                 for (int kc = 0; kc < nk; ++kc, ++it) {
                     const int s = it % S;
+                    // Debug stall (p.stall, a test of the failure path): a pair's second CTA
+                    // stops after three stages, so that the two give up with different counts
+                    // of copies and of contractions in flight.
+                    if (p.stall && rank == 1 && it == 3 && !wait_phase(STALL, 0, ctl)) { ok = false; break; }
                     if (!wait_phase(EMPTY(s), ((uint32_t)(it / S) & 1u) ^ 1u, ctl)) { ok = false; break; }
-                    const uint32_t full = mapa_shared(FULL(s), 0);
-                    if (rank == 0) mbar_arrive_expect_tx(FULL(s), 2u * (uint32_t)L::STAGE);
-                    tma_load_3d_pair(base + L::OFF_A + s * L::A_BYTES, &tm_x, full, kc * kProjK, 0, m0);
-                    tma_load_3d_pair(base + L::OFF_B + s * L::B_BYTES, &tm_w, full, kc * kProjK, 0, n0);
+                    load_stage(s, kc, m0, n0);
                 }
             }
             // every stage's last contraction has completed (and with it its copies),
             // its commit has arrived here and its rows are summed before this CTA leaves
             for (int s = 0; s < S && s < it && ok; ++s)
                 ok = wait_phase(EMPTY(s), (uint32_t)((it - 1 - s) / S) & 1u, ctl);
-            if (!ok) {  // after an abort: time enough for the copies in flight to land
-                const long long c0 = clock64();
-                while (clock64() - c0 < 1000000) {}
-            }
+            counts[0].copied = it;
         }
         __syncwarp();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (first CTA)
         if (rank == 0) {
             const uint32_t idesc = idesc_make(256, BN, 1u);
-            int it = 0, a = 0;
+            int it = 0, a = 0, tiles = 0;
             bool ok = true;
             for (int t = pair; t < ntiles && ok; t += npairs, ++a) {
                 const uint32_t d = tmem + (uint32_t)((a & 1) * BN);
@@ -326,14 +347,20 @@ __global__ void __launch_bounds__(kProjThreads, 1)
                     }
                     __syncwarp();
                 }
-                if (ok && elect_one()) mma_commit_pair(ACC_FULL(a & 1));
+                if (!ok) break;
+                if (elect_one()) mma_commit_pair(ACC_FULL(a & 1));
                 __syncwarp();
+                ++tiles;
             }
             // Every contraction above has landed once this arrives. It arrives here alone:
             // nobody in the other CTA would wait for it before leaving.
             if (elect_one()) mma_commit_pair(DRAIN, 1);
             __syncwarp();
             wait_phase_warp(DRAIN, 0, drain);
+            if (lane == 0) {
+                counts[0].contracted = it;
+                counts[0].tiles = tiles;
+            }
         }
         __syncwarp();
     } else {
@@ -415,7 +442,42 @@ __global__ void __launch_bounds__(kProjThreads, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) st_shared_cluster(mapa_shared(base + L::OFF_MISC + 8, rank ^ 1), 1);
+    __syncwarp();
     cluster_sync_all();  // both CTAs are done with each other's barriers and contractions
+    if (*abort_flag || *peer_abort) {
+        // A wait gave up in one of them: copies may be under way and arrivals
+        // outstanding that nobody waited for. The CTAs exchange what they started; the
+        // contractions of the first have completed (DRAIN).
+        const uint32_t to = mapa_shared(base + L::OFF_COUNTS + (uint32_t)sizeof(ProjCounts), rank ^ 1);
+        if (threadIdx.x == 0) {
+            st_shared_cluster(to, counts[0].copied);
+            st_shared_cluster(to + 4, counts[0].contracted);
+            st_shared_cluster(to + 8, counts[0].tiles);
+        }
+        __syncwarp();
+        cluster_sync_all();
+        if (threadIdx.x == 0) {
+            // A slot's barrier completes a phase when both CTAs have copied into it. They
+            // are at most a ring apart (a slot is refilled after a contraction over both),
+            // so the one behind copies what it lacks, into slots that no contraction reads
+            // any more. The phase before a slot's last was waited for when the slot was
+            // refilled, so the last one's parity decides; the same holds for the commits.
+            const int copied = max(counts[0].copied, counts[1].copied);
+            for (int it = counts[0].copied; it < copied; ++it) {
+                const int t = pair + it / nk * npairs;
+                load_stage(it % S, it % nk, x_row(t), w_row(t));
+            }
+            if (rank == 0)
+                for (int s = 0; s < S && s < copied; ++s) wait_phase(FULL(s), (uint32_t)((copied - 1 - s) / S) & 1u, drain);
+            const int contracted = counts[rank].contracted, tiles = counts[rank].tiles;
+            for (int s = 0; s < S && s < contracted; ++s)
+                wait_phase(DONE(s), (uint32_t)((contracted - 1 - s) / S) & 1u, drain);
+            for (int b = 0; b < 2 && b < tiles; ++b) wait_phase(ACC_FULL(b), (uint32_t)((tiles - 1 - b) / 2) & 1u, drain);
+        }
+        __syncwarp();
+        cluster_sync_all();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem, L::TMEM_COLS);

@@ -261,6 +261,11 @@ __device__ __forceinline__ float2 ld_shared_cluster_f2(uint32_t addr)
     return v;
 }
 
+__device__ __forceinline__ void st_shared_cluster(uint32_t addr, int v)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
 // ----------------------------------------------------------------------------
 // TMA
 // ----------------------------------------------------------------------------

@@ -302,6 +302,7 @@ def set_wait_budget(handle: int, cycles: int) -> None:
 
 
 DEBUG_STALL_SCORE = 1
+DEBUG_STALL_PROJECT = 4
 
 
 def set_debug_flags(handle: int, flags: int) -> None:

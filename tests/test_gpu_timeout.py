@@ -111,6 +111,41 @@ def test_wait_timeout_in_the_reread_kernel(sel):
     s.close()
 
 
+@pytest.mark.parametrize("rows,hidden,out_f,head_dim,stall", [
+    (2810, 4096, 3584, 128, True),   # 256-column tiles, 3 a pair: the first CTA a ring ahead of the second
+    (6000, 1024, 640, 64, True),     # 128-column tiles
+    (100, 200, 256, 0, True),        # one tile of 4 stages, less than a ring
+    (3000, 16384, 1024, 0, False),   # tiles of 256 stages (70 us) with a budget that lasts for a part of them
+])
+def test_wait_timeout_in_the_projection(sel, rows, hidden, out_f, head_dim, stall):
+    """The projection's failure path: waits of its epilogue, its sums, its copies and its contractions run out with
+    work in flight and the CTAs of a pair at different stages. The launch ends by itself and reports TIMEOUT, and
+    the same handle then gives the bits that it gave before. The call without a stall gives up wherever its waits
+    stand when they have lasted 20 to 40 us."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(hidden)
+    x = torch.randn(rows, hidden, generator=gen, device="cuda").to(torch.bfloat16)
+    w = torch.randn(out_f, hidden, generator=gen, device="cuda").to(torch.bfloat16)
+    s = sel.Selector(1, 128, 128, 1, 1, 128, "bf16")
+    pos = torch.randint(0, 512, (rows,), generator=gen, device="cuda", dtype=torch.int32) if head_dim else None
+    table = s.rope_table(512, head_dim, 1e4) if head_dim else None
+    want = s.project(x, w, None, 1e-6, head_dim, pos, table)
+    s.check_device()
+    for _ in range(3):
+        s.set_wait_budget(20000)
+        s.set_debug_flags(sel.DEBUG_STALL_PROJECT if stall else 0)
+        s.project(x, w, None, 1e-6, head_dim, pos, table)
+        with pytest.raises(sel.LitevlmError) as ei:
+            s.check_device()
+        assert ei.value.name == "TIMEOUT"
+        s.set_debug_flags(0)
+        s.set_wait_budget(0)
+        got = s.project(x, w, None, 1e-6, head_dim, pos, table)
+        s.check_device()
+        assert torch.equal(got, want)
+    s.close()
+
+
 def test_debug_setters_reject_bad_values(sel):
     s = sel.Selector(1, 128, 16, 4, 4, 64, "bf16")
     with pytest.raises(sel.LitevlmError) as ei:
