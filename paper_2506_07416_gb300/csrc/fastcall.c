@@ -2,9 +2,11 @@
  * Argument marshalling of the Python binding's hot calls, as a CPython extension
  * (paper_2506_07416_gb300/_fastcall.so). Each function takes the arguments of the
  * C function of the same name (include/litevlm_select.h) as Python objects:
- * device pointers as integers, objects with data_ptr() (torch tensors) or buffers
- * (numpy arrays), host offset arrays as int32 numpy arrays (anything else goes
- * through the binding's own conversion), and returns the status code. The GIL is
+ * pointers as integers, numpy arrays or objects with data_ptr() (torch tensors),
+ * host offset arrays as int32 numpy arrays (anything else goes through the binding's
+ * own conversion), handles and numbers as ctypes takes them, and returns the status
+ * code. No other object is a pointer, whatever memory it may show: the address of a
+ * numpy scalar or of a bytes object is not the value it holds. The GIL is
  * released around the call. The C functions' addresses come from the library that
  * the binding loaded (bind).
  *
@@ -23,6 +25,8 @@ static const char *const kSigs[F_COUNT] = {"hippnppnffph", "hippnppnppnpffph", "
                                            "", "hippnppnppnppnlpppph", "hliipppfippifph", ""};
 static void *g_fn[F_COUNT];
 static PyObject *g_host_i32;      /* the binding's conversion of a host offset array */
+static PyObject *g_ndarray;       /* numpy.ndarray */
+static PyObject *g_ctypes_value;  /* the value of a ctypes object of a signature's kind */
 static PyObject *g_data_ptr;      /* "data_ptr" */
 
 #define MAX_ARGS 24
@@ -48,17 +52,56 @@ static int as_ptr(PyObject *o, Held *h, void **out)
         *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(o);
         return PyErr_Occurred() ? -1 : 0;
     }
-    if (PyObject_CheckBuffer(o)) {
+    if (PyObject_TypeCheck(o, (PyTypeObject *)g_ndarray)) {
         Py_buffer *b = &h->buf[h->nbuf];
-        if (PyObject_GetBuffer(o, b, PyBUF_STRIDED_RO) != 0) return -1;
-        ++h->nbuf;
-        *out = b->buf;
-        return 0;
+        if (PyObject_GetBuffer(o, b, PyBUF_STRIDED_RO) == 0) {
+            ++h->nbuf;
+            *out = b->buf;
+            return 0;
+        }
+        PyErr_Clear(); /* a type without a buffer format */
+        PyObject *c = PyObject_GetAttrString(o, "ctypes");
+        PyObject *d = c ? PyObject_GetAttrString(c, "data") : NULL;
+        Py_XDECREF(c);
+        if (!d) return -1;
+        *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(d);
+        Py_DECREF(d);
+        return PyErr_Occurred() ? -1 : 0;
     }
     PyObject *r = PyObject_CallMethodNoArgs(o, g_data_ptr);
     if (!r) return -1;
     *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(r);
     Py_DECREF(r);
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+/* a handle, a stream or a whole number: an int, an object with __index__ (not for
+ * handles), or the ctypes object of its kind; longer ones are cut to 64 bits */
+static int as_bits(PyObject *o, char kind, uint64_t *out)
+{
+    PyObject *v;
+    if (kind == 'h' && o == Py_None) {
+        *out = 0;
+        return 0;
+    }
+    if (PyLong_Check(o)) v = Py_NewRef(o);
+    else if (kind != 'h' && PyIndex_Check(o)) v = PyNumber_Index(o);
+    else v = PyObject_CallFunction(g_ctypes_value, "OC", o, kind);
+    if (!v) return -1;
+    *out = (uint64_t)PyLong_AsUnsignedLongLongMask(v);
+    Py_DECREF(v);
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+static int as_double(PyObject *o, double *out)
+{
+    *out = PyFloat_AsDouble(o);
+    if (*out != -1.0 || !PyErr_Occurred()) return 0;
+    PyErr_Clear();
+    PyObject *v = PyObject_CallFunction(g_ctypes_value, "OC", o, 'f');
+    if (!v) return -1;
+    *out = PyFloat_AsDouble(v);
+    Py_DECREF(v);
     return PyErr_Occurred() ? -1 : 0;
 }
 
@@ -105,7 +148,6 @@ static int convert(const char *sig, PyObject *const *args, Py_ssize_t n, Held *h
         if (k >= n) break;
         PyObject *o = args[k];
         switch (sig[k]) {
-        case 'h':
         case 'p':
             if (as_ptr(o, h, &a[k].p) != 0) return -1;
             break;
@@ -115,17 +157,19 @@ static int convert(const char *sig, PyObject *const *args, Py_ssize_t n, Held *h
             a[k].p = (void *)q;
             break;
         }
+        case 'h':
         case 'i':
         case 'l': {
-            const long long v = PyLong_AsLongLong(o);
-            if (v == -1 && PyErr_Occurred()) return -1;
-            if (sig[k] == 'i') a[k].i = (int32_t)v;
-            else a[k].l = (int64_t)v;
+            uint64_t v;
+            if (as_bits(o, sig[k], &v) != 0) return -1;
+            if (sig[k] == 'i') a[k].i = (int32_t)(uint32_t)v;
+            else if (sig[k] == 'l') a[k].l = (int64_t)v;
+            else a[k].p = (void *)(uintptr_t)v;
             break;
         }
         default: {
-            const double v = PyFloat_AsDouble(o);
-            if (v == -1.0 && PyErr_Occurred()) return -1;
+            double v;
+            if (as_double(o, &v) != 0) return -1;
             a[k].f = (float)v;
         }
         }
@@ -223,16 +267,15 @@ static PyObject *f_compact(PyObject *self, PyObject *const *args, Py_ssize_t n)
     }
     Held h;
     h.nbuf = h.nobj = 0;
-    void *hd, *kept, *stream, *src[8], *dst[8];
+    void *kept, *src[8], *dst[8];
+    uint64_t hd, stream, total, rows, size;
     int64_t rb[8];
-    int bad = as_ptr(args[0], &h, &hd) || as_ptr(args[2], &h, &kept) || as_ptr(args[7], &h, &stream);
-    const long long total = bad ? 0 : PyLong_AsLongLong(args[1]);
-    const long long rows = bad ? 0 : PyLong_AsLongLong(args[3]);
-    bad = bad || PyErr_Occurred();
+    int bad = as_bits(args[0], 'h', &hd) || as_bits(args[1], 'l', &total) || as_ptr(args[2], &h, &kept) ||
+              as_bits(args[3], 'l', &rows) || as_bits(args[7], 'h', &stream);
     for (Py_ssize_t k = 0; k < t && !bad; ++k) {
-        bad = as_ptr(PyList_GET_ITEM(args[4], k), &h, &src[k]) || as_ptr(PyList_GET_ITEM(args[5], k), &h, &dst[k]);
-        if (!bad) rb[k] = (int64_t)PyLong_AsLongLong(PyList_GET_ITEM(args[6], k));
-        bad = bad || PyErr_Occurred();
+        bad = as_ptr(PyList_GET_ITEM(args[4], k), &h, &src[k]) || as_ptr(PyList_GET_ITEM(args[5], k), &h, &dst[k]) ||
+              as_bits(PyList_GET_ITEM(args[6], k), 'l', &size);
+        if (!bad) rb[k] = (int64_t)size;
     }
     if (bad) {
         release(&h);
@@ -240,8 +283,8 @@ static PyObject *f_compact(PyObject *self, PyObject *const *args, Py_ssize_t n)
     }
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = ((int (*)(P, int64_t, P, int64_t, I, P, P, P, P))g_fn[F_COMPACT])(hd, total, kept, rows, (I)t, src, dst, rb,
-                                                                         stream);
+    rc = ((int (*)(P, int64_t, P, int64_t, I, P, P, P, P))g_fn[F_COMPACT])(
+        (P)(uintptr_t)hd, (int64_t)total, kept, (int64_t)rows, (I)t, src, dst, rb, (P)(uintptr_t)stream);
     Py_END_ALLOW_THREADS
     release(&h);
     return PyLong_FromLong(rc);
@@ -259,8 +302,8 @@ static PyObject *f_keep_total(PyObject *self, PyObject *const *args, Py_ssize_t 
     h.nbuf = h.nobj = 0;
     const int32_t *so, *kk;
     Py_ssize_t len = 0;
-    const double ratio = PyFloat_AsDouble(args[2]);
-    if ((ratio == -1.0 && PyErr_Occurred()) || as_host_i32(args[0], &h, &so, &len) != 0 ||
+    double ratio;
+    if (as_double(args[2], &ratio) != 0 || as_host_i32(args[0], &h, &so, &len) != 0 ||
         as_host_i32(args[1], &h, &kk, NULL) != 0) {
         release(&h);
         return NULL;
@@ -279,12 +322,13 @@ static PyObject *f_keep_total(PyObject *self, PyObject *const *args, Py_ssize_t 
     return PyLong_FromLong(total);
 }
 
-/* bind({name: address}, host_i32) */
+/* bind({name: address}, host_i32, numpy.ndarray, ctypes_value) */
 static PyObject *f_bind(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
     (void)self;
-    if (n != 2 || !PyDict_Check(args[0]) || !PyCallable_Check(args[1])) {
-        PyErr_SetString(PyExc_TypeError, "bind takes a dict of addresses and a callable");
+    if (n != 4 || !PyDict_Check(args[0]) || !PyCallable_Check(args[1]) || !PyType_Check(args[2]) ||
+        !PyCallable_Check(args[3])) {
+        PyErr_SetString(PyExc_TypeError, "bind takes a dict of addresses, a callable, a type and a callable");
         return NULL;
     }
     for (int k = 0; k < F_COUNT; ++k) {
@@ -298,6 +342,10 @@ static PyObject *f_bind(PyObject *self, PyObject *const *args, Py_ssize_t n)
     }
     Py_INCREF(args[1]);
     Py_XSETREF(g_host_i32, args[1]);
+    Py_INCREF(args[2]);
+    Py_XSETREF(g_ndarray, args[2]);
+    Py_INCREF(args[3]);
+    Py_XSETREF(g_ctypes_value, args[3]);
     Py_RETURN_NONE;
 }
 

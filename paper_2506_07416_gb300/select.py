@@ -140,6 +140,17 @@ def _stream_ptr(stream) -> Optional[int]:
     return stream.cuda_stream
 
 
+_CTYPES = {"h": ctypes.c_void_p, "i": ctypes.c_int32, "l": ctypes.c_int64, "f": ctypes.c_float}
+
+
+def _ctypes_value(o, kind: str):
+    """What a ctypes object stands for, where an argument of the kind takes one."""
+    t = _CTYPES[kind]
+    if not isinstance(o, t):
+        raise TypeError(f"{type(o).__name__} is no argument of type {t.__name__}")
+    return 0 if o.value is None else o.value
+
+
 def _load_fastcall():
     try:
         from . import _fastcall
@@ -147,7 +158,7 @@ def _load_fastcall():
         raise ImportError(f"_fastcall.so is not built; run __graft_entry__.build() ({e})") from e
     _fastcall.bind({n: ctypes.cast(getattr(LIB, "litevlm_select_" + n), ctypes.c_void_p).value
                     for n in ("score", "score_full_keys", "score_topk", "topk", "compact", "splice", "project",
-                              "keep_offsets")}, _host_i32)
+                              "keep_offsets")}, _host_i32, np.ndarray, _ctypes_value)
     return _fastcall
 
 

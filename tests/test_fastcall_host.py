@@ -47,6 +47,72 @@ def test_keep_total_of_any_offsets(kind):
     assert select._keep_total(long, None, 0.5) == int(select.keep_offsets(long, None, 0.5)[-1])
 
 
+@pytest.fixture
+def topk_args():
+    """_FC.topk with a recorder in the place of the C function: the arguments it was called with."""
+    seen = []
+    proto = ctypes.CFUNCTYPE(ctypes.c_int, *select.LIB.litevlm_select_topk.argtypes)
+    rec = proto(lambda *a: seen.append(a) or 0)
+    names = ("score", "score_full_keys", "score_topk", "topk", "compact", "splice", "project", "keep_offsets")
+
+    def bind(**over):
+        addr = {n: ctypes.cast(getattr(select.LIB, "litevlm_select_" + n), ctypes.c_void_p).value for n in names}
+        select._FC.bind({**addr, **over}, select._host_i32, np.ndarray, select._ctypes_value)
+
+    bind(topk=ctypes.cast(rec, ctypes.c_void_p).value)
+    yield lambda **kw: _topk(seen, **kw)
+    bind()
+
+
+def _topk(seen, handle=16, batch=2, scores=32, ratio=0.25, stream=48):
+    seen.clear()
+    assert select._FC.topk(handle, batch, scores, None, [0, 1, 2], None, None, ratio, 64, 80, None, stream) == 0
+    a = seen[0]
+    return dict(handle=a[0], batch=a[1], scores=a[2], ratio=a[7], stream=a[11])
+
+
+def test_pointers_and_numbers(topk_args):
+    """Device pointers: None, ints, arrays, objects with data_ptr(); handles and numbers as ctypes takes them."""
+    torch = pytest.importorskip("torch")
+    a, t = np.arange(5, dtype=np.float32), torch.arange(5)
+    assert topk_args(scores=None)["scores"] is None
+    assert topk_args(scores=a)["scores"] == a.ctypes.data
+    assert topk_args(scores=a[1:])["scores"] == a.ctypes.data + 4
+    assert topk_args(scores=a.view("datetime64[s]" if a.itemsize == 8 else "V4"))["scores"] == a.ctypes.data
+    d = np.zeros(3, "datetime64[s]")  # a type without a buffer format
+    assert topk_args(scores=d)["scores"] == d.ctypes.data
+    assert topk_args(scores=t)["scores"] == t.data_ptr()
+    assert topk_args(handle=ctypes.c_void_p(1 << 40))["handle"] == 1 << 40
+    assert topk_args(handle=None, stream=ctypes.c_void_p(None)) == dict(topk_args(), handle=None, stream=None)
+    for three in (3, np.int64(3), np.int32(3), np.array(3), torch.tensor(3), ctypes.c_int32(3), (1 << 70) + 3):
+        assert topk_args(batch=three)["batch"] == 3
+    for half in (0.5, np.float32(0.5), np.float64(0.5), torch.tensor(0.5), ctypes.c_float(0.5)):
+        assert topk_args(ratio=half)["ratio"] == 0.5
+    assert topk_args(ratio=-1.0)["ratio"] == -1.0
+
+
+@pytest.mark.parametrize("o", [np.int64(16), np.uint64(16), np.float32(1), ctypes.c_void_p(16), ctypes.c_int64(16),
+                               (ctypes.c_char * 64)(), b"abc", bytearray(64), memoryview(bytearray(64)), "abc", 1.0,
+                               [16], object()], ids=lambda o: type(o).__name__)
+def test_no_address_of_an_object_is_taken_for_a_pointer(topk_args, o):
+    with pytest.raises(AttributeError):
+        topk_args(scores=o)
+    for n in range(3):  # kept_idx, a source, a destination of compact
+        a = [16, [16], [16]]
+        a[n] = o if n == 0 else [o]
+        with pytest.raises(AttributeError):
+            select.compact(None, 1, a[0], 1, a[1], a[2], [16], stream=0)
+    if not isinstance(o, ctypes.c_void_p):
+        with pytest.raises(TypeError):
+            topk_args(handle=o)
+
+
+@pytest.mark.parametrize("o", ["3", 1.5, None, ctypes.c_int64(3), ctypes.c_float(3)], ids=lambda o: type(o).__name__)
+def test_no_whole_number(topk_args, o):
+    with pytest.raises(TypeError):
+        topk_args(batch=o)
+
+
 def test_errors():
     with pytest.raises(select.LitevlmError) as e:
         select._keep_total(np.array([0, 5], np.int32), None, 1.5)
