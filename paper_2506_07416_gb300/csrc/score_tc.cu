@@ -42,14 +42,20 @@
 // adds them in a fixed order over all SMs (the last CTA of a request to finish
 // used to: 28 rows of 1280 tokens through one SM made a tail of 6 to 8 us).
 //
-// The reference of pass 1 is not the running maximum: any logit of the row
-// within 2^+-96 of the row's largest serves, since the sums are floating point
-// and the reference cancels in b. A thread takes the largest of the first 32
-// columns it sees, and moves it (to the larger maximum, rescaling its sum) only
-// when a sum passes 2^96, checked once per tile while the logits are still in
-// tensor memory. In units of log2 it is rounded to a whole number, so that sums
-// under two references are merged by a power of two, without error. The loop is then one fused multiply-add (packed in
-// pairs), one 2^x and one add (packed) per logit, in both passes.
+// The reference of pass 1 is not the running maximum: any logit near the row's
+// largest serves, since the sums are floating point and the reference cancels in b.
+// A thread takes the largest of the first 32 columns it sees, and moves it (to the
+// larger maximum, rescaling its sum) only when a tile adds more than 2^10 to the sum,
+// checked once per tile while the logits are still in tensor memory. So no exponent
+// that counts is above 10, where its rounding (2^-21) is that of b, and the sum's
+// logarithm stays as small as under the maximum. (A limit of 2^96, which only keeps
+// the sums finite, let errors of a row reach 3.8e-6; now 4.2e-7, and 5.4e-7 with the
+// running maximum. 2^12 left the e4m3 item above 2% less exact than the running
+// maximum, 2^10 makes it 2% more exact; 2^8 redoes tiles for 6% of its time, 2^10 for
+// 1%.) In units of log2 the reference is rounded to a whole number, so that sums
+// under two references are merged by a power of two, without error. The loop is then
+// one fused multiply-add (packed in pairs), one 2^x and one add (packed) per logit, in
+// both passes.
 //
 // Warp roles (352 threads): warp 0 = TMA producer, warps 1 and 2 = MMA issuers
 // (warp 1 also allocates TMEM), warps 3..10 = epilogue, two warpgroups (TMEM
@@ -87,7 +93,7 @@ template <int N>
 struct Blocks {
     static constexpr int value = N;
 };
-constexpr float kSumLimit = 7.9e28f;  // about 2^96: a pass-1 sum beyond moves its reference
+constexpr float kTileLimit = 1024.f;  // a tile that adds more to a pass-1 sum moves its reference
 
 // Shared-memory plan. The ring gets whatever is left of the 227 KB after the
 // Q double buffer and the bookkeeping; every variant needs more than half of
@@ -557,6 +563,7 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
                         nrc = ref == -INFINITY ? 0.f : -rintf(ref * cl);
                     }
                     const float2 o01 = s01, o23 = s23;
+                    const float before = (s01.x + s01.y) + (s23.x + s23.y);
                     if (full) {
 #pragma unroll
                         for (int k = 0; k < (kEpiWG == 4 ? 2 * NB : 0); ++k) {
@@ -579,7 +586,8 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
                     }
                     // a logit far above the reference (or not a number), or no reference
                     // yet: take the tile's maximum into the reference and redo the tile
-                    if (__any_sync(0xffffffffu, !((s01.x + s01.y) + (s23.x + s23.y) < kSumLimit) || ref == -INFINITY)) {
+                    const float added = (s01.x + s01.y) + (s23.x + s23.y) - before;
+                    if (__any_sync(0xffffffffu, !(added < kTileLimit) || ref == -INFINITY)) {
                         float m = ref;
 #pragma unroll 1
                         for (int c = 0; c < NB * 64; c += 32) {

@@ -1,8 +1,7 @@
 """The re-read score kernel where its rules change path: 64 / 65 text rows (pass 1
 with M = 64 or 128, mixed in one batch), partial and single tiles, one and several
-head groups, and logits that leave the reference of the first tile behind by more
-than the 2^96 its sums may grow (upwards, so that pass 1 redoes a tile, and
-downwards)."""
+head groups, and logits that leave the reference of the first tile far behind
+(upwards, so that pass 1 redoes a tile, and downwards)."""
 import numpy as np
 import pytest
 
@@ -124,7 +123,7 @@ def test_packed_heads_with_the_full_key_set(sel, t, query, kernel):
 def test_logits_far_from_the_first_tiles_reference(sel, t, later):
     # every query is one unit direction times 10; the keys of the first 128 tokens lie near 0 along it, those
     # of token 200 on at `later` +- 1: logits 10 * later / sqrt(128) = +-35 and, times 4 in token 333, +-141 nats
-    # (204 in log2), beyond the 96 that pass 1 lets its sums grow.
+    # (204 in log2), beyond the 10 that pass 1 lets a term exceed its reference by.
     # x = s * c - b is rounded at |x| <= 2 * 204: relative error of 2^x up to 408 * 2^-24 * ln 2 = 1.7e-5,
     # well inside the bf16 bound of 2e-3.
     w = _w("far", [700], [t], 4, 2)
@@ -141,6 +140,33 @@ def test_logits_far_from_the_first_tiles_reference(sel, t, later):
     s = sel.Selector(1, 700, t, w.hq, w.hkv, 128, "bf16", score_kernel="reread")
     o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, 128, "bf16")
     assert_scores_close(_scores(s, x, xd), o, "bf16")
+    s.close()
+
+
+@pytest.mark.parametrize("count", [1, 7, 60])
+def test_row_statistics_far_above_the_first_reference(sel, count):
+    """One text row and head whose largest logits, `count` of them around 0, lie 60 to 90 log2 units above those of
+    the first tiles. Each logit is one exact product, so a score's relative error is that of the row's statistic b and
+    of one 2^x, in units of log2: half a step of an exponent up to 16 in pass 1 and of b (2^-21 each), of an exponent
+    up to 8 in pass 2 (2^-22), one step of the logarithm of a sum below 2^20 (2^-19), and 2^-22 for either 2^x. Times
+    ln 2: 2.4e-6 in all."""
+    bound = (2 * 2.0 ** -21 + 2.0 ** -22 + 2.0 ** -19 + 2 * 2.0 ** -22) * np.log(2)
+    rng = np.random.Generator(np.random.PCG64(count))
+    n = 700
+    c = 1.4426950408889634 / np.sqrt(128)
+    q = np.zeros((1, 1, 128), np.float32)
+    q[..., 0] = 8.0
+    s = sel.Selector(1, n, 1, 1, 1, 128, "bf16", score_kernel="reread")
+    so, to = np.array([0, n], np.int32), np.array([0, 1], np.int32)
+    for gap in range(60, 92, 2):
+        k = np.zeros((n, 1, 128), np.float32)
+        k[:, 0, 0] = -gap / (8.0 * c) + 0.3 * rng.standard_normal(n)
+        k[300:300 + count, 0, 0] = 0.3 * rng.standard_normal(count)
+        x = {"q": inputs.f32_to_bf16_bits(q), "k": inputs.f32_to_bf16_bits(k), "seq_offsets": so, "text_offsets": to}
+        o = oracle.score(x["q"], x["k"], so, to, 1, 1, 128, "bf16")
+        g = _scores(s, x, to_device(x, None))
+        top = slice(300, 300 + count)
+        assert np.abs(g[top] / o[top] - 1).max() < bound, gap
     s.close()
 
 
