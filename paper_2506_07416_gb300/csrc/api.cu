@@ -48,6 +48,7 @@ struct litevlm_select {
     long long wait_budget = lvs::kWaitBudgetCycles;  // clock cycles each device-side wait may take
     int32_t debug_flags = 0;                         // LITEVLM_DEBUG_* (tests of the failure path)
     bool allow_flat = true;  // the resident kernel's flattened schedule may be chosen (not in the no-alloc path)
+    bool share_items = true; // the re-read kernel's CTAs may claim items from each other (not in the no-alloc path)
 };
 
 namespace {
@@ -625,7 +626,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     p.out = scores;
     p.partials = h->partials;
     p.counters = h->counters;
-    p.claims = h->counters + (h->n_counters - 2);
+    p.claims = h->share_items ? h->counters + (h->n_counters - 2) : nullptr;
     p.err = h->err_d;
     p.total_vis = tot_n;
     p.hq = c.num_q_heads;
@@ -695,9 +696,6 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     if (clear_tickets > 0 && choice.resident && plan.groups > 1) {
         const cudaError_t ce = cudaMemsetAsync(h->counters, 0, sizeof(int32_t) * clear_tickets, (cudaStream_t)stream);
         if (ce != cudaSuccess) return cuda_fail(h, ce, "clearing the fold tickets");
-    } else if (clear_tickets > 0 && !choice.resident && plan.cluster == 1 && plan.ctas < plan.groups * batch) {
-        const cudaError_t ce = cudaMemsetAsync(p.claims, 0, 2 * sizeof(int32_t), (cudaStream_t)stream);
-        if (ce != cudaSuccess) return cuda_fail(h, ce, "clearing the claims");
     }
     const cudaError_t e =
         choice.resident
@@ -1257,7 +1255,7 @@ constexpr int64_t kNoAllocTickets = int64_t(1) << 14;        // 64 KiB of fold t
 constexpr int kNoAllocMaxDevices = 64;
 
 static __device__ __align__(256) float g_noalloc_partials[kNoAllocPartialFloats];
-static __device__ __align__(256) int32_t g_noalloc_tickets[kNoAllocTickets + 2];  // and the claims
+static __device__ __align__(256) int32_t g_noalloc_tickets[kNoAllocTickets];
 
 struct NoAllocDevice {
     bool ready = false;
@@ -1366,7 +1364,7 @@ extern "C" litevlm_status_t litevlm_select_score_noalloc(int32_t num_q_heads, in
         h.num_sms = d.num_sms;
         h.partials = d.partials;
         h.counters = d.tickets;
-        h.n_counters = (size_t)kNoAllocTickets + 2;
+        h.n_counters = (size_t)kNoAllocTickets;
         h.encode = d.encode;
         for (int r = 0; r < 2; ++r)
             for (int c = 0; c < 17; ++c) {
@@ -1378,6 +1376,8 @@ extern "C" litevlm_status_t litevlm_select_score_noalloc(int32_t num_q_heads, in
     }
     h.err_d = err_d;
     h.allow_flat = false;  // its partial rows could exceed the static scratch
+    // no state that calls would share unless they split their heads: a CTA per item
+    h.share_items = false;
     h.cfg.max_batch = batch;
     h.cfg.max_total_visual = tot_n;
     h.cfg.max_total_text = text_offsets_h[batch] > 0 ? text_offsets_h[batch] : 0;

@@ -34,7 +34,7 @@ struct ScoreLaunch {
     int32_t hqe;  // resident kernel: heads of a request as scheduled (pseudo-heads, head blocks)
     // re-read kernel without clusters: its CTAs share `items` (request, head
     // group) items; claims[0] counts those taken beyond a CTA's first, claims[1]
-    // the CTAs that are done (zero between launches, workspace)
+    // the CTAs that are done (zero between launches, workspace). Null: a CTA per item.
     int32_t items;
     int32_t* claims;
     int32_t ctas_per_request; // cluster size * groups

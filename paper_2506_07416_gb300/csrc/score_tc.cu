@@ -843,8 +843,9 @@ cudaError_t launch_variant(const CUtensorMap& tm_q, const CUtensorMap& tm_k, con
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     // clusters: one per item; without, as many CTAs as run at once, which share the items
+    // (or one per item, where the call has no claims)
     const int items = plan.groups * batch;
-    const int ctas = plan.cluster > 1 ? plan.cluster * items : items < plan.ctas ? items : plan.ctas;
+    const int ctas = plan.cluster > 1 || !p.claims || items < plan.ctas ? plan.cluster * items : plan.ctas;
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(kThreadsOf<kEpiWG>, 1, 1);
     cfg.dynamicSmemBytes = smem;

@@ -97,6 +97,35 @@ def test_noalloc_matches_the_oracle(sel):
 
 
 @pytest.mark.gpu
+def test_calls_that_split_no_heads_share_nothing(sel):
+    """A batch with more (request, head group) items than CTAs run at once, whose heads are not split, on two streams
+    at the same time: such calls touch no scratch, as they need none for partial rows."""
+    if not torch.cuda.is_available():
+        pytest.fail("the GPU tests need a CUDA device")
+    n = [130, 700, 1, 257, 900, 64] * 60
+    w = _case("items", 1, 1, 128, "bf16", n, [1 + i % 128 for i in range(len(n))])
+    xd = inputs.make_torch(w, "cuda")
+    so, to = w.seq_offsets(), w.text_offsets()
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, 1, 1, 128, "bf16")
+    plan = s.score_plan(to, so)
+    assert plan[0] == 1 and plan[3] == 1 and w.batch > torch.cuda.get_device_properties(0).multi_processor_count
+    ref = s.score(xd["q"], xd["text_offsets"], xd["k"], xd["seq_offsets"], seq_offsets_h=so, text_offsets_h=to)
+    s.check_device()
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    outs = [torch.full((w.total_vis,), float("nan"), device="cuda") for _ in range(40)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        sel.score_noalloc(1, 1, 128, "bf16", w.batch, xd["q"], xd["text_offsets"], to, xd["k"], xd["seq_offsets"], so,
+                          1.0, 1.0, out, err, stream=streams[i % 2])
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    for out in outs:
+        assert torch.equal(out, ref)
+    s.close()
+
+
+@pytest.mark.gpu
 def test_noalloc_rejects_head_groups_beyond_the_partial_scratch(sel):
     """Limit 2: a launch that splits the query heads over G > 1 groups needs G x
     total_visual partial scores; beyond the static 1048576 floats the call
