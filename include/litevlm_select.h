@@ -497,9 +497,10 @@ litevlm_status_t litevlm_select_set_debug_flags(litevlm_select_t handle, int32_t
  *     fixed shape is launched.
  *   - A call beyond either limit returns LITEVLM_ERR_WORKSPACE and enqueues
  *     nothing. Limit 1 is checked before any CUDA call.
- *   - A call that splits the heads clears the tickets it uses with
- *     cudaMemsetAsync on `stream`, after every host-side check (a rejected
- *     call enqueues nothing).
+ *   - A call that splits the heads on the resident kernel clears the tickets it
+ *     uses with cudaMemsetAsync on `stream`, after every host-side check (a
+ *     rejected call enqueues nothing). The re-read kernel uses no tickets: its
+ *     partial rows are added by a kernel launched behind it.
  * Calls that overlap on one device (other streams, other host threads) share
  * this scratch and race. Serialise them.
  *

@@ -232,12 +232,14 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
     for (int cl = 1; cl <= lvs::kMaxCluster; ++cl)
         if (tcap[cl] < 0) tcap[cl] = lvs::tc_cluster_capacity(row_bytes, fp8, hp * max_t <= 64 ? 64 : 128, cl);
     const double u = 1.17;
-    const lvs::KernelCosts res_costs = limit_rule ? lvs::KernelCosts{6.0 * u, 6.0 * u, u, u, 0.25 * u, 2.0 * u, false}
-                                                  : lvs::KernelCosts{7.5, 7.5, 0.75, 0.75, 0.25, 2.0, false};
+    const lvs::KernelCosts res_costs = limit_rule
+                                           ? lvs::KernelCosts{6.0 * u, 6.0 * u, u, u, 0.25 * u, 2.0 * u, u, false}
+                                           : lvs::KernelCosts{7.5, 7.5, 0.75, 0.75, 0.25, 2.0, 1.0, false};
     const double two_tile = limit_rule ? 0.6 * u : 0.56, two_head = limit_rule ? 2.1 * u : 2.0;
     const lvs::KernelCosts tc_costs =
-        limit_rule ? lvs::KernelCosts{9.6 * u, 9.6 * u, 1.6 * u, 1.6 * u, 0.4 * u, 3.2 * u, false}
-                   : lvs::KernelCosts{6.0, 1.0, row_bytes == 256 ? (hp * max_t > 64 ? 1.12 : 0.86) : 0.65, 1.5, 0.5, 2.0, true};
+        limit_rule ? lvs::KernelCosts{9.6 * u, 9.6 * u, 1.6 * u, 1.6 * u, 0.4 * u, 3.2 * u, 1.6 * u, false}
+                   : lvs::KernelCosts{6.0, 1.0, row_bytes == 256 ? (hp * max_t > 64 ? 1.12 : 0.86) : 0.65, 1.5, 0.5,
+                                      2.0, 0.1, true};
     ScoreChoice best{false, lvs::plan_score(bt, hq / hp, c.num_kv_heads, row_bytes, tcap, tc_costs,
                                             limit_rule ? 2.0 : 1.0, &tc_cost)};
     best.plan.hp = hp;
@@ -296,7 +298,7 @@ ScoreChoice choose_score_kernel(litevlm_select_t h, int batch, const int32_t* se
                     const long long ctas = (long long)batch * cl * g;
                     const double active = (double)(ctas < cap ? ctas : cap);
                     auto item_cost = [&](int tiles) {
-                        if (tiles <= 0) return 1.0;
+                        if (tiles <= 0) return res_costs.empty;
                         const int t = (tiles + cl - 1) / cl;
                         double per_head;
                         if (nb == 1) {
@@ -639,7 +641,7 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     p.query_last = (c.flags & LITEVLM_FLAG_QUERY_LAST_TOKEN) != 0;
     p.extra = nullptr;
     // the top-k CTA of a request reads groups x N_b partial values: worth it
-    // for small requests (it saves the score kernel's ticketed fold), not for
+    // for small requests (it saves the score call's fold), not for
     // long ones with many groups
     p.defer_fold = allow_defer && plan.groups > 1 && (int64_t)plan.groups * sh.max_n <= 32768;
     if (p.defer_fold && deferred_groups) *deferred_groups = plan.groups;

@@ -150,10 +150,10 @@ double makespan(const BatchTiles& bt, int g, int slots, const Cost& cost)
 
 // Modelled times of the planners, in microseconds: a CTA's start and end, the step
 // from one item to the next in a CTA that works through several, a tile of a head,
-// a head's statistics exchange over a cluster / within one CTA, and a fold of
-// several head groups (per CTA, or once when it is a launch of its own).
+// a head's statistics exchange over a cluster / within one CTA, a fold of several
+// head groups (per CTA, or once when it is a launch of its own), and an empty request.
 struct KernelCosts {
-    double start, next, tile, exchange, exchange_one, fold;
+    double start, next, tile, exchange, exchange_one, fold, empty;
     bool fold_once;
 };
 // cap_by_cluster[c]: CTAs of the re-read kernel resident at once with clusters of c (<= 0: unusable)

@@ -919,7 +919,7 @@ ScorePlan plan_score(const BatchTiles& bt, int hq, int hkv, int row_bytes, const
                 const double miss = costs.fold_once && window > 110e6 ? 1.0 + (window - 110e6) / 110e6 : 1.0;
                 auto item_cost = [&](int tiles) {
                     const int t = (tiles + c - 1) / c;
-                    return tiles <= 0 ? 0.1
+                    return tiles <= 0 ? costs.empty
                                       : (c > 1 ? costs.start : costs.next) + (g > 1 && !costs.fold_once ? costs.fold : 0.0) +
                                             hpg * (t * costs.tile * miss + (c > 1 ? costs.exchange : costs.exchange_one));
                 };

@@ -42,6 +42,13 @@ CASES = [
 ]
 
 
+# visual tokens, text tokens of each request, heads, and whether the call is within the limit
+LIMITS = [
+    ([4094] * 16 + [0] * 124, 128, 28, 4, "INVALID_ARG"),
+    ([6592, 0, 6592, 6592, 0, 6592, 6592, 0, 6592, 6592], 97, 32, 8, "WORKSPACE"),
+]
+
+
 def test_noalloc_rejects_batches_beyond_the_static_scratch(sel):
     """Host-side check, before any CUDA call: total_visual / 128 + 2 * batch + 2 > 16384."""
     so = np.array([0, 3_000_000], np.int32)
@@ -94,6 +101,22 @@ def test_noalloc_matches_the_oracle(sel):
     assert int(err.item()) == 0
     o = oracle.score(x["q"], x["k"], x["seq_offsets"], x["text_offsets"], w.hq, w.hkv, w.head_dim, w.dtype)
     assert_scores_close(out.cpu().numpy(), o, w.dtype)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,t,hq,hkv,status", LIMITS, ids=["taken", "refused"])
+def test_limit_of_batches_with_empty_requests(sel, n, t, hq, hkv, status):
+    """The limit on head groups x total_visual is that of a launch shape fixed by the batch's sizes, which an empty
+    request's cost in the fixed rule takes part in. No pointers are given: a batch within the limit is refused for
+    them, before anything is enqueued."""
+    if not torch.cuda.is_available():
+        pytest.fail("the GPU tests need a CUDA device")
+    torch.zeros(1, device="cuda")
+    so = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+    to = (np.arange(len(n) + 1) * t).astype(np.int32)
+    with pytest.raises(sel.LitevlmError) as ei:
+        sel.score_noalloc(hq, hkv, 128, "bf16", len(n), 0, 0, to, 0, 0, so, 1.0, 1.0, 0, 64, stream=0)
+    assert ei.value.name == status
 
 
 @pytest.mark.gpu
