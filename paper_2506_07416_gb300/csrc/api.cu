@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <mutex>
 #include <new>
 #include <string>
@@ -633,7 +634,10 @@ litevlm_status_t score_impl(litevlm_select_t h, int32_t batch, const void* q_tex
     p.total_vis = tot_n;
     p.hq = c.num_q_heads;
     p.hkv = c.num_kv_heads;
-    p.c_log2 = (float)((double)q_scale * (double)k_scale / sqrt((double)c.head_dim) * 1.4426950408889634);
+    // (not 0, where the scales' product is below 32 bits: the kernels weigh columns past a
+    // request's end 2^(-inf * c), and at the smallest normal value every 2^(s * c) is 1 too)
+    p.c_log2 = std::max((float)((double)q_scale * (double)k_scale / sqrt((double)c.head_dim) * 1.4426950408889634),
+                        std::numeric_limits<float>::min());
     p.wait_budget = h->wait_budget;
     p.stall = (h->debug_flags & LITEVLM_DEBUG_STALL_SCORE) != 0;
     p.slot_cols = ((qsplit ? (max_t + 1) / 2 : max_t * plan.hp) + 15) & ~15;

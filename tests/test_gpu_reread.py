@@ -143,6 +143,21 @@ def test_logits_far_from_the_first_tiles_reference(sel, t, later):
     s.close()
 
 
+@pytest.mark.parametrize("kernel", ["reread", "resident"])
+def test_scales_whose_product_vanishes(sel, kernel):
+    """Two e4m3 scales of 1e-25: every logit is 0 in 32 bits, so a request's tokens share its score, also where its
+    last tile is partly empty."""
+    w = _w("tiny_scales", [300, 128, 1], [20, 65, 3], 4, 2, dtype="e4m3")
+    x = inputs.make_numpy(w)
+    x["q_scale"] = x["k_scale"] = 1e-25
+    s = sel.Selector(w.batch, w.total_vis, w.total_txt, w.hq, w.hkv, w.head_dim, w.dtype, score_kernel=kernel)
+    g = _scores(s, x, to_device(x, w))
+    for b in range(3):
+        n0, n1 = x["seq_offsets"][b:b + 2]
+        np.testing.assert_allclose(g[n0:n1], 1.0 / (n1 - n0), rtol=2e-6)  # fp32 sums of up to 300 ones and 260 rows
+    s.close()
+
+
 @pytest.mark.parametrize("count", [1, 7, 60])
 def test_row_statistics_far_above_the_first_reference(sel, count):
     """One text row and head whose largest logits, `count` of them around 0, lie 60 to 90 log2 units above those of
