@@ -53,10 +53,10 @@ __device__ __forceinline__ bool wait_phase_cluster(uint32_t bar, uint32_t parity
 
 // The same waits for the re-read score kernel, whose warps wait often and for a
 // short time: kPolls polls of a few instructions between two looks at the abort
-// flag and the clock. The suspend-time hint above compiles to a loop around
-// NANOSLEEP, and a look at flag and clock on every poll to a dozen instructions;
-// both took issue slots from the warps of the SM sub-partition that had work
-// (fp8_ragged 151 -> 141 us). The resident kernel's long waits are better asleep
+// flag and the clock. Waits with the suspend-time hint above, which looked at flag
+// and clock after every test, made up a third of the kernel's executed instructions,
+// NANOSLEEP among them (counted by opcode), and took issue slots from the warps of
+// the SM sub-partition that had work (fp8_ragged 151 -> 141 us). The resident kernel's long waits are better asleep
 // (sweep 734 us, 739 with polls).
 constexpr uint32_t kPolls = 64;
 

@@ -28,11 +28,14 @@
 // the tile's stages with the contraction: 27648 x 4096 -> 4096 755 -> 617 us, 6157
 // x 3584 -> 512 (e4m3) 34.3 -> 26.6 us, 1536 x 2048 -> 2048 25.5 -> 19.4 us (48 tiles
 // on 76 pairs: 10 us of it are launch, set-up and the one epilogue); with the
-// contractions issued from uniform registers (elect_one) 588, 24.9 and 18.5 us. A
+// contractions issued from uniform registers (elect_one) 588, 24.9 and 18.5 us, and
+// with stages held until their sums have their values and the closing exchange about
+// waits that gave up 603, 25.5 and 18.8. A
 // kernel of its own for the row scales, overlapping the first tiles, was slower on
 // all of them (623, 29 and 21 us against 617, 26.6 and 19.4): its loads compete with
 // the copies.
-// Every wait is bounded.
+// Every wait is bounded. When one gives up the pair brings its copies level and waits
+// for the barriers of all that it started before it leaves.
 
 #include <math.h>
 
@@ -46,7 +49,7 @@ namespace lvs {
 
 namespace {
 
-constexpr int kProjThreads = 320;  // producer, MMA issuer, two epilogue warpgroups
+constexpr int kProjThreads = 320;  // producer, MMA issuer, epilogue warpgroup, summing warpgroup
 constexpr int kProjK = 64;         // hidden values per stage (128 bytes of bf16)
 constexpr int kProjRows = 128;     // rows of a tile per CTA
 

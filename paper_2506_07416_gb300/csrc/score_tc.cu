@@ -25,9 +25,11 @@
 // other in 128 rows (hp * T <= 128) form a head block, row i * hp + h of its Q
 // tile being text row i of head h. "Head" below means such a block: it streams
 // the key head's tiles once instead of hp times (last-token queries of 64
-// requests, 32 / 8 heads: 314 -> 106 us).
+// requests, 32 / 8 heads: 282 -> 106 us; choose_score_kernel now gives that call to
+// the resident kernel, 80).
 // A CTA without a cluster works through several (request, head group) items,
-// claimed largest first: its set-up and teardown (5 us) are paid once, and the
+// claimed largest first (in the no-alloc call, which shares nothing, there is a CTA
+// per item): its set-up and teardown (5 us) are paid once, and the
 // groups can be finer. Scores of 12 requests of 322 to 2491 tokens, 32 / 8 heads: 45
 // -> 38 us; 16 requests of 636 to 2586, 16 heads: 36.5 -> 33.9; 32 requests of 629 to
 // 3404 in e4m3, 32 heads: 109 -> 106.

@@ -61,14 +61,14 @@ def _run(sel, rows, hidden, out_f, head_dim, bias, eps=1e-6, base=1e6, max_pos=4
     (129, 136, 384, 0, False),       # no rotation, 128-column tiles
     (200, 3584, 512, 128, True),     # 4 KV heads x 128 from hidden 3584
     (1, 512, 256, 128, False),       # one row
-    (4900, 128, 4096, 128, True),    # enough tiles for the 256-row variant, ragged last tile
+    (4900, 128, 4096, 128, True),    # several tiles a pair of CTAs, ragged last row tile
 ])
 def test_project_matches_oracle(sel, rows, hidden, out_f, head_dim, bias):
     _run(sel, rows, hidden, out_f, head_dim, bias)
 
 
 @pytest.mark.parametrize("rows,hidden,out_f,head_dim,bias", [
-    (127, 64, 128, 128, False),      # one 128-column tile: one warpgroup takes the whole head; the pair's second half empty
+    (127, 64, 128, 128, False),      # one 128-column tile, one head: two warpgroups; the pair's second half empty
     (129, 8, 256, 64, True),         # the smallest hidden; one row in the pair's second half
     (256, 72, 640, 0, True),         # 128-column tiles, a stage that is almost all padding
     (257, 1000, 512, 128, False),    # a second row tile with one row

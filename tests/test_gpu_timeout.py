@@ -81,8 +81,8 @@ def test_wait_timeout_is_reported_and_the_handle_recovers(sel):
 def test_wait_timeout_in_the_reread_kernel(sel):
     """The same failure path in the kernel that streams K twice per head: its
     producer stalls the same way, the launch gives up within the budget, and the
-    handle is exact again afterwards (the heads are split over CTA groups, so
-    the fold tickets are in use here too)."""
+    handle is exact again afterwards (the heads are split over CTA groups, whose
+    partial rows the launch behind the kernel adds up)."""
     w = inputs.workload("single")
     x = inputs.make_numpy(w)
     xd = to_device(x, w)

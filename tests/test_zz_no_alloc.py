@@ -4,8 +4,8 @@ library's static device arrays, no handle and no allocation.
 The GPU test compares two consecutive calls with the handle-based
 litevlm_select_score on the same inputs. Both take the same launch plan and
 the kernels reduce in a fixed order, so the scores must be bit-identical; the
-second call runs on scratch the first one has used (each call clears the fold
-tickets it needs before its launch). One case is also compared directly with
+second call runs on scratch the first one has used (a call that folds by
+tickets clears those it needs before its launch). One case is also compared directly with
 the oracle at the bf16 tolerance. Named to be collected after the other test
 files, so it also runs after them in one process (and the library's static
 scratch has already been used)."""
