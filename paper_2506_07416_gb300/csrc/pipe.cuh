@@ -205,9 +205,9 @@ __device__ __forceinline__ float log2_add(float x, float y)
 }
 
 // Merges the (reference, sum) partials of one row from every CTA of the cluster in
-// rank order and returns b = M + log2(L). All remote loads are issued
-// before any is used, so their latencies overlap.
-__device__ __forceinline__ float merge_cluster_row(uint32_t my_addr, uint32_t csize)
+// rank order and returns M and L. All remote loads are issued before any is used, so
+// their latencies overlap.
+__device__ __forceinline__ float2 merge_cluster_row(uint32_t my_addr, uint32_t csize)
 {
     float2 st[kMaxCluster];
 #pragma unroll
@@ -221,7 +221,7 @@ __device__ __forceinline__ float merge_cluster_row(uint32_t my_addr, uint32_t cs
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r)
         if (r < (int)csize && st[r].y > 0.f) L += st[r].y * ex2(st[r].x - M);
-    return M + __log2f(L);
+    return make_float2(M, L);
 }
 
 // Ticket slot of tile t of the request starting at row n0 (request b): unique

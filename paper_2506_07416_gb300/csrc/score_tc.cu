@@ -670,13 +670,15 @@ __global__ void __launch_bounds__(kThreadsOf<kEpiWG>, 1)
                     // (a CTA that is its own cluster reads its own rows, ordered by the named barrier above)
                     if (csize > 1) poll_phase<true>(BAR(STATS + slot), (uint32_t)(hs / kStatSlots) & 1u, ctl);
                     if (wt < R) {
-                        float bm;
-                        if (csize > 1) {
-                            bm = merge_cluster_row(base + L::OFF_STATS + (uint32_t)(slot * kMaxText + wt) * 8u, csize);
-                        } else {
-                            const float2 st = stats_s[slot * kMaxText + wt];
-                            bm = st.x + __log2f(st.y);
-                        }
+                        const uint32_t row = (uint32_t)(slot * kMaxText + wt);
+                        const float2 st = csize > 1 ? merge_cluster_row(base + L::OFF_STATS + row * 8u, csize) : stats_s[row];
+                        // For e4m3 the logarithm's error is a good part of a score's: mean
+                        // relative error over 8 draws of 13 requests of up to 3248 tokens
+                        // 1.34e-7 with __log2f and 1.19e-7 with log2f (0.97e-7 in the resident
+                        // kernel that had this call), of 32 of up to 3456 1.04e-7 and 0.81e-7,
+                        // at the same time. For bf16 and with other keys' terms it offsets
+                        // another one (12 requests, 32 / 8 heads: 1.5e-7, 2.3e-7 with log2f).
+                        float bm = st.x + (FP8 && !p.extra ? log2f(st.y) : __log2f(st.y));
                         if (p.extra) {
                             griddep_wait();
                             bm = log2_add(bm, p.extra[(int64_t)(t0 + wt / hp) * p.hq + (hg * hpg + hs) * hp + wt % hp]);
