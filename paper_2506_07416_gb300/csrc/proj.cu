@@ -30,7 +30,7 @@
 // on 76 pairs: 10 us of it are launch, set-up and the one epilogue); with the
 // contractions issued from uniform registers (elect_one) 588, 24.9 and 18.5 us, and
 // with stages held until their sums have their values and the closing exchange about
-// waits that gave up 603, 25.5 and 18.8. A
+// waits that gave up 603, 25.2 and 18.8. A
 // kernel of its own for the row scales, overlapping the first tiles, was slower on
 // all of them (623, 29 and 21 us against 617, 26.6 and 19.4): its loads compete with
 // the copies.

@@ -1,5 +1,5 @@
-"""The device-side failure path of the score kernels, made to run on purpose
-without faulting, trapping or hanging the GPU.
+"""The device-side failure path of the score kernels and of the projection, made
+to run on purpose without faulting, trapping or hanging the GPU.
 
 Every wait of the kernels (mbarrier phases, cluster arrivals) is bounded by the
 handle's wait budget. With LITEVLM_DEBUG_STALL_SCORE the TMA producer of either
