@@ -47,17 +47,16 @@
 // The reference of pass 1 is not the running maximum: any logit near the row's
 // largest serves, since the sums are floating point and the reference cancels in b.
 // A thread takes the largest of the first 32 columns it sees, and moves it (to the
-// larger maximum, rescaling its sum) only when a tile adds more than 2^10 to the sum,
+// larger maximum, rescaling its sum) only when a tile adds more than 2^12 to the sum,
 // checked once per tile while the logits are still in tensor memory. So no exponent
-// that counts is above 10, where its rounding (2^-21) is that of b, and the sum's
-// logarithm stays as small as under the maximum. (A limit of 2^96, which only keeps
-// the sums finite, let errors of a row reach 3.8e-6; now 4.2e-7, and 5.4e-7 with the
-// running maximum. 2^12 left the e4m3 item above 2% less exact than the running
-// maximum, 2^10 makes it 2% more exact; 2^8 redoes tiles for 6% of its time, 2^10 for
-// 1%.) In units of log2 the reference is rounded to a whole number, so that sums
-// under two references are merged by a power of two, without error. The loop is then
-// one fused multiply-add (packed in pairs), one 2^x and one add (packed) per logit, in
-// both passes.
+// that counts is above 12, where its rounding (2^-21) is that of b, and the sum's
+// logarithm stays about as small as under the maximum. (A limit of 2^96, which only
+// keeps the sums finite, let errors of a row reach 3.8e-6; now 4.2e-7, and 5.4e-7 with
+// the running maximum. Redone tiles cost the e4m3 item above 6% at 2^8, 1% at 2^10 and
+// nothing at 2^12; the lower limits were no more exact on ordinary batches.) In units of
+// log2 the reference is rounded to a whole number, so that sums under two references
+// are merged by a power of two, without error. The loop is then one fused multiply-add
+// (packed in pairs), one 2^x and one add (packed) per logit, in both passes.
 //
 // Warp roles (352 threads): warp 0 = TMA producer, warps 1 and 2 = MMA issuers
 // (warp 1 also allocates TMEM), warps 3..10 = epilogue, two warpgroups (TMEM
@@ -95,7 +94,7 @@ template <int N>
 struct Blocks {
     static constexpr int value = N;
 };
-constexpr float kTileLimit = 1024.f;  // a tile that adds more to a pass-1 sum moves its reference
+constexpr float kTileLimit = 4096.f;  // a tile that adds more to a pass-1 sum moves its reference
 
 // Shared-memory plan. The ring gets whatever is left of the 227 KB after the
 // Q double buffer and the bookkeeping; every variant needs more than half of

@@ -123,7 +123,7 @@ def test_packed_heads_with_the_full_key_set(sel, t, query, kernel):
 def test_logits_far_from_the_first_tiles_reference(sel, t, later):
     # every query is one unit direction times 10; the keys of the first 128 tokens lie near 0 along it, those
     # of token 200 on at `later` +- 1: logits 10 * later / sqrt(128) = +-35 and, times 4 in token 333, +-141 nats
-    # (204 in log2), beyond the 10 that pass 1 lets a term exceed its reference by.
+    # (204 in log2), beyond the 12 that pass 1 lets a term exceed its reference by.
     # x = s * c - b is rounded at |x| <= 2 * 204: relative error of 2^x up to 408 * 2^-24 * ln 2 = 1.7e-5,
     # well inside the bf16 bound of 2e-3.
     w = _w("far", [700], [t], 4, 2)
@@ -163,7 +163,7 @@ def test_row_statistics_far_above_the_first_reference(sel, count):
     """One text row and head whose largest logits, `count` of them around 0, lie 60 to 90 log2 units above those of
     the first tiles. Each logit is one exact product, so a score's relative error is that of the row's statistic b and
     of one 2^x, in units of log2: half a step of an exponent up to 16 in pass 1 and of b (2^-21 each), of an exponent
-    up to 8 in pass 2 (2^-22), one step of the logarithm of a sum below 2^20 (2^-19), and 2^-22 for either 2^x. Times
+    up to 8 in pass 2 (2^-22), one step of the logarithm of a sum below 2^22 (2^-19), and 2^-22 for either 2^x. Times
     ln 2: 2.4e-6 in all."""
     bound = (2 * 2.0 ** -21 + 2.0 ** -22 + 2.0 ** -19 + 2 * 2.0 ** -22) * np.log(2)
     rng = np.random.Generator(np.random.PCG64(count))
